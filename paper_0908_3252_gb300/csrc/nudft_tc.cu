@@ -1011,26 +1011,38 @@ k_tc_pair_gemm(const int64_t* __restrict__ ka, const int64_t* __restrict__ kb, c
 }
 
 // out[i][c] = scale * 2^e * (sum of the partials of the tile holding output
-// (i, c) in owner order); 2^e undoes the weight scaling.  A block sums a
-// patch of 32 rows x 32 columns of a partial tile (column q < 128: j = 128
-// tcol + q at c+(j); q >= 128: j = 128 tcol + q - 128 at c-(j)).  The owners
-// (CTAs, or CTA pairs when `pairs`) holding units of tile t are c_lo..c_hi (of
-// P), the last owners whose ranges start at or before the tile's first and
-// last unit; owner c keeps its partial of tile t in slot c + t, or, for a
-// pair, CTA h its 128 rows' partial in slot 2 (c + t) + h.  Each thread reads four
-// columns of one row as a vector, the patch turns in shared memory, and
-// writes run along the rows of out (the mirrored half in descending columns).
-// c-(0) = c+(0) for integer offsets and is written once.
-__global__ void __launch_bounds__(256) k_reduce_pair(const float* __restrict__ part, int64_t U, int64_t K, int64_t P,
-                                                     bool pairs, PairGeom pg, int tilesC, float scale,
-                                                     const unsigned* __restrict__ amax2, float2* __restrict__ out)
+// (i, c)); 2^e undoes the weight scaling.  A block sums a patch of 32 rows x
+// 4 TY columns of a partial tile (column q < 128: j = 128 tcol + q at c+(j);
+// q >= 128: j = 128 tcol + q - 128 at c-(j)).  The owners (CTAs, or CTA pairs
+// when `pairs`) holding units of tile t are c_lo..c_hi (of P), the last owners
+// whose ranges start at or before the tile's first and last unit; owner c
+// keeps its partial of tile t in slot c + t, or, for a pair, CTA h its 128
+// rows' partial in slot 2 (c + t) + h.  Each thread reads four columns of one
+// row as a vector; the S slices of a block take S contiguous ranges of the
+// owners, whose sums slice 0 adds in order (a fixed order, whatever the
+// scheduling); the patch turns in shared memory and writes run along the rows
+// of out (the mirrored half in descending columns).  c-(0) = c+(0) for integer
+// offsets and is written once.
+//
+// Bound by the latency of the partials' loads: a small image has one tile and
+// 76 partials of it, which one slice reads four at a time, one after the
+// other, on 64 SMs (48 us at N = 250, L = 31665 for 40 MB of L2-resident
+// partials).  launch_reduce picks the shape.
+template <int TY, int S>
+__global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* __restrict__ part, int64_t U, int64_t K,
+                                                             int64_t P, bool pairs, PairGeom pg, int tilesC,
+                                                             float scale, const unsigned* __restrict__ amax2,
+                                                             float2* __restrict__ out)
 {
-    __shared__ float2 patch[32][33];
+    constexpr int W = 4 * TY;  // columns of the patch
+    __shared__ float2 patch[W][33];
+    __shared__ float4 sums[S > 1 ? 2 * (S - 1) * TY * 32 : 1];
+    const int i0 = blockIdx.y * 32;
+    const int tcol = blockIdx.x / (TC_COLS / W), q0 = (blockIdx.x % (TC_COLS / W)) * W;  // tile column, first partial column
+    if (tcol * PG_COLS + (q0 & (PG_COLS - 1)) >= pg.J) return;  // no output column in the patch
     float sc = scale;
     if (amax2) sc = scale / weight_scale_inv(amax2);
-    const int i0 = blockIdx.y * 32;
-    const int tcol = blockIdx.x >> 3, q0 = (blockIdx.x & 7) * 32;  // tile column, first partial column
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    const int tx = threadIdx.x, ty = threadIdx.y, sl = threadIdx.z;  // 32 x TY x S
     const int tr = i0 / TC_ROWS;                   // 128-row block: tile row tr (or tr / 2 with CTA tr % 2)
     const int64_t t = (int64_t)(pairs ? tr >> 1 : tr) * tilesC + tcol;
     const int h = pairs ? tr & 1 : 0;
@@ -1042,21 +1054,24 @@ __global__ void __launch_bounds__(256) k_reduce_pair(const float* __restrict__ p
         const int cg = (q0 >> 2) + ty;
         float4 ar = make_float4(0.f, 0.f, 0.f, 0.f), ai = ar;
         // four partials' loads in flight at a time, added in pair order; an
-        // empty range (or one past c_hi) adds zeros, which change no sum.
-        // Ranges can be empty only when there are fewer units than pairs.
+        // empty range (or one past the slice) adds zeros, which change no
+        // sum.  Ranges can be empty only when there are fewer units than pairs.
         constexpr int B = 4;
         const bool any_empty = U < P;
-        for (int64_t c0 = c_lo; c0 <= c_hi; c0 += B) {
+        const int n = (int)(c_hi + 1 - c_lo), cs = n * sl / S, ce = n * (sl + 1) / S;
+        // owner c_lo's rows of the tile; the next owner's slot is one (two) tiles further
+        const float* base = part + (pairs ? 2 * (c_lo + t) + h : c_lo + t) * TC_TILE_FLOATS +
+                            ((size_t)cg * TC_ROWS + row) * 4;
+        const size_t next = (size_t)(pairs ? 2 : 1) * TC_TILE_FLOATS;
+        for (int c0 = cs; c0 < ce; c0 += B) {
             float4 r[B], m[B];
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                const int64_t cc = c0 + b;
-                const bool use =
-                    cc <= c_hi && (!any_empty || unit_start(cc + 1, U, P) != unit_start(cc, U, P));
-                const int64_t sl = pairs ? 2 * ((use ? cc : c_lo) + t) + h : (use ? cc : c_lo) + t;
-                const float* pt = part + sl * TC_TILE_FLOATS;
-                r[b] = *reinterpret_cast<const float4*>(pt + ((size_t)cg * TC_ROWS + row) * 4);
-                m[b] = *reinterpret_cast<const float4*>(pt + ((size_t)(TC_COLS / 4 + cg) * TC_ROWS + row) * 4);
+                const int c = c0 + b;
+                const bool use = c < ce && (!any_empty || unit_start(c_lo + c + 1, U, P) != unit_start(c_lo + c, U, P));
+                const float* pt = base + (use ? c : cs) * next;
+                r[b] = *reinterpret_cast<const float4*>(pt);
+                m[b] = *reinterpret_cast<const float4*>(pt + (size_t)TC_COLS * TC_ROWS);
                 if (!use) r[b] = m[b] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
@@ -1065,22 +1080,38 @@ __global__ void __launch_bounds__(256) k_reduce_pair(const float* __restrict__ p
                 ai.x += m[b].x; ai.y += m[b].y; ai.z += m[b].z; ai.w += m[b].w;
             }
         }
-        patch[4 * ty + 0][tx] = make_float2(ar.x * sc, ai.x * sc);
-        patch[4 * ty + 1][tx] = make_float2(ar.y * sc, ai.y * sc);
-        patch[4 * ty + 2][tx] = make_float2(ar.z * sc, ai.z * sc);
-        patch[4 * ty + 3][tx] = make_float2(ar.w * sc, ai.w * sc);
+        if constexpr (S > 1) {
+            if (sl > 0) {
+                sums[(2 * (sl - 1) * TY + ty) * 32 + tx] = ar;
+                sums[((2 * (sl - 1) + 1) * TY + ty) * 32 + tx] = ai;
+            }
+            __syncthreads();
+            if (sl == 0)
+#pragma unroll
+                for (int k = 0; k < S - 1; ++k) {
+                    const float4 r = sums[(2 * k * TY + ty) * 32 + tx], m = sums[((2 * k + 1) * TY + ty) * 32 + tx];
+                    ar.x += r.x; ar.y += r.y; ar.z += r.z; ar.w += r.w;
+                    ai.x += m.x; ai.y += m.y; ai.z += m.z; ai.w += m.w;
+                }
+        }
+        if (sl == 0) {
+            patch[4 * ty + 0][tx] = make_float2(ar.x * sc, ai.x * sc);
+            patch[4 * ty + 1][tx] = make_float2(ar.y * sc, ai.y * sc);
+            patch[4 * ty + 2][tx] = make_float2(ar.z * sc, ai.z * sc);
+            patch[4 * ty + 3][tx] = make_float2(ar.w * sc, ai.w * sc);
+        }
     }
     __syncthreads();
-    const int q = q0 + tx;
-    const bool mirrored = q >= PG_COLS;
-    const int j = tcol * PG_COLS + (mirrored ? q - PG_COLS : q);
-    const int off = 2 * j + pg.half;
-    const int c = mirrored ? (pg.C2 - off) / 2 : (pg.C2 + off) / 2;
-    const bool ok = j < pg.J && c >= 0 && c < pg.C && !(mirrored && off == 0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = i0 + ty + 8 * k;
-        if (ok && i < pg.R) out[(int64_t)i * pg.C + c] = patch[tx][ty + 8 * k];
+    // W consecutive threads write one row of the patch
+    for (int e = (sl * TY + ty) * 32 + tx; e < 32 * W; e += 32 * TY * S) {
+        const int ii = e / W, qq = e % W;
+        const int q = q0 + qq, i = i0 + ii;
+        const bool mirrored = q >= PG_COLS;
+        const int j = tcol * PG_COLS + (mirrored ? q - PG_COLS : q);
+        const int off = 2 * j + pg.half;
+        const int c = mirrored ? (pg.C2 - off) / 2 : (pg.C2 + off) / 2;
+        if (i < pg.R && j < pg.J && c >= 0 && c < pg.C && !(mirrored && off == 0))
+            out[(int64_t)i * pg.C + c] = patch[qq][ii];
     }
 }
 
@@ -1498,6 +1529,36 @@ cudaError_t launch_pair_any(bool bf16, int64_t P, cudaStream_t stream, const int
                                                   part, err, wait_ns, stall);
 }
 
+template <int TY, int S>
+void launch_reduce_shape(cudaStream_t st, const float* part, int64_t U, int64_t K, int64_t P, bool pairs,
+                         const PairGeom& pg, int tilesC, float scale, const unsigned* amax2, float2* out)
+{
+    const dim3 grid((unsigned)(tilesC * (TC_COLS / (4 * TY))), (unsigned)((pg.R + 31) / 32));
+    k_reduce_pair<TY, S><<<grid, dim3(32, TY, S), 0, st>>>(part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+}
+
+// The shape of k_reduce_pair by the owners of a tile, P / T: how many partials
+// one output is the sum of.  Many owners (small images: one or two tiles)
+// leave few outputs, so narrow patches and eight slices spread the partials
+// over the SMs; with few owners the patches alone do.  Measured, one adjoint
+// or set-up (FP16x3, us) with <8, 1> (the only shape before), <4, 2>, <4, 4>,
+// <2, 8>:
+//   76 owners  N = 128, L = 8192     adjoint  50.8   40.2   33.8   31.6
+//   76 owners  N = 250, L = 31665    adjoint  65.5   53.9   47.9   45.8
+//   38 owners  N = 192, L = 65536    set-up  241.7  224.2  214.0  212.3
+//   25 owners  N = 384, L = 65536    adjoint 159.4  154.9  152.9  155.1
+//   19 owners  N = 512, L = 131072   adjoint 340.8  338.2  340.7  343.7
+//    9 owners  N = 512, L = 65536    set-up  550.1  549.0  554.0  563.0
+void launch_reduce(cudaStream_t st, const float* part, int64_t U, int64_t K, int64_t P, bool pairs, const PairGeom& pg,
+                   int tilesR, int tilesC, float scale, const unsigned* amax2, float2* out)
+{
+    const int64_t owners = P / ((int64_t)tilesR * tilesC);
+    if (owners >= 32) launch_reduce_shape<2, 8>(st, part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+    else if (owners >= 20) launch_reduce_shape<4, 4>(st, part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+    else if (owners >= 4) launch_reduce_shape<4, 2>(st, part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+    else launch_reduce_shape<8, 1>(st, part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+}
+
 // The paired contraction out[i][c] = scale sum_l A(l,i) B(l,c) with
 // A(l,i) = exp(sa i2pi ka_l (i + oa)), B(l,c) = w_l exp(sb i2pi kb_l (c + ob)).
 int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, const float2* w, int oa, int ob,
@@ -1550,9 +1611,7 @@ int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, 
               : launch_pair_any<false>(bf16, P, p->stream, ka, kb, w, amax, p->L, tilesC, oa, sa, sb, pg.half, pg.J,
                                        K, U, part, p->dflag, wait_ns, stall);
     SPIREC_CK(le);
-    const dim3 rgrid((unsigned)(tilesC * 8), (unsigned)((pg.R + 31) / 32));
-    k_reduce_pair<<<rgrid, dim3(32, 8), 0, p->stream>>>(part, U, K, pairs ? P / 2 : P, pairs, pg, tilesC, scale,
-                                                        amax, out);
+    launch_reduce(p->stream, part, U, K, pairs ? P / 2 : P, pairs, pg, tilesR, tilesC, scale, amax, out);
     SPIREC_CK(cudaGetLastError());
     p->launches += 2;
     return SPIREC_OK;

@@ -1,0 +1,55 @@
+"""Launch shapes that depend on sizes, at the sizes where they can go wrong,
+against the FP64 oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_0908_3252_gb300 import synth
+from tests.helpers import c64, empty_c64, from_dev, rel, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0908_3252_gb300 import build, spirec
+    build.build()
+    spirec.load()
+    yield spirec
+
+
+def _stream():
+    import torch
+    return torch.cuda.current_stream().cuda_stream
+
+
+# The sum of the contraction's partials: CTA counts that give every shape of
+# the sum (76, 25, 9 and 2 owners a tile and more than there are units), one
+# and two column tiles, ragged rows and columns.  The operand split and the
+# FP32 partial sums are below 1e-5 of the result (4e-7 a phase, at most 384
+# accumulation steps between FP32 sums).
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("ctas", [2, 4, 18, 50, 152])
+@pytest.mark.parametrize("N,L", [(5, 40), (37, 2500), (130, 2600)])
+def test_partial_sum_shapes(sp, N, L, ctas, prec):
+    g = synth.rng(N + ctas)
+    kx, ky = synth.uniform_k(L, g)
+    y = c64(synth.complex_normal(L, g))
+    sp.spirec_tune_clear()
+    p = sp.Plan(N, L, 0, prec, _stream())
+    try:
+        for knob in (sp.SPIREC_KNOB_GRAM_SPLIT, sp.SPIREC_KNOB_ADJOINT_SPLIT):
+            sp.spirec_tune_set(knob, N, p.M, prec, L, ctas)
+        sp.spirec_set_trajectory(p.h, kx, ky)
+        G, x = empty_c64((N, 2 * N - 1)), empty_c64((N, N))
+        sp.spirec_gram_dev(p.h, G)
+        sp.spirec_adjoint_dev(p.h, to_dev(y), x)
+        sp.spirec_sync(p.h)
+        assert rel(from_dev(G), O.gram(kx, ky, N)[:, N - 1:].T) < 1e-5
+        assert rel(from_dev(x), O.adjoint(kx, ky, y, N)) < 1e-5
+    finally:
+        p.close()
+        sp.spirec_tune_clear()
