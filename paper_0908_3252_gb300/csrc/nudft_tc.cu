@@ -80,14 +80,10 @@ namespace {
 constexpr int TC_ROWS = 128;        // complex rows per tile (MMA M)
 constexpr int TC_COLS = 256;        // complex columns per tile (MMA N)
 constexpr int TC_KS = 32;           // samples per stage
-constexpr int TC_STAGES = 2;
 constexpr int TC_PRODUCERS = 512;   // 16 warps
 constexpr int TC_THREADS = TC_PRODUCERS + 32;
 constexpr int TC_SEG = 32;          // stages per accumulator segment (at most)
 constexpr int TC_TILE_FLOATS = 2 * TC_COLS * TC_ROWS;  // partial tile: 512 columns x 128 rows
-constexpr uint32_t A_BYTES = TC_ROWS * 128;          // 128 rows x 64 halves
-constexpr uint32_t B_BYTES = TC_COLS * 128;          // 256 rows x 64 halves
-constexpr uint32_t STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // A_hi, A_lo, B_hi, B_lo
 // The paired contraction (G, D): a tile is ROWS rows x 128 B columns, each B
 // column giving two output columns (see PairGeom).  The operands are stored
 // in 64-byte-swizzled K-major tiles of 32 samples per row: A's real and
@@ -215,28 +211,6 @@ __device__ __forceinline__ void tc_fence_before()
 __device__ __forceinline__ void tc_fence_after()
 {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-__device__ __forceinline__ void producers_sync()
-{
-    asm volatile("bar.sync 1, %0;" ::"n"(TC_PRODUCERS) : "memory");
-}
-
-// producers_sync that also returns, to every producer alike, whether any of
-// them passed v = true (a barrier with an OR reduction): a decision every
-// producer takes the same way, as it must be before a named barrier.
-__device__ __forceinline__ bool producers_any(bool v)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)v), "n"(TC_PRODUCERS)
-        : "memory");
-    return r != 0;
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols)
@@ -377,20 +351,24 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t t1, uint32_t t2
     }
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
+// Two loads of 8 TMEM columns behind one wait.
+__device__ __forceinline__ void tmem_ld8x2(uint32_t t0, uint32_t t1, float* a, float* b)
 {
     uint32_t r[16];
-    // load and wait in one statement: the registers are valid only after the wait
+    // loads and wait in one statement: the registers are valid only after the wait
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
         "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
           "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+        : "r"(t0), "r"(t1));
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; ++i) {
+        a[i] = __uint_as_float(r[i]);
+        b[i] = __uint_as_float(r[8 + i]);
+    }
 }
 
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v)
@@ -1138,185 +1116,295 @@ __global__ void k_pair_weights(const float2* __restrict__ w, const int64_t* __re
 // ------------------------------------------------------------ forward H f
 
 // The forward NUDFT (Hf)_l = (1/N) sum_n e^{+i2pi ky_l n} sum_m f[n][m]
-// e^{+i2pi kx_l m} (Eq. ModDirect) as the contraction
-//      P[l][m] = sum_n e^{+i2pi ky_l n} f[n][m]        (tensor cores, K = n)
-// followed by the per-sample dot product y_l = (1/N) sum_m P[l][m]
-// e^{+i2pi kx_l m}.  A tile is 128 samples (TMEM lanes) x 256 image columns
-// m, so each thread of the epilogue owns one sample and sums its own lane's
-// columns: no reduction across lanes.  A (the phases) is generated by the
-// producers; B (the image, split into hi/lo and laid out exactly as a stage
-// expects, k_split_image) arrives per stage by one 64 KB TMA bulk copy.
-// CTA c takes the sample tiles c, c + P, ...; per tile the m-tiles in order,
-// per m-tile the 32-row chunks of n.
+// e^{+i2pi kx_l m} (Eq. ModDirect) as a contraction over the image rows n on
+// the tensor cores, then the per-sample dot product over the columns m.
+//
+// The rows come in pairs n+-(j) = (N - 1 +- (2j + half)) / 2 mirrored about
+// the image centre (half = 1 for even N), whose phases about the centre are
+// conjugate, so with the even and odd parts of the rows
+//      E_j = f[n+] + f[n-],   O_j = f[n+] - f[n-]   (the centre row of odd
+//      N: E_0 = f, O_0 = 0),
+//      P[l][m] = sum_n e^{+i2pi ky n} f[n][m]
+//              = e^{+i2pi ky (N-1)/2} sum_j (cos a_j E_j[m] + i sin a_j O_j[m]),
+// a_j = 2 pi ky (j + half / 2): four real products of depth K = J = ceil(N/2)
+// instead of N, and half the phases.  Re P = C Er - S Oi, Im P = C Ei + S Or;
+// y_l = (1/N) e^{+i2pi ky (N-1)/2} sum_m P'[l][m] e^{+i2pi kx_l m}.
+//
+// The kernel runs on CTA pairs: a pair tile is 256 samples (CTA h: TMEM lanes
+// = samples 128 h .. +127) x mw image columns (mw <= 256, the columns spread
+// evenly over the m-tiles), so each thread of the epilogue owns one sample
+// and sums its own lane's columns: no reduction across lanes.  A (cos and
+// sin, generated by the producers) is each CTA's own; B (the folded image,
+// split into hi/lo and laid out as a stage expects, k_split_image) is halved
+// over the pair, so a stage of 32 j brings 64 KB (mw = 256) to each SM by one
+// TMA bulk copy: with one CTA a tile it would be 128 KB, 10 TB/s out of the
+// L2.  Pair c takes the sample tiles c, c + P, ...; per tile the m-tiles in
+// order, per m-tile the 32-row chunks of j.
+//
+// Bound by the tensor core: 4.12e11 issued flop (three split products of half
+// the algorithmic 8 N^2 L) at 512^2, L = 131072 in a call of 242 us, 87% of
+// the measured bf16 rate over the whole call (482 us with all N rows as the
+// depth and one CTA a tile); N = 64, L = 8000: 23.1 -> 20.1 us, N = 300,
+// L = 32000: 99.6 -> 52.3 us.
 
-constexpr uint32_t FW_YPART = TC_STAGES * STAGE_BYTES;  // 4 x 128 float2
-constexpr uint32_t FW_BAR = FW_YPART + 4 * TC_ROWS * 8;
-constexpr uint32_t FW_SMEM = FW_BAR + 128 + 1024;
+constexpr int FW_STAGES = 2;
+constexpr uint32_t FW_A = TC_ROWS * 128;              // [cos 32 | sin 32] halves a row; hi, then lo
+constexpr uint32_t FW_BMAX = 4 * (TC_COLS / 2) * 128;  // E hi, E lo, O hi, O lo of 128 columns
+constexpr uint32_t FW_STAGE = 2 * FW_A + FW_BMAX;
+constexpr uint32_t FW_YPART = FW_STAGES * FW_STAGE;    // 2 (tile parity) x 3 x 128 float2
+constexpr uint32_t FW_BAR = FW_YPART + 2 * 3 * TC_ROWS * 8;
+constexpr uint32_t FW_SMEM = FW_BAR + 256 + 1024;
 static_assert(FW_SMEM <= 232448, "shared memory per CTA");
-constexpr uint32_t FW_BLOCK = 2 * B_BYTES;  // one m-tile x 32-row chunk: hi then lo
+static_assert(8 * (3 * FW_STAGES + 3 + 8) + 8 <= 256, "barrier area");
+constexpr int FW_ARRIVALS = 2 * TC_PRODUCERS / 32 + 1;  // the pair's producer warps, CTA 1's image block
 
-// Image f (N x N, row n, column m) -> per (m-tile, n-chunk) block the B
-// operand of a stage: rows m (256), K = 32 values of n as [re | im], hi and
-// lo halves, 128-byte-swizzled K-major.  Rows m >= N and n >= N are zero.
-// The values are scaled by 2^-e, 2^e >= max |f| (amax2 = max |f|^2), so the
-// FP16 halves stay in range; k_tc_forward undoes the scale.
+// Sizes of the forward contraction of an N x N image.
+struct FwGeom {
+    int N, J, half;  // folded rows j < J, at offsets j + half / 2 from the centre
+    int kchunks;     // chunks of 32 j
+    int mtiles, mw;  // m-tiles of mw columns, a multiple of 32 (the pair MMA's N)
+    __host__ __device__ uint32_t plane() const { return (uint32_t)mw * 64; }  // mw / 2 rows of 128 bytes
+    __host__ __device__ uint32_t block() const { return 4 * plane(); }        // one CTA's B of a stage
+};
+
+__host__ __device__ __forceinline__ FwGeom fw_geom(int N)
+{
+    FwGeom g;
+    g.N = N;
+    g.half = (N & 1) ? 0 : 1;
+    g.J = (N + 1) / 2;
+    g.kchunks = (g.J + TC_KS - 1) / TC_KS;
+    g.mtiles = (N + TC_COLS - 1) / TC_COLS;
+    g.mw = ((N + g.mtiles - 1) / g.mtiles + 31) / 32 * 32;
+    return g;
+}
+
+// Image f (N x N, row n, column m) -> per (m-tile, j-chunk, CTA of the pair)
+// block the B operand of a stage: planes E hi, E lo, O hi, O lo of mw / 2
+// rows (columns m) x 32 values of j as [re | im] halves, 128-byte-swizzled
+// K-major.  Rows m >= N and j >= J are zero.  The values are scaled by
+// 2^-(e+1), 2^e >= max |f| (amax2 = max |f|^2), so the FP16 halves stay in
+// range; k_tc_forward undoes the scale.
 template <bool BF16>
-__global__ void k_split_image(const float2* __restrict__ f, int N, int kchunks, const unsigned* __restrict__ amax2,
+__global__ void k_split_image(const float2* __restrict__ f, FwGeom fg, const unsigned* __restrict__ amax2,
                               uint8_t* __restrict__ FB)
 {
-    const float wmul = weight_scale_inv(amax2);
-    const int mtiles = (N + TC_COLS - 1) / TC_COLS;
-    const int64_t total = (int64_t)mtiles * TC_COLS * kchunks * 4;  // (m, chunk, group of 8 n)
+    const float wmul = 0.5f * weight_scale_inv(amax2);
+    const int N = fg.N, cols = fg.mtiles * fg.mw;
+    const int64_t total = (int64_t)cols * fg.kchunks * 4;  // (m, chunk, group of 8 j)
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int m = (int)(e % (mtiles * TC_COLS));  // consecutive threads: consecutive m
-        const int64_t rest = e / (mtiles * TC_COLS);
+        const int m = (int)(e % cols);  // consecutive threads: consecutive m
+        const int64_t rest = e / cols;
         const int g = (int)(rest & 3), kc = (int)(rest >> 2);
-        float re[8], im[8];
+        float er[8], ei[8], orr[8], oi[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int n = 32 * kc + 8 * g + j;
-            const float2 v = (m < N && n < N) ? f[(int64_t)n * N + m] : make_float2(0.f, 0.f);
-            re[j] = v.x * wmul;
-            im[j] = v.y * wmul;
+        for (int i = 0; i < 8; ++i) {
+            const int j = 32 * kc + 8 * g + i, off = 2 * j + fg.half;
+            const bool in = m < N && j < fg.J;
+            const int np = (N - 1 + off) / 2, nm = (N - 1 - off) / 2;
+            const float2 a = in ? f[(int64_t)np * N + m] : make_float2(0.f, 0.f);
+            const float2 b = in && off > 0 ? f[(int64_t)nm * N + m] : make_float2(0.f, 0.f);
+            er[i] = (a.x + b.x) * wmul;
+            ei[i] = (a.y + b.y) * wmul;
+            orr[i] = off > 0 ? (a.x - b.x) * wmul : 0.f;
+            oi[i] = off > 0 ? (a.y - b.y) * wmul : 0.f;
         }
-        uint4 rh, rl, ih, il;
-        split8<BF16>(re, rh, rl);
-        split8<BF16>(im, ih, il);
-        const int mt = m / TC_COLS, r = m % TC_COLS;
-        uint8_t* blk = FB + ((int64_t)mt * kchunks + kc) * FW_BLOCK;
-        *reinterpret_cast<uint4*>(blk + sw128(r, g)) = rh;
-        *reinterpret_cast<uint4*>(blk + sw128(r, 4 + g)) = ih;
-        *reinterpret_cast<uint4*>(blk + B_BYTES + sw128(r, g)) = rl;
-        *reinterpret_cast<uint4*>(blk + B_BYTES + sw128(r, 4 + g)) = il;
+        const int mt = m / fg.mw, mm = m % fg.mw, h = mm / (fg.mw / 2), r = mm % (fg.mw / 2);
+        uint8_t* blk = FB + (((int64_t)mt * fg.kchunks + kc) * 2 + h) * fg.block();
+        uint4 hi, lo;
+        split8<BF16>(er, hi, lo);
+        *reinterpret_cast<uint4*>(blk + sw128(r, g)) = hi;
+        *reinterpret_cast<uint4*>(blk + fg.plane() + sw128(r, g)) = lo;
+        split8<BF16>(ei, hi, lo);
+        *reinterpret_cast<uint4*>(blk + sw128(r, 4 + g)) = hi;
+        *reinterpret_cast<uint4*>(blk + fg.plane() + sw128(r, 4 + g)) = lo;
+        split8<BF16>(orr, hi, lo);
+        *reinterpret_cast<uint4*>(blk + 2 * fg.plane() + sw128(r, g)) = hi;
+        *reinterpret_cast<uint4*>(blk + 3 * fg.plane() + sw128(r, g)) = lo;
+        split8<BF16>(oi, hi, lo);
+        *reinterpret_cast<uint4*>(blk + 2 * fg.plane() + sw128(r, 4 + g)) = hi;
+        *reinterpret_cast<uint4*>(blk + 3 * fg.plane() + sw128(r, 4 + g)) = lo;
     }
 }
 
+// Barriers: full[s] (the leader's) completes when the producer warps of both
+// CTAs have stored their A rows of the stage and CTA 1's image block has
+// landed (its warp 16 relays bblk[s], which counts the CTA's own block; the
+// leader's MMA issuer waits on its own bblk[s] itself); empty[s] in both CTAs
+// by the commit of the stage's MMAs; acc_full in both CTAs by the commit of a
+// segment (one m-tile of one sample tile); acc_empty (the leader's) by every
+// producer warp of the pair once it has read its columns.
 template <bool BF16>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_tc_forward(const int64_t* __restrict__ kxq, const int64_t* __restrict__ kyq, const uint8_t* __restrict__ FB,
-             const unsigned* __restrict__ amax2, int64_t L, int N, int kchunks, float scale, float2* __restrict__ y,
-             int* err, unsigned long long wait_ns, int stall)
+             const unsigned* __restrict__ amax2, int64_t L, FwGeom fg, float scale, float2* __restrict__ y, int* err,
+             unsigned long long wait_ns, int stall)
 {
-    scale /= weight_scale_inv(amax2);  // undoes k_split_image's 2^-e
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar_full = sbase + FW_BAR;             // TC_STAGES: A generated and B landed
-    const uint32_t bar_empty = bar_full + 8 * TC_STAGES;  // TC_STAGES: stage consumed
-    const uint32_t bar_acc_full = bar_empty + 8 * TC_STAGES;
+    const uint32_t bar_full = sbase + FW_BAR;
+    const uint32_t bar_empty = bar_full + 8 * FW_STAGES;
+    const uint32_t bar_bblk = bar_empty + 8 * FW_STAGES;
+    const uint32_t bar_acc_full = bar_bblk + 8 * FW_STAGES;
     const uint32_t bar_acc_empty = bar_acc_full + 8;
     const uint32_t bar_drain = bar_acc_empty + 8;  // every MMA issued has completed
-    const uint32_t misc = FW_BAR + 8 * (2 * TC_STAGES + 3);
+    const uint32_t bar_y = bar_drain + 8;          // [tile parity][lane quarter]: the column quarters' sums are stored
+    const uint32_t misc = FW_BAR + 8 * (3 * FW_STAGES + 3 + 8);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + misc);
-    float2* ypart = reinterpret_cast<float2*>(smem + FW_YPART);  // [4 column quarters][128 samples]
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + misc + 4);
+    float2* ypart = reinterpret_cast<float2*>(smem + FW_YPART);  // [tile parity][quarter 1..3][sample]
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int mtiles = (N + TC_COLS - 1) / TC_COLS;
-    const int64_t ntiles = (L + TC_ROWS - 1) / TC_ROWS;
-    const int64_t my_tiles = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
-    const int per_tile = mtiles * kchunks;
-    const int n = (int)(my_tiles * per_tile);
+    // the launch's clusters are pairs of consecutive blocks
+    const uint32_t rank = blockIdx.x & 1u;
+    const int64_t pair = blockIdx.x >> 1, P2 = gridDim.x >> 1;
+    const int64_t ntiles = (L + 2 * TC_ROWS - 1) / (2 * TC_ROWS);
+    const int my_tiles = (int)((ntiles - pair + P2 - 1) / P2);
+    const int per_tile = fg.mtiles * fg.kchunks;
+    const int n = my_tiles * per_tile;
+    const uint32_t plane = fg.plane(), bbytes = fg.block();
 
     if (tid == 0) {
-        for (int i = 0; i < TC_STAGES; ++i) {
-            mbar_init(bar_full + 8 * i, TC_PRODUCERS + 1);
+        for (int i = 0; i < FW_STAGES; ++i) {
+            mbar_init(bar_full + 8 * i, FW_ARRIVALS);
             mbar_init(bar_empty + 8 * i, 1);
+            mbar_init(bar_bblk + 8 * i, 1);
         }
         mbar_init(bar_acc_full, 1);
-        mbar_init(bar_acc_empty, TC_PRODUCERS);
+        mbar_init(bar_acc_empty, FW_ARRIVALS - 1);
         mbar_init(bar_drain, 1);
+        for (int q = 0; q < 8; ++q) mbar_init(bar_y + 8 * q, 3);
+        *abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == TC_PRODUCERS / 32) tmem_alloc(smem_u32(tmem_slot), 512);
+    if (warp == TC_PRODUCERS / 32) tmem_alloc2(smem_u32(tmem_slot), 512);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();  // both CTAs' barriers are initialised before any arrival from the other
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp < TC_PRODUCERS / 32) {
         // ------------------------------------------------ producers
-        // A wait that runs out sets the thread's `late`; the producers decide
-        // to stop together, at the OR-barrier that starts each stage, so none
-        // is left alone at a named barrier of the epilogue.
-        const int r = tid & 127, g = tid >> 7;  // A row (sample in the tile), group of 8 n
+        scale *= 2.f / weight_scale_inv(amax2);  // undoes k_split_image's 2^-(e+1)
+        const int r = tid & 127, g = tid >> 7;   // A row (sample of this CTA), group of 8 j
+        const int lq = warp & 3, cq = warp >> 2;  // epilogue: lane quarter, column quarter
+        const int rs = 32 * lq + lane;           // epilogue: sample of this CTA
         int issued = 0;                          // stages whose image block thread 0 requested
-        bool late = false, stopped = false;
-        int64_t ka = 0;                          // ky of this thread's sample (fixed point)
-        int64_t cur_tile = -1;
-        float2 ysum = make_float2(0.f, 0.f);     // threads 0..127: y of sample tid over m-tiles
-        // the epilogue of the segment (tile t, m-tile mt): this warp's 64 columns
-        auto epilogue = [&](int64_t t, int mt) {
-            __syncwarp();  // the tensor-memory loads are warp-collective
-            const int lq = warp & 3, cq = warp >> 2;
-            const int rs = 32 * lq + lane;
-            const int64_t l = t * TC_ROWS + rs;
-            const int64_t kx = l < L ? kxq[l] : 0;
-            float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 1
-            for (int cc = 0; cc < 64; cc += 16) {
-                float re[16], im[16];
-                const uint32_t ta = tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(64 * cq + cc);
-                tmem_ld16(ta, re);
-                tmem_ld16(ta + TC_COLS, im);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float2 w = phasor_fast(kx, mt * TC_COLS + 64 * cq + cc + j);
-                    acc.x = fmaf(re[j], w.x, fmaf(-im[j], w.y, acc.x));
-                    acc.y = fmaf(re[j], w.y, fmaf(im[j], w.x, acc.y));
-                }
+        bool failed = false;                     // a wait of this thread ran out
+        uint32_t klo = 0, khi = 0, kch = 0;      // ky of sample r: low, high word, the half offset's top word
+        int64_t kx = 0;                          // kx of the epilogue's sample
+        float2 ysum = make_float2(0.f, 0.f);     // this thread's columns of that sample's dot product
+        auto sample = [&](int tile, int row) {
+            return (pair + (int64_t)tile * P2) * (2 * TC_ROWS) + (int64_t)rank * TC_ROWS + row;
+        };
+        // the epilogue of the segment seg = (tile number `tile` of this pair,
+        // m-tile mt): this warp's mw / 4 columns, eight at a time.  The
+        // phasor of column c0 + j is that of c0 times that of j, j < 8: 8 + 8
+        // instead of 64 sin/cos pairs a thread.
+        auto epilogue = [&](int seg, int tile, int mt) {
+            const bool landed = mbar_wait(bar_acc_full, (uint32_t)seg & 1, wait_ns);
+            if (!landed) {
+                atomicOr(err, kErrTimeout);
+                *abort_flag = 1;
             }
-            ypart[cq * TC_ROWS + rs] = acc;
-            producers_sync();
-            if (tid < TC_ROWS) {
-                const float2 a = ypart[tid], b = ypart[TC_ROWS + tid], c = ypart[2 * TC_ROWS + tid],
-                             d = ypart[3 * TC_ROWS + tid];
-                ysum.x += ((a.x + b.x) + c.x) + d.x;
-                ysum.y += ((a.y + b.y) + c.y) + d.y;
-                if (mt == mtiles - 1) {
-                    const int64_t lo = t * TC_ROWS + tid;
-                    if (lo < L) y[lo] = make_float2(ysum.x * scale, ysum.y * scale);
-                    ysum = make_float2(0.f, 0.f);
+            if (!__all_sync(0xffffffffu, landed)) {
+                failed = true;
+                return;
+            }
+            tc_fence_after();
+            const int w4 = fg.mw / 4;
+            const uint32_t ta = tmem + ((uint32_t)(32 * lq) << 16) + (uint32_t)(w4 * cq);
+            float2 wj[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) wj[j] = phasor_fast(kx, j);
+#pragma unroll 1
+            for (int cc = 0; cc < w4; cc += 8) {
+                float re[8], im[8];
+                tmem_ld8x2(ta + cc, ta + TC_COLS + cc, re, im);
+                float2 a = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    a.x = fmaf(re[j], wj[j].x, fmaf(-im[j], wj[j].y, a.x));
+                    a.y = fmaf(re[j], wj[j].y, fmaf(im[j], wj[j].x, a.y));
                 }
+                const float2 w = phasor_fast(kx, mt * fg.mw + w4 * cq + cc);
+                ysum.x = fmaf(a.x, w.x, fmaf(-a.y, w.y, ysum.x));
+                ysum.y = fmaf(a.x, w.y, fmaf(a.y, w.x, ysum.y));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(bar_acc_empty, 0);
+            if (mt == fg.mtiles - 1) {
+                // the four column quarters' sums of a sample, added by quarter
+                // 0's warp in order.  Buffers and barriers by tile parity: a
+                // warp writes tile t + 2 only after every warp has arrived on
+                // acc_empty for tile t + 1, which quarter 0's warp does after
+                // it has read tile t.
+                const uint32_t by = bar_y + 8 * (4 * (tile & 1) + lq);
+                float2* yp = ypart + (tile & 1) * 3 * TC_ROWS + rs;
+                if (cq > 0) {
+                    yp[(cq - 1) * TC_ROWS] = ysum;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(by);
+                } else {
+                    const int64_t l = sample(tile, rs);
+                    const int64_t ky = l < L ? kyq[l] : 0;
+                    const float2 c = phasor_q(ky >> 1, fg.N - 1);  // the centre row's phase
+                    if (!mbar_wait(by, (uint32_t)(tile >> 1) & 1, wait_ns)) {
+                        atomicOr(err, kErrTimeout);
+                        *abort_flag = 1;
+                        failed = true;
+                    } else if (l < L) {
+                        const float2 b = yp[0], d = yp[TC_ROWS], e = yp[2 * TC_ROWS];
+                        const float2 v = make_float2(((ysum.x + b.x) + d.x) + e.x, ((ysum.y + b.y) + d.y) + e.y);
+                        const float2 o = cmul(v, c);
+                        y[l] = make_float2(o.x * scale, o.y * scale);
+                    }
+                }
+                ysum = make_float2(0.f, 0.f);
             }
         };
-        int64_t seg_t = 0;  // the segment being accumulated
-        int seg_mt = 0;
+        int tile = 0, mt = 0, kc = 0;  // of stage `it`
+        int ptile = 0, pmt = 0, seg = 0;  // of the segment being accumulated
+        bool stopped = false;
         for (int it = 0; it < n; ++it) {
-            const int s = it % TC_STAGES;
-            const uint32_t use = (uint32_t)(it / TC_STAGES);
-            const int64_t t = blockIdx.x + (int64_t)(it / per_tile) * gridDim.x;
-            const int rem = it % per_tile, mt = rem / kchunks, kc = rem % kchunks;
-            if (tid == 0 && it >= TC_STAGES && !mbar_wait(bar_empty + 8 * s, (use - 1) & 1, wait_ns)) {
-                late = true;
+            const int s = it % FW_STAGES;
+            const uint32_t use = (uint32_t)(it / FW_STAGES);
+            if (lane == 0 && it >= FW_STAGES && !mbar_wait(bar_empty + 8 * s, (use - 1) & 1, wait_ns)) {
+                *abort_flag = 1;
                 atomicOr(err, kErrTimeout);
+                failed = true;
             }
-            if (producers_any(late)) {  // stage s is free, or every producer stops here
+            // the warp stops as one: at once on a wait of its own that ran
+            // out, on another warp's (the shared flag) within four stages
+            if (__any_sync(0xffffffffu, failed || ((it & 3) == 0 && *abort_flag != 0))) {
                 stopped = true;
                 break;
             }
-            const uint32_t st = sbase + (uint32_t)s * STAGE_BYTES;
-            const uint32_t aH = st, aL = st + A_BYTES, bH = st + 2 * A_BYTES;
-            // from here to its arrival below every producer completes the
-            // stage, so the phase of bar_full[s] ends once the block lands
+            const uint32_t st = sbase + (uint32_t)s * FW_STAGE;
+            const uint32_t aH = st, aL = st + FW_A;
             if (tid == 0) {
                 ++issued;
                 fence_proxy_async();
-                mbar_expect_tx(bar_full + 8 * s, FW_BLOCK);
-                bulk_g2s(bH, FB + ((int64_t)mt * kchunks + kc) * FW_BLOCK, FW_BLOCK, bar_full + 8 * s);
+                mbar_expect_tx(bar_bblk + 8 * s, bbytes);
+                bulk_g2s(st + 2 * FW_A, FB + (((int64_t)mt * fg.kchunks + kc) * 2 + rank) * bbytes, bbytes,
+                         bar_bblk + 8 * s);
             }
-            if (t != cur_tile) {
-                const int64_t l = t * TC_ROWS + r;
-                ka = l < L ? kyq[l] : 0;
-                cur_tile = t;
+            if (mt == 0 && kc == 0) {
+                const int64_t l = sample(tile, r);
+                const uint64_t k = l < L ? (uint64_t)kyq[l] : 0;
+                klo = (uint32_t)k;
+                khi = (uint32_t)(k >> 32);
+                kch = fg.half ? (uint32_t)((int32_t)khi >> 1) : 0u;
             }
-            const bool valid = t * TC_ROWS + r < L;
             float re[8], im[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                float2 v = phasor_fast(ka, 32 * kc + 8 * g + e);
-                if (!valid) v = make_float2(0.f, 0.f);
+                const float2 v = phasor_top(klo, khi, kch, (uint32_t)(32 * kc + 8 * g + e), 1.4629180792671596e-09f);
                 re[e] = v.x;
                 im[e] = v.y;
             }
@@ -1328,97 +1416,108 @@ k_tc_forward(const int64_t* __restrict__ kxq, const int64_t* __restrict__ kyq, c
             st_shared_v4(aL + sw128(r, g), rl);
             st_shared_v4(aL + sw128(r, 4 + g), il);
             fence_proxy_async();
-            mbar_arrive(bar_full + 8 * s);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(bar_full + 8 * s, 0);
             if (kc == 0) {
-                if (it > 0) {
-                    // the MMA has the first stage of a new segment queued: the
-                    // epilogue of the previous one
-                    const int j = it / kchunks - 1;
-                    if (!mbar_wait(bar_acc_full, (uint32_t)j & 1, wait_ns)) {
-                        atomicOr(err, kErrTimeout);
-                        late = true;  // every producer still runs the epilogue (it holds a named barrier)
-                    }
-                    tc_fence_after();
-                    epilogue(seg_t, seg_mt);
-                    tc_fence_before();
-                    mbar_arrive(bar_acc_empty);
+                // the MMA has the first stage of a new segment queued: the
+                // epilogue of the previous one
+                if (it > 0) epilogue(seg++, ptile, pmt);
+                ptile = tile;
+                pmt = mt;
+                if (mt == 0) {
+                    const int64_t l = sample(tile, rs);
+                    kx = l < L ? kxq[l] : 0;
                 }
-                seg_t = t;
-                seg_mt = mt;
+            }
+            if (++kc == fg.kchunks) {
+                kc = 0;
+                if (++mt == fg.mtiles) {
+                    mt = 0;
+                    ++tile;
+                }
             }
         }
-        if (n > 0 && !stopped) {
-            const int j = n / kchunks - 1;
-            if (!mbar_wait(bar_acc_full, (uint32_t)j & 1, wait_ns)) {
-                atomicOr(err, kErrTimeout);
-                late = true;
-            }
-            if (!producers_any(late)) {  // the last epilogue: all producers or none
-                tc_fence_after();
-                epilogue(seg_t, seg_mt);
-            }
-        }
+        // the last segment (a warp runs it as one, or not at all)
+        if (n > 0 && !stopped && !__any_sync(0xffffffffu, failed || *abort_flag != 0)) epilogue(seg, ptile, pmt);
         // every requested image block has landed before the CTA goes (the
-        // open requests are among the last TC_STAGES stages)
+        // open requests are among the last FW_STAGES stages)
         if (tid == 0)
-            for (int j = issued > TC_STAGES ? issued - TC_STAGES : 0; j < issued; ++j)
-                if (!mbar_wait(bar_full + 8 * (j % TC_STAGES), (uint32_t)(j / TC_STAGES) & 1, kDrainNs))
+            for (int j = issued > FW_STAGES ? issued - FW_STAGES : 0; j < issued; ++j)
+                if (!mbar_wait(bar_bblk + 8 * (j % FW_STAGES), (uint32_t)(j / FW_STAGES) & 1, kDrainNs))
                     atomicOr(err, kErrTimeout);
-    } else if (lane == 0) {
-        // ------------------------------------------------ MMA issuer
+    } else if (rank == 1 && lane == 0) {
+        // ------------------------------------------------ CTA 1: its image block has landed
+        for (int it = 0; it < n; ++it) {
+            const int s = it % FW_STAGES;
+            if (!mbar_wait(bar_bblk + 8 * s, (uint32_t)(it / FW_STAGES) & 1, wait_ns)) {
+                atomicOr(err, kErrTimeout);
+                *abort_flag = 1;
+                break;
+            }
+            fence_proxy_async();
+            mbar_arrive_cluster(bar_full + 8 * s, 0);
+        }
+    } else if (rank == 0 && lane == 0) {
+        // ------------------------------------------------ MMA issuer (the pair's)
         const uint32_t fmt = BF16 ? 1u : 0u;
-        const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
-        const uint32_t idesc_neg = idesc | (1u << 13);
+        const uint32_t idesc =
+            (1u << 4) | (fmt << 7) | (fmt << 10) | (((uint32_t)fg.mw >> 3) << 17) | ((256u >> 4) << 24);
+        const uint32_t idesc_neg = idesc | (1u << 13);  // negates A
         const uint32_t tre = tmem, tim = tmem + TC_COLS;
         int issued = 0;  // stages whose MMAs were issued
         // a test's injected stall (as in k_tc_pair_gemm)
         if (stall && !mbar_wait(bar_drain, 0, wait_ns)) atomicOr(err, kErrTimeout);
+        int kc = 0, seg = 0;
         for (int it = 0; !stall && it < n; ++it) {
-            const int s = it % TC_STAGES;
-            const uint32_t use = (uint32_t)(it / TC_STAGES);
-            const int kc = (it % per_tile) % kchunks;
-            const int seg = it / kchunks;
+            const int s = it % FW_STAGES;
+            const uint32_t use = (uint32_t)(it / FW_STAGES);
             if (kc == 0 && seg >= 1 && !mbar_wait(bar_acc_empty, (uint32_t)(seg - 1) & 1, wait_ns)) {
                 atomicOr(err, kErrTimeout);
                 break;
             }
-            if (!mbar_wait(bar_full + 8 * s, use & 1, wait_ns)) {
+            if (!mbar_wait(bar_full + 8 * s, use & 1, wait_ns) || !mbar_wait(bar_bblk + 8 * s, use & 1, wait_ns)) {
                 atomicOr(err, kErrTimeout);
                 break;
             }
             ++issued;
             tc_fence_after();
-            const uint32_t st = sbase + (uint32_t)s * STAGE_BYTES;
-            const uint32_t aH = st, aL = st + A_BYTES, bH = st + 2 * A_BYTES, bL = bH + B_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
+            const uint32_t st = sbase + (uint32_t)s * FW_STAGE;
+            const uint32_t aH = st, aL = st + FW_A, eH = st + 2 * FW_A, oH = eH + 2 * plane;
+            const int slices = fg.J - 32 * kc > 16 ? 2 : 1;  // 16 j each
+            for (int kk = 0; kk < slices; ++kk) {
                 const uint32_t oR = 32u * kk, oI = 64u + 32u * kk;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {  // hi*hi, hi*lo, lo*hi
-                    const uint32_t A = q == 2 ? aL : aH, B = q == 1 ? bL : bH;
+                    const uint32_t A = q == 2 ? aL : aH, E = q == 1 ? eH + plane : eH, O = q == 1 ? oH + plane : oH;
                     const uint32_t acc = (kc > 0 || kk > 0 || q > 0) ? 1u : 0u;
-                    mma_f16(tre, sdesc(A + oR), sdesc(B + oR), idesc, acc);
-                    mma_f16(tre, sdesc(A + oI), sdesc(B + oI), idesc_neg, 1u);
-                    mma_f16(tim, sdesc(A + oR), sdesc(B + oI), idesc, acc);
-                    mma_f16(tim, sdesc(A + oI), sdesc(B + oR), idesc, 1u);
+                    mma2_f16(tre, sdesc(A + oR), sdesc(E + oR), idesc, acc);
+                    mma2_f16(tim, sdesc(A + oR), sdesc(E + oI), idesc, acc);
+                    mma2_f16(tre, sdesc(A + oI), sdesc(O + oI), idesc_neg, 1u);
+                    mma2_f16(tim, sdesc(A + oI), sdesc(O + oR), idesc, 1u);
                 }
             }
-            mma_commit(bar_empty + 8 * s);
-            if (kc == kchunks - 1) mma_commit(bar_acc_full);
+            mma2_commit_pair(bar_empty + 8 * s);
+            if (++kc == fg.kchunks) {
+                mma2_commit_pair(bar_acc_full);
+                kc = 0;
+                ++seg;
+            }
         }
-        // no MMA may still read the stages or write TMEM once the CTA frees it
+        // no MMA may still read the stages (of either CTA) or write TMEM once
+        // the CTAs free it
         if (issued > 0) {
-            mma_commit(bar_drain);
+            mma2_commit_pair(bar_drain);
             if (!mbar_wait(bar_drain, 0, kDrainNs)) atomicOr(err, kErrTimeout);
         }
     }
 
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     if (warp == TC_PRODUCERS / 32) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc2(tmem, 512);
     }
 }
 
@@ -1622,10 +1721,8 @@ int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, 
 int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
 {
     const int N = p->N;
-    const int kchunks = (N + TC_KS - 1) / TC_KS;
-    const int mtiles = (N + TC_COLS - 1) / TC_COLS;
-    const size_t fb_bytes = (size_t)mtiles * kchunks * FW_BLOCK;
-    if (!p->fsplit || p->fsplit_bytes < fb_bytes) {
+    const FwGeom fg = fw_geom(N);
+    if (!p->fsplit || p->fsplit_bytes < fsplit_bytes_tc(N, p->precision)) {
         set_error("plan has no split-image buffer for the forward contraction");
         return SPIREC_ESTATE;
     }
@@ -1638,33 +1735,44 @@ int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
         if (blocks > 4 * kMaxCtas) blocks = 4 * kMaxCtas;
         k_absmax2<<<blocks, 256, 0, p->stream>>>(x, NN, amax);
         SPIREC_CK(cudaGetLastError());
-        const int64_t total = (int64_t)mtiles * TC_COLS * kchunks * 4;
+        const int64_t total = (int64_t)fg.mtiles * fg.mw * fg.kchunks * 4;
         blocks = (int)((total + 255) / 256);
         if (blocks > 8 * kMaxCtas) blocks = 8 * kMaxCtas;
         if (bf16)
-            k_split_image<true><<<blocks, 256, 0, p->stream>>>(x, N, kchunks, amax, p->fsplit);
+            k_split_image<true><<<blocks, 256, 0, p->stream>>>(x, fg, amax, p->fsplit);
         else
-            k_split_image<false><<<blocks, 256, 0, p->stream>>>(x, N, kchunks, amax, p->fsplit);
+            k_split_image<false><<<blocks, 256, 0, p->stream>>>(x, fg, amax, p->fsplit);
         SPIREC_CK(cudaGetLastError());
     }
-    int dev = 0, sms = 0;
-    SPIREC_CK(cudaGetDevice(&dev));
-    SPIREC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t ntiles = (p->L + TC_ROWS - 1) / TC_ROWS;
-    int64_t P = sms < kMaxCtas ? sms : kMaxCtas;
-    if (P > ntiles) P = ntiles;
+    int sms = 0, clusters = 0, rc;
+    if ((rc = device_sms(&sms)) != SPIREC_OK) return rc;
+    if ((rc = pair_clusters(&clusters)) != SPIREC_OK) return rc;
+    const int64_t ntiles = (p->L + 2 * TC_ROWS - 1) / (2 * TC_ROWS);
+    int64_t P2 = (sms < kMaxCtas ? sms : kMaxCtas) / 2;
+    if (P2 > clusters) P2 = clusters;
+    if (P2 > ntiles) P2 = ntiles;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(2 * P2));
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = FW_SMEM;
+    cfg.stream = p->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     const float scale = 1.0f / (float)N;
+    const int stall = injected_stall(kStallContraction) ? 1 : 0;
+    const uint8_t* fb = p->fsplit;
+    const unsigned* am = amax;
     if (bf16)
-        k_tc_forward<true><<<(unsigned)P, TC_THREADS, FW_SMEM, p->stream>>>(p->kxq, p->kyq, p->fsplit, amax, p->L,
-                                                                           N, kchunks, scale, yout, p->dflag,
-                                                                           wait_limit_ns(),
-                                                                           injected_stall(kStallContraction) ? 1 : 0);
+        SPIREC_CK(cudaLaunchKernelEx(&cfg, k_tc_forward<true>, (const int64_t*)p->kxq, (const int64_t*)p->kyq, fb, am,
+                                     p->L, fg, scale, yout, p->dflag, wait_limit_ns(), stall));
     else
-        k_tc_forward<false><<<(unsigned)P, TC_THREADS, FW_SMEM, p->stream>>>(p->kxq, p->kyq, p->fsplit, amax,
-                                                                            p->L, N, kchunks, scale, yout, p->dflag,
-                                                                            wait_limit_ns(),
-                                                                            injected_stall(kStallContraction) ? 1 : 0);
-    SPIREC_CK(cudaGetLastError());
+        SPIREC_CK(cudaLaunchKernelEx(&cfg, k_tc_forward<false>, (const int64_t*)p->kxq, (const int64_t*)p->kyq, fb, am,
+                                     p->L, fg, scale, yout, p->dflag, wait_limit_ns(), stall));
     p->launches += 3;
     return SPIREC_OK;
 }
@@ -1672,8 +1780,8 @@ int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
 size_t fsplit_bytes_tc(int N, int precision)
 {
     if (precision == SPIREC_FP32) return 0;
-    const size_t kchunks = (size_t)(N + TC_KS - 1) / TC_KS, mtiles = (size_t)(N + TC_COLS - 1) / TC_COLS;
-    return mtiles * kchunks * FW_BLOCK;
+    const FwGeom fg = fw_geom(N);
+    return (size_t)fg.mtiles * fg.kchunks * 2 * fg.block();
 }
 
 size_t kpart_floats_tc(int N, int64_t, int precision)

@@ -53,3 +53,22 @@ def test_partial_sum_shapes(sp, N, L, ctas, prec):
     finally:
         p.close()
         sp.spirec_tune_clear()
+
+
+# The forward contraction: odd and even image sides (the centre row alone or
+# paired), one and several chunks of folded rows with one or two 16-deep
+# slices in the last, one and two column tiles of uneven width, sample counts
+# around the 256 samples of a pair tile and around the pairs of the device.
+# Bound as above.
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("N,L", [(2, 1), (31, 255), (33, 257), (64, 256), (65, 130), (97, 3000), (130, 20000), (257, 513),
+                                 (300, 700)])
+def test_forward_shapes(sp, N, L, prec):
+    g = synth.rng(N + L)
+    kx, ky = synth.uniform_k(L, g)
+    f = c64(synth.complex_normal((N, N), g))
+    with sp.Plan(N, L, 0, prec, _stream(), kx, ky) as p:
+        y = empty_c64((L,))
+        sp.spirec_forward_dev(p.h, to_dev(f), y)
+        sp.spirec_sync(p.h)
+        assert rel(from_dev(y), O.forward(kx, ky, f)) < 1e-5
