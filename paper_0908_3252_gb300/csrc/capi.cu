@@ -728,9 +728,7 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     // whole 16-byte multiples of a 32-sample chunk by TMA bulk copy
     TRY(dalloc(p, &p->kxq, (size_t)L + 32));
     TRY(dalloc(p, &p->kyq, (size_t)L + 32));
-    if (precision != SPIREC_FP32) {
-        TRY(dalloc(p, &p->wpair, (size_t)L + 32));
-    }
+    TRY(dalloc(p, &p->wpair, (size_t)L + 32));
     TRY(dalloc(p, &p->kstage, 2 * (size_t)L));
     TRY(dalloc(p, &p->dflag, 1));
     TRY(dalloc(p, &p->G, (size_t)N * (2 * N - 1)));
@@ -754,7 +752,8 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRY(dalloc(p, &p->scal, (size_t)S_NSCAL));
     TRY(dalloc(p, &p->counters, (size_t)C_N));
     {
-        size_t a = 8 * (size_t)N * (2 * N - 1) * 2;  // floats: 8 splits of G
+        size_t a = kpart_floats_simt(N, L);           // slices of G, FP32
+        if (precision != SPIREC_FP32) a = 0;
         size_t b = 4 * (size_t)L * 2;                 // forward row-block partials
         size_t c = kpart_floats_tc(N, L, precision);
         size_t n = a > b ? a : b;
@@ -767,7 +766,7 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     // zero, so a contraction chunk that runs past L gets zero weights
     TRYCUDA(cudaMemsetAsync(p->s, 0, sizeof(float2) * ((size_t)L + 32), p->stream));
     TRYCUDA(cudaMemsetAsync(p->ystage, 0, sizeof(float2) * ((size_t)L + 32), p->stream));
-    if (p->wpair) TRYCUDA(cudaMemsetAsync(p->wpair, 0, sizeof(float2) * ((size_t)L + 32), p->stream));
+    TRYCUDA(cudaMemsetAsync(p->wpair, 0, sizeof(float2) * ((size_t)L + 32), p->stream));
     TRYCUDA(cudaMemsetAsync(p->scal, 0, S_NSCAL * sizeof(double), p->stream));
     TRYCUDA(cudaMemsetAsync(p->dbuf[0], 0, NN * sizeof(float2), p->stream));
     TRYCUDA(cudaMemsetAsync(p->dbuf[1], 0, NN * sizeof(float2), p->stream));
@@ -796,6 +795,7 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
         if (!once || !attrs_set[p->device].load(std::memory_order_acquire)) {
             TRY(fft_setup_attributes(M));
             TRY(tc_setup_attributes());
+            TRY(simt_setup_attributes());
             if (once) attrs_set[p->device].store(true, std::memory_order_release);
         }
     }

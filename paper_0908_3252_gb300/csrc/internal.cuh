@@ -122,8 +122,8 @@ struct spirec_plan_s {
     // trajectory, fixed point: k * 2^64 mod 2^64
     int64_t* kxq;
     int64_t* kyq;
-    // the weights of a paired tensor-core contraction (mixed precisions; 32
-    // zero entries of padding): w_l times the phase of the pairing's centre
+    // the weights of a paired contraction (32 zero entries of padding): w_l
+    // times the phase of the pairing's centre
     float2* wpair;
     double* kstage;  // 2L: host trajectory staged on the device
     int* dflag;  // device error flag
@@ -233,6 +233,41 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev);
 // shared-memory caches.  The iterate ends in f[0].
 bool loop_supported(int M);
 int launch_cg_loop(spirec_plan p, int iters);
+
+// Pairing of the output columns.  The B operand is a pure phase,
+// E(l, j) = exp(sb i2pi kb_l (j + half/2)), and its conjugate is the phase of
+// the mirrored column, so one set of four real products
+//      P_ac = Ar Br^T   P_bd = Ai Bi^T   P_ad = Ar Bi^T   P_bc = Ai Br^T
+// (A' = Ar + i Ai, E = Br + i Bi, summed over the samples) gives two output
+// columns:
+//      sum A' E       = (P_ac - P_bd) + i (P_ad + P_bc)   at column c+(j)
+//      sum A' conj(E) = (P_ac + P_bd) + i (P_bc - P_ad)   at column c-(j)
+// with c+-(j) = (C2 +- (2j + half)) / 2.  The weight of the original B operand
+// and the phase of the centre column move into A (A' = w' A,
+// w'_l = w_l exp(sb i2pi kb_l (C2 / 2 + ob)), launch_pair_weights).
+//   G (Eq. AnnMatG): columns v + N - 1, centre v = 0 (C2 = 2N - 2, half 0),
+//     j = 0 .. N - 1: the lags v and -v, unweighted.
+//   D (Eq. AnnMatGD): columns m, centre (N - 1) / 2 (C2 = N - 1); for even N
+//     the offsets are half-integers (half 1, j = 0 .. N/2 - 1: m = N/2 + j
+//     and N/2 - 1 - j), for odd N integers (half 0, j = 0 .. (N - 1)/2).
+// A half-integer phase k (j + 1/2) is k j + k/2: the fixed-point k times j
+// plus k shifted right by one bit (an error of 2^-65 cycles, and one unit of
+// 2^-32 cycle from adding the two top words without the low words' carry).
+struct PairGeom {
+    int R, C;   // output rows and columns
+    int C2;     // twice the centre column
+    int half;   // offsets j + 1/2
+    int J;      // B columns j = 0 .. J - 1
+};
+
+PairGeom pair_geom(const spirec_plan_s* p, int knob);
+// p->wpair = w' (see PairGeom): w_l exp(sb i2pi (kb_l / 2) shift2) for l < L, its
+// padding past L left at zero; with amax2 also max_l |w'_l|^2 as float bits.
+int launch_pair_weights(spirec_plan p, const float2* w, const int64_t* kb, int sb, int shift2, unsigned* amax2);
+
+// FP32 contractions (nudft_simt.cu)
+size_t kpart_floats_simt(int N, int64_t L);
+int simt_setup_attributes();
 
 // tensor-core contractions (FP16x3 / BF16x3)
 int launch_gram_tc(spirec_plan p);

@@ -487,32 +487,6 @@ __device__ __forceinline__ float weight_scale_inv(const unsigned* amax2_bits)
     return ldexpf(1.f, -e);
 }
 
-// Pairing of the output columns.  The B operand is a pure phase,
-// E(l, j) = exp(sb i2pi kb_l (j + half/2)), and its conjugate is the phase of
-// the mirrored column, so one set of four real products
-//      P_ac = Ar Br^T   P_bd = Ai Bi^T   P_ad = Ar Bi^T   P_bc = Ai Br^T
-// (A' = Ar + i Ai, E = Br + i Bi, summed over the samples) gives two output
-// columns:
-//      sum A' E       = (P_ac - P_bd) + i (P_ad + P_bc)   at column c+(j)
-//      sum A' conj(E) = (P_ac + P_bd) + i (P_bc - P_ad)   at column c-(j)
-// with c+-(j) = (C2 +- (2j + half)) / 2.  The weight of the original B operand
-// and the phase of the centre column move into A (A' = w' A,
-// w'_l = w_l exp(sb i2pi kb_l (C2 / 2 + ob)), k_pair_weights).
-//   G (Eq. AnnMatG): columns v + N - 1, centre v = 0 (C2 = 2N - 2, half 0),
-//     j = 0 .. N - 1: the lags v and -v, unweighted.
-//   D (Eq. AnnMatGD): columns m, centre (N - 1) / 2 (C2 = N - 1); for even N
-//     the offsets are half-integers (half 1, j = 0 .. N/2 - 1: m = N/2 + j
-//     and N/2 - 1 - j), for odd N integers (half 0, j = 0 .. (N - 1)/2).
-// A half-integer phase k (j + 1/2) is k j + k/2: the fixed-point k times j
-// plus k shifted right by one bit (an error of 2^-65 cycles, and one unit of
-// 2^-32 cycle from adding the two top words without the low words' carry).
-struct PairGeom {
-    int R, C;   // output rows and columns
-    int C2;     // twice the centre column
-    int half;   // offsets j + 1/2
-    int J;      // B columns j = 0 .. J - 1
-};
-
 // Adds (first: stores) this CTA's 128 rows of the four products as the two
 // paired outputs into its partial tile.  B column j (0..127) of the tile is
 // row j % BCOLS (Br) and BCOLS + j % BCOLS (Bi) of the stacked operand of
@@ -1096,7 +1070,8 @@ __global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* __rest
 // w'_l = w_l exp(sb i2pi (kb_l / 2) shift2) for l < L (the weight of the
 // original B operand and the phase of the pairing's centre column, shift2 =
 // C2 + 2 ob); the plan's buffer keeps its zero padding past L.  amax2 (zeroed
-// before the launch) receives max_l |w'_l|^2 as float bits, as k_absmax2.
+// before the launch; may be null) receives max_l |w'_l|^2 as float bits, as
+// k_absmax2.
 __global__ void k_pair_weights(const float2* __restrict__ w, const int64_t* __restrict__ kb, int64_t L, int sb,
                                int shift2, float2* __restrict__ wp, unsigned* amax2)
 {
@@ -1110,7 +1085,7 @@ __global__ void k_pair_weights(const float2* __restrict__ w, const int64_t* __re
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0 && isfinite(mx)) atomicMax(amax2, __float_as_uint(mx));
+    if (amax2 && (threadIdx.x & 31) == 0 && isfinite(mx)) atomicMax(amax2, __float_as_uint(mx));
 }
 
 // ------------------------------------------------------------ forward H f
@@ -1535,27 +1510,6 @@ __global__ void k_absmax2(const float2* __restrict__ y, int64_t n, unsigned* ama
     if ((threadIdx.x & 31) == 0 && isfinite(m)) atomicMax(amax2, __float_as_uint(m));
 }
 
-// The pairing geometry of G (knob SPIREC_KNOB_GRAM_SPLIT) or of D and every
-// other H^H y (SPIREC_KNOB_ADJOINT_SPLIT): see PairGeom.
-PairGeom pair_geom(const spirec_plan_s* p, int knob)
-{
-    const int N = p->N;
-    PairGeom g{};
-    g.R = N;
-    if (knob == SPIREC_KNOB_GRAM_SPLIT) {
-        g.C = 2 * N - 1;
-        g.C2 = 2 * N - 2;
-        g.half = 0;
-        g.J = N;
-    } else {
-        g.C = N;
-        g.C2 = N - 1;
-        g.half = (N % 2 == 0) ? 1 : 0;
-        g.J = g.half ? N / 2 : (N + 1) / 2;
-    }
-    return g;
-}
-
 // Clusters of two k_tc_pair_gemm CTAs the device runs at once (cached per
 // device): the pairs a launch may spread its work over.
 int pair_clusters(int* out)
@@ -1689,16 +1643,9 @@ int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, 
         return SPIREC_EUNSUPPORTED;
     }
     if (w) {
-        // w' = w exp(sb i2pi kb shift2 / 2) into the plan's padded buffer
-        // (its padding past L stays zero), and max |w'|^2 for the scaling
-        int blocks = (int)((p->L + 255) / 256);
-        if (blocks > 4 * kMaxCtas) blocks = 4 * kMaxCtas;
         amax = p->counters + C_AMAX;
-        SPIREC_CK(cudaMemsetAsync(amax, 0, sizeof(unsigned), p->stream));
-        k_pair_weights<<<blocks, 256, 0, p->stream>>>(w, kb, p->L, sb, shift2, p->wpair, amax);
-        SPIREC_CK(cudaGetLastError());
+        if ((rc = launch_pair_weights(p, w, kb, sb, shift2, amax)) != SPIREC_OK) return rc;
         w = p->wpair;
-        p->launches += 1;
     }
     float* part = p->kpart;
     const bool bf16 = p->precision == SPIREC_MIXED_BF16X3;
@@ -1717,6 +1664,38 @@ int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, 
 }
 
 }  // namespace
+
+// The pairing geometry of G (knob SPIREC_KNOB_GRAM_SPLIT) or of D and every
+// other H^H y (SPIREC_KNOB_ADJOINT_SPLIT): see PairGeom.
+PairGeom pair_geom(const spirec_plan_s* p, int knob)
+{
+    const int N = p->N;
+    PairGeom g{};
+    g.R = N;
+    if (knob == SPIREC_KNOB_GRAM_SPLIT) {
+        g.C = 2 * N - 1;
+        g.C2 = 2 * N - 2;
+        g.half = 0;
+        g.J = N;
+    } else {
+        g.C = N;
+        g.C2 = N - 1;
+        g.half = (N % 2 == 0) ? 1 : 0;
+        g.J = g.half ? N / 2 : (N + 1) / 2;
+    }
+    return g;
+}
+
+int launch_pair_weights(spirec_plan p, const float2* w, const int64_t* kb, int sb, int shift2, unsigned* amax2)
+{
+    int blocks = (int)((p->L + 255) / 256);
+    if (blocks > 4 * kMaxCtas) blocks = 4 * kMaxCtas;
+    if (amax2) SPIREC_CK(cudaMemsetAsync(amax2, 0, sizeof(unsigned), p->stream));
+    k_pair_weights<<<blocks, 256, 0, p->stream>>>(w, kb, p->L, sb, shift2, p->wpair, amax2);
+    SPIREC_CK(cudaGetLastError());
+    p->launches += 1;
+    return SPIREC_OK;
+}
 
 int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
 {

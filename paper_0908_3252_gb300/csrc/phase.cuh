@@ -12,10 +12,11 @@
 namespace spirec {
 
 // exp(+i 2 pi k j) for the fixed-point k.  sincospif(x) gives sin(pi x) and
-// cos(pi x); x = 2 * (phase in cycles), in [-1, 1).
-__device__ __forceinline__ float2 phasor_q(int64_t kq, int j)
+// cos(pi x); x = 2 * (phase in cycles), in [-1, 1).  `add` is a fixed-point
+// phase added to k j.
+__device__ __forceinline__ float2 phasor_q(int64_t kq, int j, int64_t add = 0)
 {
-    const uint64_t th = (uint64_t)kq * (uint64_t)(int64_t)j;
+    const uint64_t th = (uint64_t)kq * (uint64_t)(int64_t)j + (uint64_t)add;
     const int hi = (int)(th >> 32);
     const float x = (float)hi * 0x1p-31f;
     float sn, cs;

@@ -99,7 +99,7 @@ size_t plan_bytes(int N, int64_t L, int M, int precision)
     const size_t NN = (size_t)N * N;
     size_t b = 0;
     b += 2 * ((size_t)L + 32) * 8;              // fixed-point trajectory
-    if (precision != SPIREC_FP32) b += ((size_t)L + 32) * 8;  // the paired contractions' weights
+    b += ((size_t)L + 32) * 8;                   // the paired contractions' weights
     b += 2 * (size_t)L * 8;                      // staging
     b += (size_t)N * (2 * N - 1) * 8;            // G
     b += (size_t)M * M * 4 + (size_t)M * M * 8;  // spectrum + work
@@ -108,7 +108,7 @@ size_t plan_bytes(int N, int64_t L, int M, int precision)
     b += 10 * NN * 8;                            // iterates, directions, gradients, D, scratch
     b += (size_t)M * 8 + (size_t)P_NSLOTS * kMaxParts * 8 + 4096;
     b += fsplit_bytes_tc(N, precision);  // split image of the tensor-core forward
-    size_t a = 8 * (size_t)N * (2 * N - 1) * 2, c = 4 * (size_t)L * 2, t = kpart_floats_tc(N, L, precision);
+    size_t a = precision == SPIREC_FP32 ? kpart_floats_simt(N, L) : 0, c = 4 * (size_t)L * 2, t = kpart_floats_tc(N, L, precision);
     b += std::max(std::max(a, c), t) * 4;        // split-K partials
     return b;
 }

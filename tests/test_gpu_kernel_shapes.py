@@ -72,3 +72,29 @@ def test_forward_shapes(sp, N, L, prec):
         sp.spirec_forward_dev(p.h, to_dev(f), y)
         sp.spirec_sync(p.h)
         assert rel(from_dev(y), O.forward(kx, ky, f)) < 1e-5
+
+
+# The FP32 contractions: blocks of 64 and of 128 rows, one to three row and
+# column blocks, ragged chunks of 32 samples, one slice, a few, and more than
+# there are chunks.  FP32 sums of at most 2500 terms: below 1e-5.
+@pytest.mark.parametrize("slices", [0, 1, 3, 100])
+@pytest.mark.parametrize("N,L", [(2, 1), (33, 31), (64, 33), (65, 2500), (129, 64), (130, 1000), (200, 500)])
+def test_fp32_contraction_shapes(sp, N, L, slices):
+    g = synth.rng(N + L)
+    kx, ky = synth.uniform_k(L, g)
+    y = c64(synth.complex_normal(L, g))
+    sp.spirec_tune_clear()
+    p = sp.Plan(N, L, 0, 0, _stream())
+    try:
+        for knob in (sp.SPIREC_KNOB_GRAM_SPLIT, sp.SPIREC_KNOB_ADJOINT_SPLIT):
+            sp.spirec_tune_set(knob, N, p.M, 0, L, slices)
+        sp.spirec_set_trajectory(p.h, kx, ky)
+        G, x = empty_c64((N, 2 * N - 1)), empty_c64((N, N))
+        sp.spirec_gram_dev(p.h, G)
+        sp.spirec_adjoint_dev(p.h, to_dev(y), x)
+        sp.spirec_sync(p.h)
+        assert rel(from_dev(G), O.gram(kx, ky, N)[:, N - 1:].T) < 1e-5
+        assert rel(from_dev(x), O.adjoint(kx, ky, y, N)) < 1e-5
+    finally:
+        p.close()
+        sp.spirec_tune_clear()
