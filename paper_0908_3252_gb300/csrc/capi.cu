@@ -117,20 +117,24 @@ __global__ void k_sum_cached(const float* __restrict__ src, int64_t stride, Cach
     }
 }
 
+// The plan's stream after the caller's stream, and the caller's stream after
+// the plan's.
+void join_in(spirec_plan p)
+{
+    cudaEventRecord(p->ev_join, p->user_stream);
+    cudaStreamWaitEvent(p->stream, p->ev_join, 0);
+}
+void join_out(spirec_plan p)
+{
+    cudaEventRecord(p->ev_join, p->stream);
+    cudaStreamWaitEvent(p->user_stream, p->ev_join, 0);
+}
+
+// Both, on entry and on exit of a call.
 struct Join {
-    // Orders the plan's stream after the caller's stream on entry, and the
-    // caller's stream after the plan's stream on exit.
     spirec_plan p;
-    explicit Join(spirec_plan pp) : p(pp)
-    {
-        cudaEventRecord(p->ev_join, p->user_stream);
-        cudaStreamWaitEvent(p->stream, p->ev_join, 0);
-    }
-    ~Join()
-    {
-        cudaEventRecord(p->ev_join, p->stream);
-        cudaStreamWaitEvent(p->user_stream, p->ev_join, 0);
-    }
+    explicit Join(spirec_plan pp) : p(pp) { join_in(p); }
+    ~Join() { join_out(p); }
 };
 
 // Plan buffers come from the device's stream-ordered pool (cudaMallocAsync on
@@ -1163,15 +1167,11 @@ int spirec_solve(spirec_plan p, const float* x0, int32_t iters, float* x_out, do
     return SPIREC_OK;
 }
 
-int spirec_solve_dev(spirec_plan p, const float* x0, int32_t iters, float* x_out, double* J_hist)
+// The device solve's work on the plan's stream, joined to the caller's by the
+// caller.
+static int solve_dev_enqueue(spirec_plan p, const float* x0, int32_t iters, float* x_out, double* J_hist)
 {
-    int rc = check_plan(p);
-    if (rc) return rc;
-    if (!x_out) {
-        set_error("x_out must not be NULL");
-        return SPIREC_EINVAL;
-    }
-    Join j(p);
+    int rc;
     if ((rc = solve_core(p, x0, true, iters)) != SPIREC_OK) return rc;
     const size_t img = (size_t)p->N * p->N * sizeof(float2);
     SPIREC_CK(cudaMemcpyAsync(x_out, p->f[p->result_slot], img, cudaMemcpyDeviceToDevice, p->stream));
@@ -1179,6 +1179,92 @@ int spirec_solve_dev(spirec_plan p, const float* x0, int32_t iters, float* x_out
         SPIREC_CK(cudaMemcpyAsync(J_hist, p->Jdev, sizeof(double) * (iters + 1), cudaMemcpyDeviceToDevice,
                                   p->stream));
     return SPIREC_OK;
+}
+
+static int check_solve_dev(spirec_plan p, const float* x_out)
+{
+    const int rc = check_plan(p);
+    if (rc) return rc;
+    if (!x_out) {
+        set_error("x_out must not be NULL");
+        return SPIREC_EINVAL;
+    }
+    return SPIREC_OK;
+}
+
+int spirec_solve_dev(spirec_plan p, const float* x0, int32_t iters, float* x_out, double* J_hist)
+{
+    const int rc = check_solve_dev(p, x_out);
+    if (rc) return rc;
+    Join j(p);
+    return solve_dev_enqueue(p, x0, iters, x_out, J_hist);
+}
+
+// Whether a solve of the batch writes an array that another one reads or
+// writes.
+static bool batch_arrays_overlap(const spirec_plan* plans, int n, const float* const* x0, int iters,
+                                 float* const* x_out, double* const* J_hist)
+{
+    struct Range {
+        uintptr_t a, b;
+        bool write;
+        int plan;
+    };
+    std::vector<Range> v;
+    auto add = [&](const void* q, size_t bytes, bool write, int i) {
+        if (q) v.push_back(Range{(uintptr_t)q, (uintptr_t)q + bytes, write, i});
+    };
+    for (int i = 0; i < n; ++i) {
+        if (!plans[i]) continue;
+        const size_t img = (size_t)plans[i]->N * plans[i]->N * sizeof(float2);
+        add(x0 ? x0[i] : nullptr, img, false, i);
+        add(x_out[i], img, true, i);
+        add(J_hist ? J_hist[i] : nullptr, sizeof(double) * ((size_t)std::max(iters, 0) + 1), true, i);
+    }
+    std::sort(v.begin(), v.end(), [](const Range& p, const Range& q) { return p.a < q.a; });
+    for (size_t i = 0; i < v.size(); ++i)
+        for (size_t j = i + 1; j < v.size() && v[j].a < v[i].b; ++j)
+            if (v[i].plan != v[j].plan && (v[i].write || v[j].write)) return true;
+    return false;
+}
+
+int spirec_batch_solve(const spirec_plan* plans, int32_t n, const float* const* x0, int32_t iters,
+                       float* const* x_out, double* const* J_hist)
+{
+    if (!plans || n < 0 || !x_out) {
+        set_error("bad batch arguments");
+        return SPIREC_EINVAL;
+    }
+    // Every plan's stream joins its caller's stream before the first solve is
+    // enqueued and is joined back after the last: plans that share a caller's
+    // stream would otherwise wait for each other, one solve after the next (12
+    // frames of 128^2 to 256^2 on one stream, four iterations: 2.73 -> 1.63 ms
+    // with their set-up).  Solves whose arrays overlap (one starting from
+    // another's result) keep that order.
+    // A plan that cannot be solved ends the batch there; the solves before it
+    // are enqueued.
+    const bool ordered = batch_arrays_overlap(plans, n, x0, iters, x_out, J_hist);
+    int rc = SPIREC_OK, m = 0;
+    for (; m < n && (rc = check_solve_dev(plans[m], x_out[m])) == SPIREC_OK; ++m)
+        if (!ordered) join_in(plans[m]);
+    int done = 0;
+    for (int r = SPIREC_OK; done < m; ++done) {
+        if (ordered) join_in(plans[done]);
+        r = solve_dev_enqueue(plans[done], x0 ? x0[done] : nullptr, iters, x_out[done], J_hist ? J_hist[done] : nullptr);
+        if (ordered) join_out(plans[done]);
+        if (r != SPIREC_OK) {
+            rc = r;
+            break;
+        }
+    }
+    for (int i = 0; i < m && !ordered; ++i) join_out(plans[i]);
+    if (rc != SPIREC_OK) return rc;
+    int first = SPIREC_OK;
+    for (int i = 0; i < n; ++i) {
+        rc = spirec_sync(plans[i]);
+        if (rc != SPIREC_OK && first == SPIREC_OK) first = rc;
+    }
+    return first;
 }
 
 int spirec_forward_dev(spirec_plan p, const float* x, float* y)

@@ -1,5 +1,5 @@
 // server.cu -- request loop for many reconstructions on one GPU (continuous
-// batching), and the batched solve.
+// batching).
 //
 // A server owns `max_slots` worker threads.  Each worker keeps one plan (its
 // own CUDA stream, trajectory tables, iterate and scratch resident on the
@@ -422,26 +422,6 @@ int spirec_server_destroy(spirec_server srv)
     for (auto& t : srv->workers) t.join();
     delete srv;
     return SPIREC_OK;
-}
-
-int spirec_batch_solve(const spirec_plan* plans, int32_t n, const float* const* x0, int32_t iters,
-                       float* const* x_out, double* const* J_hist)
-{
-    if (!plans || n < 0 || !x_out) {
-        set_error("bad batch arguments");
-        return SPIREC_EINVAL;
-    }
-    // enqueue every solve on its own plan's stream, then wait for all
-    for (int i = 0; i < n; ++i) {
-        const int rc = spirec_solve_dev(plans[i], x0 ? x0[i] : nullptr, iters, x_out[i], J_hist ? J_hist[i] : nullptr);
-        if (rc != SPIREC_OK) return rc;
-    }
-    int first = SPIREC_OK;
-    for (int i = 0; i < n; ++i) {
-        const int rc = spirec_sync(plans[i]);
-        if (rc != SPIREC_OK && first == SPIREC_OK) first = rc;
-    }
-    return first;
 }
 
 }  // extern "C"
