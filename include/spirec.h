@@ -89,7 +89,10 @@ typedef enum {
  *              M >= 2N-1 (M = 2N for the usual sizes).  M must be >= 2N-1 and
  *              factor into 2, 3 and 5.  Sections 3.4 and Appendix B: the
  *              convolution by conj(G) is linear, so the FFT grid must hold the
- *              (2N-1)^2 lags without wrap-around.
+ *              (2N-1)^2 lags without wrap-around.  M is the grid of
+ *              spirec_kernel_spectrum_dev; the plan's own transforms run on M
+ *              when it is a power of two (16 to 4096), else on the next power
+ *              of two that holds the lags (the same convolution).
  *   precision  spirec_precision.
  *   stream     cudaStream_t the plan orders its work after and before (NULL:
  *              the legacy default stream).  Internally the plan works on its

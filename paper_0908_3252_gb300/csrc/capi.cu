@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <atomic>
 #include <map>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -17,11 +18,11 @@
 
 // the per-interleave kernel cache (spirec_kcache_*)
 struct spirec_kcache_s {
-    int N = 0, M = 0, precision = 0, n = 0, device = 0;
+    int N = 0, M = 0, MF = 0, precision = 0, n = 0, device = 0;
     std::vector<int64_t> off;  // n + 1 sample offsets
     int64_t* kxq = nullptr;    // all samples, fixed point (device)
     int64_t* kyq = nullptr;
-    float* spec = nullptr;     // n x M x M kernel spectra
+    float* spec = nullptr;     // n x MF x MF kernel spectra
     float2* G = nullptr;       // n x N x (2N-1) halves of G
 };
 
@@ -78,17 +79,6 @@ __global__ void k_traj_fixed(const double* __restrict__ kx, const double* __rest
             if (c == 0) kxq[l] = q;
             else kyq[l] = q;
         }
-    }
-}
-
-// out[ky*M + kx] = Chat[kx*M + ky]
-__global__ void k_transpose_real(const float* __restrict__ in, int M, float* __restrict__ out)
-{
-    const int64_t MM = (int64_t)M * M;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < MM;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t ky = e / M, kx = e % M;
-        out[e] = in[kx * M + ky];
     }
 }
 
@@ -198,7 +188,7 @@ void free_plan(spirec_plan p)
 {
     if (!p) return;
     void* bufs[] = {p->kxq, p->kyq, p->dflag, p->G, p->Chat, p->cwork, p->X, p->D, p->s, p->fsplit, p->ydir,
-                    p->f[0], p->f[1], p->dbuf[0], p->dbuf[1], p->g, p->res, p->Td, p->tmp, p->twiddle,
+                    p->f[0], p->f[1], p->dbuf[0], p->dbuf[1], p->g, p->res, p->Td, p->tmp, p->twiddle, p->twiddle_M,
                     p->part, p->scal, p->counters, p->Jdev, p->kpart, p->kstage, p->ystage, p->hqw,
                     p->wpair, p->s_in};
     for (void* b : bufs)
@@ -413,7 +403,7 @@ int run_iterations(spirec_plan p, int iters)
 
 bool solve_uses_loop(spirec_plan p)
 {
-    return p->mode != SPIREC_MODE_DIRECT && p->minimiser == SPIREC_MIN_PRCG && loop_supported(p->M) &&
+    return p->mode != SPIREC_MODE_DIRECT && p->minimiser == SPIREC_MIN_PRCG && loop_supported(p->MF) &&
            !getenv("SPIREC_NO_LOOP");
 }
 
@@ -615,7 +605,7 @@ int tune_tile(spirec_plan p, int split_knob, int objective, int sms, int* chosen
 int tune_loop(spirec_plan p, int objective, int iters, int sms, int* chosen, double* best_ms)
 {
     *chosen = 0;
-    if (p->mode == SPIREC_MODE_DIRECT || p->minimiser != SPIREC_MIN_PRCG || !loop_supported(p->M) ||
+    if (p->mode == SPIREC_MODE_DIRECT || p->minimiser != SPIREC_MIN_PRCG || !loop_supported(p->MF) ||
         getenv("SPIREC_NO_LOOP"))
         return SPIREC_OK;
     int rc;
@@ -699,6 +689,7 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     p->N = N;
     p->L = L;
     p->M = M;
+    p->MF = fft_grid(N, M);
     p->precision = precision;
     p->user_stream = (cudaStream_t)stream;
     int rc = SPIREC_OK;
@@ -707,7 +698,9 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
         delete p;
         return cuda_fail(e, "cudaGetDevice");
     }
-    make_fft_plan(M, &p->fft);
+    const int MF = p->MF;
+    make_fft_plan(MF, &p->fft);
+    make_fft_plan(M, &p->fft_M);
 #define TRY(x)                       \
     do {                             \
         if ((rc = (x)) != SPIREC_OK) { \
@@ -736,9 +729,9 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRY(dalloc(p, &p->kstage, 2 * (size_t)L));
     TRY(dalloc(p, &p->dflag, 1));
     TRY(dalloc(p, &p->G, (size_t)N * (2 * N - 1)));
-    TRY(dalloc(p, &p->Chat, (size_t)M * M));
-    TRY(dalloc(p, &p->cwork, (size_t)M * M));
-    TRY(dalloc(p, &p->X, (size_t)N * M));
+    TRY(dalloc(p, &p->Chat, (size_t)MF * MF));
+    TRY(dalloc(p, &p->cwork, cwork_elems(N, M, MF)));
+    TRY(dalloc(p, &p->X, (size_t)N * MF));
     if ((p->fsplit_bytes = fsplit_bytes_tc(N, precision)) > 0) TRY(dalloc(p, &p->fsplit, p->fsplit_bytes));
     TRY(dalloc(p, &p->D, NN));
     TRY(dalloc(p, &p->s, (size_t)L + 32));
@@ -751,7 +744,8 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRY(dalloc(p, &p->res, NN));
     TRY(dalloc(p, &p->Td, NN));
     TRY(dalloc(p, &p->tmp, NN));
-    TRY(dalloc(p, &p->twiddle, (size_t)M));
+    TRY(dalloc(p, &p->twiddle, (size_t)MF));
+    if (M != MF) TRY(dalloc(p, &p->twiddle_M, (size_t)M));
     TRY(dalloc(p, &p->part, (size_t)P_NSLOTS * kMaxParts));
     TRY(dalloc(p, &p->scal, (size_t)S_NSCAL));
     TRY(dalloc(p, &p->counters, (size_t)C_N));
@@ -776,19 +770,24 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRYCUDA(cudaMemsetAsync(p->dbuf[1], 0, NN * sizeof(float2), p->stream));
     TRYCUDA(cudaMemsetAsync(p->g, 0, NN * sizeof(float2), p->stream));
     {
-        float2* tw = (float2*)malloc(sizeof(float2) * M);
+        std::unique_ptr<float2[]> tw(new (std::nothrow) float2[(size_t)MF + M]);
         if (!tw) {
             free_plan(p);
             set_error("host allocation failed");
             return SPIREC_ENOMEM;
         }
-        for (int k = 0; k < M; ++k) {
-            const double a = -2.0 * M_PI * (double)k / (double)M;
-            tw[k] = make_float2((float)cos(a), (float)sin(a));
-        }
-        e = cudaMemcpyAsync(p->twiddle, tw, sizeof(float2) * M, cudaMemcpyHostToDevice, p->stream);
+        auto table = [](int m, float2* t) {
+            for (int k = 0; k < m; ++k) {
+                const double a = -2.0 * M_PI * (double)k / (double)m;
+                t[k] = make_float2((float)cos(a), (float)sin(a));
+            }
+        };
+        table(MF, tw.get());
+        if (M != MF) table(M, tw.get() + MF);
+        e = cudaMemcpyAsync(p->twiddle, tw.get(), sizeof(float2) * MF, cudaMemcpyHostToDevice, p->stream);
+        if (e == cudaSuccess && M != MF)
+            e = cudaMemcpyAsync(p->twiddle_M, tw.get() + MF, sizeof(float2) * M, cudaMemcpyHostToDevice, p->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-        free(tw);
         TRYCUDA(e);
     }
     {
@@ -880,8 +879,9 @@ int spirec_kcache_create(spirec_kcache* out, int32_t N, int32_t M, int32_t preci
             if (i == 0) {
                 c->N = h->N;
                 c->M = h->M;
+                c->MF = h->MF;
                 c->precision = h->precision;
-                const size_t MM = (size_t)c->M * c->M, NG = (size_t)c->N * (2 * c->N - 1);
+                const size_t MM = (size_t)c->MF * c->MF, NG = (size_t)c->N * (2 * c->N - 1);
                 if ((e = cudaMalloc((void**)&c->kxq, sizeof(int64_t) * (size_t)(Ltot + 32))) != cudaSuccess ||
                     (e = cudaMalloc((void**)&c->kyq, sizeof(int64_t) * (size_t)(Ltot + 32))) != cudaSuccess ||
                     (e = cudaMalloc((void**)&c->spec, sizeof(float) * MM * n)) != cudaSuccess ||
@@ -894,7 +894,7 @@ int spirec_kcache_create(spirec_kcache* out, int32_t N, int32_t M, int32_t preci
             h = it->second;
         }
         if ((rc = spirec_set_trajectory(h, kx + offsets[i], ky + offsets[i])) != SPIREC_OK) return fail(rc);
-        const size_t MM = (size_t)c->M * c->M, NG = (size_t)c->N * (2 * c->N - 1);
+        const size_t MM = (size_t)c->MF * c->MF, NG = (size_t)c->N * (2 * c->N - 1);
         const cudaMemcpyKind d2d = cudaMemcpyDeviceToDevice;
         if ((e = cudaMemcpyAsync(c->kxq + offsets[i], h->kxq, sizeof(int64_t) * Li, d2d, h->stream)) != cudaSuccess ||
             (e = cudaMemcpyAsync(c->kyq + offsets[i], h->kyq, sizeof(int64_t) * Li, d2d, h->stream)) != cudaSuccess ||
@@ -955,7 +955,7 @@ int spirec_set_trajectory_cached(spirec_plan p, spirec_kcache c, const int32_t* 
         SPIREC_CK(cudaMemcpyAsync(p->kyq + pos, c->kyq + o, sizeof(int64_t) * Li, cudaMemcpyDeviceToDevice, p->stream));
         pos += Li;
     }
-    const int64_t MM = (int64_t)p->M * p->M, NG2 = 2 * (int64_t)p->N * (2 * p->N - 1);
+    const int64_t MM = (int64_t)p->MF * p->MF, NG2 = 2 * (int64_t)p->N * (2 * p->N - 1);
     int blocks = (int)((MM + 255) / 256);
     if (blocks > 8 * 152) blocks = 8 * 152;
     k_sum_cached<<<blocks, 256, 0, p->stream>>>(c->spec, MM, t, p->Chat);
@@ -1207,24 +1207,22 @@ static bool batch_arrays_overlap(const spirec_plan* plans, int n, const float* c
 {
     struct Range {
         uintptr_t a, b;
-        bool write;
-        int plan;
     };
-    std::vector<Range> v;
-    auto add = [&](const void* q, size_t bytes, bool write, int i) {
-        if (q) v.push_back(Range{(uintptr_t)q, (uintptr_t)q + bytes, write, i});
-    };
-    for (int i = 0; i < n; ++i) {
-        if (!plans[i]) continue;
-        const size_t img = (size_t)plans[i]->N * plans[i]->N * sizeof(float2);
-        add(x0 ? x0[i] : nullptr, img, false, i);
-        add(x_out[i], img, true, i);
-        add(J_hist ? J_hist[i] : nullptr, sizeof(double) * ((size_t)std::max(iters, 0) + 1), true, i);
-    }
-    std::sort(v.begin(), v.end(), [](const Range& p, const Range& q) { return p.a < q.a; });
-    for (size_t i = 0; i < v.size(); ++i)
-        for (size_t j = i + 1; j < v.size() && v[j].a < v[i].b; ++j)
-            if (v[i].plan != v[j].plan && (v[i].write || v[j].write)) return true;
+    auto range = [](const void* q, size_t bytes) { return Range{(uintptr_t)q, q ? (uintptr_t)q + bytes : 0}; };
+    auto image = [&](int i) { return (size_t)plans[i]->N * plans[i]->N * sizeof(float2); };
+    const size_t jb = sizeof(double) * ((size_t)std::max(iters, 0) + 1);
+    auto meet = [](Range u, Range v) { return u.a < v.b && v.a < u.b; };
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) {
+            if (i == j || !plans[i] || !plans[j]) continue;
+            // what i writes against what j touches
+            const Range w[2] = {range(x_out[i], image(i)), range(J_hist ? J_hist[i] : nullptr, jb)};
+            const Range t[3] = {range(x_out[j], image(j)), range(J_hist ? J_hist[j] : nullptr, jb),
+                                range(x0 ? x0[j] : nullptr, image(j))};
+            for (const Range& u : w)
+                for (const Range& v : t)
+                    if (meet(u, v)) return true;
+        }
     return false;
 }
 
@@ -1330,10 +1328,7 @@ int spirec_kernel_spectrum_dev(spirec_plan p, float* C)
         return SPIREC_ESTATE;
     }
     Join j(p);
-    k_transpose_real<<<4 * 152, 256, 0, p->stream>>>(p->Chat, p->M, C);
-    SPIREC_CK(cudaGetLastError());
-    p->launches += 1;
-    return SPIREC_OK;
+    return launch_spectrum_out(p, C);
 }
 
 int spirec_data_adjoint_dev(spirec_plan p, float* D)

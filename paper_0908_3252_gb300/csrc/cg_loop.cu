@@ -1216,14 +1216,14 @@ struct LaunchLoop {
     int operator()()
     {
         if constexpr (MC == 0) {
-            set_error("no compile-time FFT size for M=%d", p->M);
+            set_error("no compile-time FFT size for M=%d", p->MF);
             return SPIREC_EUNSUPPORTED;
         } else {
             int RB = 0, grid = 0;
             size_t smem = 0;
             if (!loop_shape<MC>(p, &RB, &grid, &smem)) {
                 cudaGetLastError();
-                set_error("the persistent loop does not fit N=%d, M=%d", p->N, p->M);
+                set_error("the persistent loop does not fit N=%d, M=%d", p->N, p->MF);
                 return SPIREC_EUNSUPPORTED;
             }
             LoopArgs A{};
@@ -1307,7 +1307,7 @@ struct Shapes {
 int shapes_for(const spirec_plan_s* p, int* RB, int* grid, int max, bool current, int* capacity = nullptr)
 {
     Shapes s{p, RB, grid, max, current, capacity};
-    switch (p->M) {
+    switch (p->MF) {
     case 64: return s.run<64>();
     case 128: return s.run<128>();
     case 256: return s.run<256>();
@@ -1328,13 +1328,13 @@ int loop_demand(spirec_plan p, int* blocks, int* capacity)
     int RB = 0;
     *blocks = 0;
     *capacity = 0;
-    if (!loop_supported(p->M)) return 0;
+    if (!loop_supported(p->MF)) return 0;
     return shapes_for(p, &RB, blocks, 1, true, capacity);
 }
 
 int launch_cg_loop(spirec_plan p, int iters)
 {
-    switch (p->M) {
+    switch (p->MF) {
     case 64: return LaunchLoop{p, iters}.operator()<64>();
     case 128: return LaunchLoop{p, iters}.operator()<128>();
     case 256: return LaunchLoop{p, iters}.operator()<256>();

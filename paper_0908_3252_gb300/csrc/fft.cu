@@ -17,10 +17,12 @@
 // cg_loop.cu); this file holds the stand-alone kernels and their launchers.
 //
 // FFTs are self-sorting Stockham transforms in shared memory.  For
-// power-of-two M (the sizes the plan picks) the transform is compile-time:
+// power-of-two M (what every plan's transforms run on, fft_grid) the transform
+// is compile-time:
 // one radix-4 butterfly per thread per stage (plus one radix-2 stage for odd
 // log2 M), values in registers between a read and a write phase.  Any other
-// M = 2^a 3^b 5^c runs the runtime mixed-radix path with a ping-pong buffer.
+// M = 2^a 3^b 5^c (a caller's spectrum on such a grid, spirec_toeplitz_noalloc)
+// runs the runtime mixed-radix path with a ping-pong buffer.
 // At M = 2048 and 4096, where every transform of the apply has at most M/2
 // nonzero inputs and keeps at most M/2 outputs, the three passes instead
 // split each transform into S = M / 1024 warp-sized 1024-point DFTs, one per
@@ -529,11 +531,49 @@ k_rows_inv_split(const float2* X, int rows, float2* out, int n_out, const float2
     }
 }
 
-// Column FFTs of the M x M circulant and the real spectrum:
-// Chat[x][ky] = Re(FFT2 c)[ky][x] / M^2.
+// ------------------------------------------------------- kernel spectrum
+//
+// Chat[kx][ky] = (1 / M^2) sum_{u,v} c_{u,v} exp(-i2pi (kx u + ky v) / M) with
+// c_{u,v} = conj G_{u,v}, |u|, |v| < N.  G is point-symmetric, c_{-u,-v} = conj
+// c_{u,v}, so the transforms T[u][ky] along v satisfy T[-u] = conj T[u] and
+//      M^2 Chat[kx][ky] = 2 Re sum_{u = 0}^{N-1} e_u T[u][ky] exp(-i2pi kx u / M),
+// e_0 = 1/2, e_u = 1: N row transforms straight from G's stored half (u >= 0)
+// and column transforms of N inputs, instead of M and M over an embedded
+// M x M array (embedding, rows and columns at M = 1024, N = 512: 34 -> 25 us).
+
+// Rows u of G's half, conjugated, at v mod M: T[u][ky] to X[u * M + ky].
 template <int MC>
-__global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* cwork, FftPlan fp, const float2* __restrict__ tw,
-                                float* Chat, int cpc)
+__global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict__ G, int N, float2* X, FftPlan fp,
+                                                        const float2* __restrict__ tw, int rpc)
+{
+    extern __shared__ float2 sm[];
+    const int M = fp.M, ld = seq_len<MC>(M), W = 2 * N - 1;
+    float2* a = sm;
+    float2* b = sm + rpc * ld;
+    const int u0 = blockIdx.x * rpc, nr = min(rpc, N - u0);
+    for (int e = threadIdx.x; e < rpc * M; e += blockDim.x) {
+        const int q = e / M, y = e - q * M;
+        const int v = y < N ? y : y - M;  // -N < v < N holds a lag
+        float2 c = make_float2(0.f, 0.f);
+        if (q < nr && v > -N) {
+            const float2 g = __ldg(G + (int64_t)(u0 + q) * W + (v + N - 1));
+            c = make_float2(g.x, -g.y);
+        }
+        a[q * ld + sidx<MC>(y)] = c;
+    }
+    __syncthreads();
+    float2* res = fft_block<MC, false>(a, b, fp, rpc, ld, tw);
+    for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
+        const int q = e / M, m = e - q * M;
+        X[(int64_t)(u0 + q) * M + m] = res[q * ld + sidx<MC>(m)];
+    }
+}
+
+// Column transforms of X (rows u < N) and the real spectrum: to
+// out[kx * M + ky] (Chat), or out[ky * M + kx] (ROWS_KY).
+template <int MC, bool ROWS_KY>
+__global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* __restrict__ X, int N, FftPlan fp, const float2* __restrict__ tw,
+                                float* out, int cpc)
 {
     extern __shared__ float2 sm[];
     const int M = fp.M;
@@ -544,51 +584,20 @@ __global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* cwork, Fft
     const int nc = min(cpc, M - x0);
     for (int e = threadIdx.x; e < cpc * M; e += blockDim.x) {
         const int y = e / cpc, cc = e - y * cpc;
-        a[cc * ld + sidx<MC>(y)] = cc < nc ? cwork[(int64_t)y * M + x0 + cc] : make_float2(0.f, 0.f);
+        float2 v = make_float2(0.f, 0.f);
+        if (cc < nc && y < N) {
+            v = X[(int64_t)y * M + x0 + cc];
+            if (y == 0) v = make_float2(0.5f * v.x, 0.5f * v.y);
+        }
+        a[cc * ld + sidx<MC>(y)] = v;
     }
     __syncthreads();
     float2* res = fft_block<MC, false>(a, b, fp, cpc, ld, tw);
-    const float inv = 1.0f / ((float)M * (float)M);
+    const float inv = 2.0f / ((float)M * (float)M);
     for (int e = threadIdx.x; e < nc * M; e += blockDim.x) {
-        const int cc = e / M, ky = e - cc * M;
-        Chat[(int64_t)(x0 + cc) * M + ky] = res[cc * ld + sidx<MC>(ky)].x * inv;
-    }
-}
-
-// c[y][x] = K[v][u] = conj G_{u,v} with v = y (y < N) or y - M (y > M - N),
-// u likewise from x; zero where |u| or |v| >= N.  G holds u >= 0; the rest is
-// G_{u,v} = conj G_{-u,-v}.
-__global__ void __launch_bounds__(256) k_embed(const float2* __restrict__ G, int N, int M, float2* cwork)
-{
-    // one 32 x 32 tile of cwork through shared memory: G is read along its
-    // rows (the lags v of one u) and cwork written along its rows (x)
-    __shared__ float2 tile[32][33];  // [x - x0][y - y0]
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    const int W = 2 * N - 1;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int x = x0 + ty + 8 * k, y = y0 + tx;
-        float2 c = make_float2(0.f, 0.f);
-        if (x < M && y < M) {
-            const int v = y < N ? y : (y > M - N ? y - M : INT32_MIN);
-            const int u = x < N ? x : (x > M - N ? x - M : INT32_MIN);
-            if (v != INT32_MIN && u != INT32_MIN) {
-                if (u >= 0) {
-                    const float2 g = G[(int64_t)u * W + (v + N - 1)];
-                    c = make_float2(g.x, -g.y);
-                } else {
-                    c = G[(int64_t)(-u) * W + (-v + N - 1)];
-                }
-            }
-        }
-        tile[ty + 8 * k][tx] = c;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int x = x0 + tx, y = y0 + ty + 8 * k;
-        if (x < M && y < M) cwork[(int64_t)y * M + x] = tile[tx][ty + 8 * k];
+        const int cc = ROWS_KY ? e / M : e % nc, kx = ROWS_KY ? e - cc * M : e / nc;
+        const float v = res[cc * ld + sidx<MC>(kx)].x * inv;
+        out[ROWS_KY ? (int64_t)(x0 + cc) * M + kx : (int64_t)kx * M + x0 + cc] = v;
     }
 }
 
@@ -624,7 +633,8 @@ Shape col_shape(int M, bool pow2)
         while (cpc > 1 && (size_t)cpc * ld * sizeof(float2) > (size_t)kFftSmemCap) cpc /= 2;
         return Shape{cpc, cpc * nb, (size_t)cpc * ld * sizeof(float2)};
     }
-    int cpc = M >= 1024 ? 4 : (M >= 512 ? 8 : 16);
+    // few columns a block: a small grid has to fill the SMs
+    int cpc = 4;
     while (cpc > 1 && 2 * (size_t)cpc * (M + 4) * sizeof(float2) > (size_t)kFftSmemCap) --cpc;
     return Shape{cpc, 256, 2 * (size_t)cpc * (M + 4) * sizeof(float2)};
 }
@@ -642,7 +652,9 @@ int set_attrs()
     SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     SPIREC_CK(cudaFuncSetAttribute(k_cols_filter<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_cols_spectrum<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_spectrum<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_cols_spectrum<MC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_cols_spectrum<MC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     return SPIREC_OK;
 }
 
@@ -815,25 +827,51 @@ struct LaunchRowsInv {
     }
 };
 
+// The spectrum on the grid of fp from G, by way of the N x M rows in cwork, to
+// out (rows_ky: in the caller's layout).
 struct LaunchSpectrum {
     spirec_plan p;
+    const FftPlan* fp;
+    const float2* tw;
+    bool rows_ky;
+    float* out;
     Shape rs, cs;
     template <int MC>
     int operator()()
     {
-        const int M = p->M;
-        CgPass c{};
-        // rows of the circulant, in place (each block reads its rows fully first)
-        k_rows_fwd<MC, 0><<<(M + rs.per_cta - 1) / rs.per_cta, rs.threads, rs.smem, p->stream>>>(
-            p->cwork, M, M, M, p->cwork, p->fft, p->twiddle, rs.per_cta, c);
+        const int M = fp->M, N = p->N;
+        k_rows_spectrum<MC><<<(N + rs.per_cta - 1) / rs.per_cta, rs.threads, rs.smem, p->stream>>>(
+            p->G, N, p->cwork, *fp, tw, rs.per_cta);
         SPIREC_CK(cudaGetLastError());
-        k_cols_spectrum<MC><<<(M + cs.per_cta - 1) / cs.per_cta, cs.threads, cs.smem, p->stream>>>(
-            p->cwork, p->fft, p->twiddle, p->Chat, cs.per_cta);
+        const int blocks = (M + cs.per_cta - 1) / cs.per_cta;
+        if (rows_ky)
+            k_cols_spectrum<MC, true><<<blocks, cs.threads, cs.smem, p->stream>>>(p->cwork, N, *fp, tw, out, cs.per_cta);
+        else
+            k_cols_spectrum<MC, false><<<blocks, cs.threads, cs.smem, p->stream>>>(p->cwork, N, *fp, tw, out, cs.per_cta);
         SPIREC_CK(cudaGetLastError());
         p->launches += 2;
         return SPIREC_OK;
     }
 };
+
+// out[e'] of the transposed real in[e] (M x M)
+__global__ void __launch_bounds__(256) k_transpose_real(const float* __restrict__ in, int M, float* __restrict__ out)
+{
+    __shared__ float tile[32][33];
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int x = x0 + tx, y = y0 + ty + 8 * k;
+        if (x < M && y < M) tile[ty + 8 * k][tx] = __ldg(in + (int64_t)y * M + x);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int x = x0 + ty + 8 * k, y = y0 + tx;
+        if (x < M && y < M) out[(int64_t)x * M + y] = tile[tx][ty + 8 * k];
+    }
+}
 
 }  // namespace
 
@@ -855,7 +893,7 @@ int fft_setup_attributes(int)
 int launch_rows_fwd(spirec_plan p, const float2* in, int ld_in, int n_in, int rows, int mode,
                     const CgPass* cg)
 {
-    const int M = p->M;
+    const int M = p->MF;
     const Shape s = row_shape(M, is_pow2_specialised(M));
     const int blocks = (rows + s.per_cta - 1) / s.per_cta;
     if (mode == 1 && blocks > kMaxParts) {
@@ -870,7 +908,7 @@ int launch_rows_fwd(spirec_plan p, const float2* in, int ld_in, int n_in, int ro
 
 int launch_cols(spirec_plan p, int n_in, int n_out)
 {
-    const int M = p->M;
+    const int M = p->MF;
     const Shape s = col_shape(M, is_pow2_specialised(M));
     const int blocks = (M + s.per_cta - 1) / s.per_cta;
     return with_size(M, LaunchCols{p, n_in, n_out, blocks, s});
@@ -879,7 +917,7 @@ int launch_cols(spirec_plan p, int n_in, int n_out)
 int launch_rows_inv(spirec_plan p, float2* out, int mode, const float2* dotx, const CgPass* cg,
                     int dot_scalar)
 {
-    const int M = p->M, N = p->N;
+    const int M = p->MF, N = p->N;
     const Shape s = row_shape(M, is_pow2_specialised(M));
     const int blocks = (N + s.per_cta - 1) / s.per_cta;
     if (dotx && blocks > kMaxParts) {
@@ -901,15 +939,52 @@ int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, int dot_scalar)
     return launch_rows_inv(p, Tx, 0, dot_scalar >= 0 ? x : nullptr, nullptr, dot_scalar);
 }
 
+// A power of two as it is; anything else (the 2^a 3^b 5^c grids a plan picks
+// by default among them) is embedded in the next power of two that holds the
+// lags: T is the same linear convolution on any grid of at least 2N - 1, and
+// the power-of-two passes are the faster ones at every N although the grid
+// grows by up to 1.9 times a side.  Measured, M = 2^a 3^b 5^c against the power of two
+// (us): one T apply and one CG iteration
+//   N = 50,   M = 100 / 128      26.5 / 17.8    40 / 23
+//   N = 129,  M = 270 / 512      45.5 / 22.0    63 / 30
+//   N = 384,  M = 768 / 1024     55.3 / 38.0    76 / 30
+//   N = 520,  M = 1080 / 2048    66.4 / 50.3    92 / 89
+//   N = 1030, M = 2160 / 4096   250   / 169    342 / 227
+int fft_grid(int N, int M)
+{
+    if (is_pow2_specialised(M)) return M;
+    int g = 16;
+    while (g < 2 * N - 1) g *= 2;
+    return g;
+}
+
 int launch_spectrum(spirec_plan p)
 {
-    const int N = p->N, M = p->M;
-    k_embed<<<dim3((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32)), dim3(32, 8), 0, p->stream>>>(p->G, N, M,
-                                                                                                   p->cwork);
+    const int M = p->MF;
+    const bool pow2 = is_pow2_specialised(M);
+    return with_size(M, LaunchSpectrum{p, &p->fft, p->twiddle, false, p->Chat, row_shape(M, pow2), col_shape(M, pow2)});
+}
+
+// Complex values of cwork: the N x M rows of a spectrum build on either grid,
+// and the persistent loop's split-order spectrum at MF = 1024 (k_chat_split).
+size_t cwork_elems(int N, int M, int MF)
+{
+    const size_t rows = (size_t)N * (M > MF ? M : MF), split = MF == 1024 ? (size_t)1024 * 1024 / 2 : 0;
+    return rows > split ? rows : split;
+}
+
+int launch_spectrum_out(spirec_plan p, float* out)
+{
+    if (p->M != p->MF) {
+        const int M = p->M;
+        const bool pow2 = is_pow2_specialised(M);
+        return with_size(M, LaunchSpectrum{p, &p->fft_M, p->twiddle_M, true, out, row_shape(M, pow2), col_shape(M, pow2)});
+    }
+    const unsigned t = (unsigned)((p->M + 31) / 32);
+    k_transpose_real<<<dim3(t, t), dim3(32, 8), 0, p->stream>>>(p->Chat, p->M, out);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
-    const bool pow2 = is_pow2_specialised(M);
-    return with_size(M, LaunchSpectrum{p, row_shape(M, pow2), col_shape(M, pow2)});
+    return SPIREC_OK;
 }
 
 }  // namespace spirec

@@ -104,7 +104,8 @@ struct CgPass {
 struct spirec_plan_s {
     int N;
     int64_t L;
-    int M;
+    int M;   // the embedding grid side the caller sees (the kernel spectrum's)
+    int MF;  // the grid side of every transform (fft_grid): M, or a power of two
     int precision;
     int device;
     cudaStream_t user_stream;
@@ -133,9 +134,9 @@ struct spirec_plan_s {
     double* hpin;
 
     float2* G;     // N x (2N-1)
-    float* Chat;   // M x M real, transposed: Chat[kx*M + ky]
-    float2* cwork; // M x M complex (spectrum build)
-    float2* X;     // N x M complex (Toeplitz rows)
+    float* Chat;   // MF x MF real, transposed: Chat[kx*MF + ky]
+    float2* cwork; // cwork_elems: rows of the spectrum builds, the loop's split-order spectrum
+    float2* X;     // N x MF complex (Toeplitz rows)
     float2* D;     // N x N
     float2* s;     // L (+32 padding)
     float2* ystage;  // L (+32 padding): a caller's y staged for the tensor-core adjoint
@@ -145,7 +146,8 @@ struct spirec_plan_s {
     float2* res;   // T f - D of the iterate (the data term's gradient is 2 res)
     float2* Td;
     float2* tmp;   // N x N scratch for operator calls
-    float2* twiddle;  // M entries, exp(-2 pi i k / M)
+    float2* twiddle;  // MF entries, exp(-2 pi i k / MF)
+    float2* twiddle_M;  // M entries, exp(-2 pi i k / M), when M != MF
     double* part;  // P_NSLOTS x kMaxParts (float-float pairs)
     double* scal;  // S_NSCAL
     unsigned* counters;  // C_N
@@ -157,7 +159,8 @@ struct spirec_plan_s {
     size_t kpart_bytes;
     size_t device_bytes;
 
-    spirec::FftPlan fft;
+    spirec::FftPlan fft;    // of MF
+    spirec::FftPlan fft_M;  // of M
     spirec::Reg reg;
     bool have_traj, have_data, have_reg;
 
@@ -194,6 +197,12 @@ namespace spirec {
 
 int launch_gram(spirec_plan p);            // G from the trajectory
 int launch_spectrum(spirec_plan p);        // Chat from G
+// The M x M kernel spectrum in the caller's layout, out[ky*M + kx]: from Chat,
+// or, when the transforms run on another grid than M, from G.
+int launch_spectrum_out(spirec_plan p, float* out);
+// The grid side the transforms of an N x N image on the caller's grid M use.
+int fft_grid(int N, int M);
+size_t cwork_elems(int N, int M, int MF);
 int launch_adjoint(spirec_plan p, const float2* y, float2* x);  // x = H^H y
 int launch_forward(spirec_plan p, const float2* x, float2* y);  // y = H x
 

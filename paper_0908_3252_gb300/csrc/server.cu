@@ -102,11 +102,12 @@ size_t plan_bytes(int N, int64_t L, int M, int precision)
     b += ((size_t)L + 32) * 8;                   // the paired contractions' weights
     b += 2 * (size_t)L * 8;                      // staging
     b += (size_t)N * (2 * N - 1) * 8;            // G
-    b += (size_t)M * M * 4 + (size_t)M * M * 8;  // spectrum + work
-    b += (size_t)N * M * 8;                      // rows
+    const size_t MF = (size_t)fft_grid(N, M);
+    b += MF * MF * 4 + cwork_elems(N, M, (int)MF) * 8;  // spectrum + work
+    b += (size_t)N * MF * 8;                     // rows
     b += 3 * ((size_t)L + 32) * 8;               // data, its staging, the host upload buffer
     b += 10 * NN * 8;                            // iterates, directions, gradients, D, scratch
-    b += (size_t)M * 8 + (size_t)P_NSLOTS * kMaxParts * 8 + 4096;
+    b += (MF + M) * 8 + (size_t)P_NSLOTS * kMaxParts * 8 + 4096;
     b += fsplit_bytes_tc(N, precision);  // split image of the tensor-core forward
     size_t a = precision == SPIREC_FP32 ? kpart_floats_simt(N, L) : 0, c = 4 * (size_t)L * 2, t = kpart_floats_tc(N, L, precision);
     b += std::max(std::max(a, c), t) * 4;        // split-K partials

@@ -98,3 +98,33 @@ def test_fp32_contraction_shapes(sp, N, L, slices):
     finally:
         p.close()
         sp.spirec_tune_clear()
+
+
+# The kernel spectrum in the caller's layout and T, on grids that are a power
+# of two (the transforms' own) and that are not (the spectrum then comes from
+# G on the caller's grid, the transforms run on a power of two, smaller than M
+# in the last case).  G and FP32 transforms of at most 4096 points: below 1e-5.
+@pytest.mark.parametrize("N,M", [(2, 0), (5, 0), (5, 16), (8, 0), (20, 0), (33, 0), (33, 128), (64, 160), (100, 0), (150, 512),
+                                 (150, 0), (260, 0), (513, 0), (520, 2048)])
+def test_spectrum_and_toeplitz_grids(sp, N, M):
+    import torch
+    from oracle import toeplitz_cpu as TC
+    L = 300
+    g = synth.rng(N + M)
+    kx, ky = synth.uniform_k(L, g)
+    x = c64(synth.complex_normal((N, N), g))
+    with sp.Plan(N, L, M, 0, _stream(), kx, ky) as p:
+        C = torch.zeros((p.M, p.M), dtype=torch.float32, device="cuda")
+        Tx = empty_c64((N, N))
+        sp.spirec_kernel_spectrum_dev(p.h, C)
+        sp.spirec_toeplitz_dev(p.h, to_dev(x), Tx)
+        sp.spirec_sync(p.h)
+        G = O.gram(kx, ky, N)
+        # spirec_kernel_spectrum_dev divides by M^2
+        want = TC.kernel_spectrum(G, N, p.M)
+        assert rel(from_dev(C) * float(p.M) ** 2, want) < 1e-5
+        Mp = 1 << (2 * N - 1).bit_length()
+        assert rel(from_dev(Tx), TC.toeplitz_apply(TC.kernel_spectrum(G, N, Mp), x)) < 1e-5
+        if N <= 512 and p.M <= 1024:
+            sp.spirec_toeplitz_noalloc(to_dev(x), C, Tx, N, p.M, _stream())
+            assert rel(from_dev(Tx), TC.toeplitz_apply(want, x)) < 1e-5
