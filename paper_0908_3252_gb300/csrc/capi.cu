@@ -430,7 +430,7 @@ int solve_core(spirec_plan p, const float* x0, bool x0_dev, int iters)
     if (x0) {
         SPIREC_CK(cudaMemcpyAsync(p->f[0], x0, img,
                                   x0_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, p->stream));
-        if ((rc = direct ? launch_normal_direct(p, p->f[0], p->res, false) : launch_toeplitz(p, p->f[0], p->res, -1)) !=
+        if ((rc = direct ? launch_normal_direct(p, p->f[0], p->res, false) : launch_toeplitz(p, p->f[0], p->res)) !=
             SPIREC_OK)
             return rc;
     } else {
@@ -731,7 +731,7 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRY(dalloc(p, &p->G, (size_t)N * (2 * N - 1)));
     TRY(dalloc(p, &p->Chat, (size_t)MF * MF));
     TRY(dalloc(p, &p->cwork, cwork_elems(N, M, MF)));
-    TRY(dalloc(p, &p->X, (size_t)N * MF));
+    TRY(dalloc(p, &p->X, x_elems(N, MF)));
     if ((p->fsplit_bytes = fsplit_bytes_tc(N, precision)) > 0) TRY(dalloc(p, &p->fsplit, p->fsplit_bytes));
     TRY(dalloc(p, &p->D, NN));
     TRY(dalloc(p, &p->s, (size_t)L + 32));
@@ -1362,7 +1362,7 @@ int spirec_toeplitz_dev(spirec_plan p, const float* x, float* Tx)
         return SPIREC_ESTATE;
     }
     Join j(p);
-    return launch_toeplitz(p, (const float2*)x, (float2*)Tx, -1);
+    return launch_toeplitz(p, (const float2*)x, (float2*)Tx);
 }
 
 int spirec_objective_grad_dev(spirec_plan p, const float* x, double* J_host, float* g)
@@ -1378,7 +1378,7 @@ int spirec_objective_grad_dev(spirec_plan p, const float* x, double* J_host, flo
         return SPIREC_ESTATE;
     }
     Join j(p);
-    if ((rc = launch_toeplitz(p, (const float2*)x, p->tmp, -1)) != SPIREC_OK) return rc;
+    if ((rc = launch_toeplitz(p, (const float2*)x, p->tmp)) != SPIREC_OK) return rc;
     if ((rc = launch_res_init(p, p->tmp, true)) != SPIREC_OK) return rc;  // T x - D
     if ((rc = launch_update(p, (const float2*)x, (float2*)x, p->dbuf[0], p->tmp, nullptr, (float2*)g, 1,
                             nullptr)) != SPIREC_OK)
@@ -1459,7 +1459,7 @@ int spirec_gram_apply(spirec_plan p, const float* x, float* Tx)
     Join j(p);
     const size_t img = sizeof(float2) * (size_t)p->N * p->N;
     SPIREC_CK(cudaMemcpyAsync(p->tmp, x, img, cudaMemcpyHostToDevice, p->stream));
-    if ((rc = launch_toeplitz(p, p->tmp, p->Td, -1)) != SPIREC_OK) return rc;
+    if ((rc = launch_toeplitz(p, p->tmp, p->Td)) != SPIREC_OK) return rc;
     SPIREC_CK(cudaMemcpyAsync(Tx, p->Td, img, cudaMemcpyDeviceToHost, p->stream));
     return finish_host_call(p);
 }
@@ -1479,7 +1479,7 @@ int spirec_objective_grad(spirec_plan p, const float* x, double* J, float* g)
     Join j(p);
     const size_t img = sizeof(float2) * (size_t)p->N * p->N;
     SPIREC_CK(cudaMemcpyAsync(p->Td, x, img, cudaMemcpyHostToDevice, p->stream));
-    if ((rc = launch_toeplitz(p, p->Td, p->tmp, -1)) != SPIREC_OK) return rc;
+    if ((rc = launch_toeplitz(p, p->Td, p->tmp)) != SPIREC_OK) return rc;
     if ((rc = launch_res_init(p, p->tmp, true)) != SPIREC_OK) return rc;  // T x - D
     if ((rc = launch_update(p, p->Td, p->Td, p->dbuf[0], p->tmp, nullptr, p->g, 1, nullptr)) != SPIREC_OK)
         return rc;

@@ -7,9 +7,10 @@
 // moves by t T d with every step.
 //   R(f)      = lambda1 sum_edges phi1(|f_q - f_p|) + lambda0 sum_p phi0(|f_p|)
 //
-// One iteration k is six kernels, all on the device, no host round trip:
-//   rows_fwd  d = -g + beta d_old; q1 = Re<d, 2 res>; line-search
-//             sums at t = 0; row FFTs of d                         (fft.cu)
+// One iteration k is seven kernels, all on the device, no host round trip:
+//   direction d = -g + beta d_old; q1 = Re<d, 2 res>; line-search sums
+//             at t = 0                                             (here)
+//   rows_fwd  row FFTs of d                                        (fft.cu)
 //   cols      column FFT * Chat * IFFT                             (fft.cu)
 //   rows_inv  row IFFTs -> T d; q2 = Re<d, T d>; t1                (fft.cu)
 //   2 x line-search step j -> t_{j+1} = t_j - h'(t_j) / curvature (here)
@@ -24,6 +25,7 @@
 #include <stdint.h>
 
 #include "cg_device.cuh"
+#include "fft_device.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
 
@@ -67,6 +69,85 @@ __global__ void k_sumsq(const float2* __restrict__ s, int64_t L, float2* parts, 
         sum_parts_ff<1>(parts, kMaxParts, gridDim.x, t);
         if (threadIdx.x == 0) {
             scal[S_SS] = ff_to_double(t[0]);
+            *counter = 0u;
+        }
+    }
+}
+
+// A block's part of an N x N image: `rows` rows (fewer at the end) of a strip of
+// 256 columns, a thread a column.  The right neighbour of a value comes from
+// the next lane, that of a warp's last lane (`edge`) from memory.
+struct Strip {
+    int n0, n1;
+    bool in, has_r, edge;
+    int64_t first;  // the thread's pixel of row n0
+    __device__ __forceinline__ Strip(int N, int rows)
+    {
+        const int m = blockIdx.x * kVecThreads + threadIdx.x;
+        n0 = blockIdx.y * rows;
+        n1 = min(N, n0 + rows);
+        in = m < N && n0 < n1;
+        has_r = m + 1 < N;
+        edge = (threadIdx.x & 31) == 31 && has_r && n0 < n1;
+        first = (int64_t)n0 * N + m;
+    }
+    // the right neighbour's value: `own` of the next lane, `mem` in the last
+    static __device__ __forceinline__ float2 right(float2 own, float2 mem)
+    {
+        const float2 s = make_float2(__shfl_down_sync(0xffffffffu, own.x, 1), __shfl_down_sync(0xffffffffu, own.y, 1));
+        return (threadIdx.x & 31) == 31 ? mem : s;
+    }
+};
+
+// The new direction d = -g + beta d_old (into d_new) and the first line-search
+// sums: q1 = Re<d, 2 res> and, over the right and down edges and the pixels,
+//   num0 = sum lambda b(|z|) Re(conj(z) w), den0 = sum lambda b(|z|) |w|^2
+// (z of f, w of d).  A block walks `rows` rows down a strip of 256 columns: the
+// row below's d and f are formed once and kept, the right neighbour's come
+// from the next lane, so a pixel costs its own four loads.
+//
+// Bound by memory latency: 41 us at 2048^2 (five images of 33.5 MB).  With the row FFTs
+// in one kernel, where 16 warps an SM hid neither the loads nor each other, the
+// two took 160 us; they take 41 + 48.
+template <int KIND>
+__global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
+k_direction(const float2* __restrict__ g, const float2* __restrict__ d_old, float2* __restrict__ d_new,
+            const float2* __restrict__ f, const float2* __restrict__ res, int N, int rows, Reg reg, float2* parts,
+            unsigned* counter, double* scal)
+{
+    const double bd = scal[S_BETA];
+    const float beta = (float)bd;
+    const bool restart = (__double_as_longlong(bd) << 1) == 0;  // beta = 0 (an FP64 compare would be redone every pixel)
+    const Strip st(N, rows);
+    const float2 zero = make_float2(0.f, 0.f);
+    auto dir = [&](int64_t o) { return fftd::new_direction(g[o], restart ? zero : d_old[o], beta, restart); };
+    float v[3] = {0.f, 0.f, 0.f};
+    int64_t o = st.first;
+    float2 dn = st.in ? dir(o) : zero, fn = st.in ? f[o] : zero;
+#pragma unroll 2
+    for (int n = st.n0; n < st.n1; ++n, o += N) {
+        const bool has_d = n + 1 < N;
+        const float2 dd = st.in && has_d ? dir(o + N) : dn, fd = st.in && has_d ? f[o + N] : fn;
+        const float2 rs = st.in ? res[o] : zero;
+        const float2 dr = st.right(dn, st.edge ? dir(o + 1) : dn), fr = st.right(fn, st.edge ? f[o + 1] : fn);
+        if (st.in) {
+            d_new[o] = dn;
+            v[0] += 2.f * redot(dn, rs);
+            cgd::ls_terms<KIND>(fn, dn, fr, dr, fd, dd, st.has_r, has_d, reg, 0.f, v[1], v[2]);
+        }
+        dn = dd;
+        fn = fd;
+    }
+    FF bt[3];
+    block_partial<3>(v, bt);
+    store_parts<3>(bt, parts, kMaxParts);
+    if (last_block(counter)) {
+        FF t[3];
+        sum_parts_ff<3>(parts, kMaxParts, gridDim.x * gridDim.y, t);
+        if (threadIdx.x == 0) {
+            scal[S_Q1] = ff_to_double(t[0]);
+            scal[S_NUM0] = ff_to_double(t[1]);
+            scal[S_DEN0] = ff_to_double(t[2]);
             *counter = 0u;
         }
     }
@@ -214,6 +295,42 @@ int launch_update(spirec_plan p, const float2* f_in, float2* f_out, const float2
     return SPIREC_OK;
 }
 
+namespace {
+// Strips of 256 columns by as many rows as fill the resident blocks once.
+dim3 strip_grid(int N, int* rows)
+{
+    int sms = 0;
+    if (device_sms(&sms) != SPIREC_OK || sms <= 0) sms = 152;
+    const int strips = (N + kVecThreads - 1) / kVecThreads, slots = kVecBlocksPerSm * sms;
+    *rows = (int)(((int64_t)N * strips + slots - 1) / slots);
+    if (*rows < 1) *rows = 1;
+    return dim3((unsigned)strips, (unsigned)((N + *rows - 1) / *rows));
+}
+
+template <int KIND>
+void direction_k(spirec_plan p, int k)
+{
+    int rows = 0;
+    const dim3 grid = strip_grid(p->N, &rows);
+    k_direction<KIND><<<grid, kVecThreads, 0, p->stream>>>(p->g, p->dbuf[(k + 1) & 1], p->dbuf[k & 1], p->f[k & 1], p->res,
+                                                           p->N, rows, p->reg, slot(p, P_ROWA), p->counters + C_ROWA,
+                                                           p->scal);
+}
+
+// d of iteration k, q1 and the t = 0 line-search sums.
+int launch_direction(spirec_plan p, int k)
+{
+    switch (p->reg.kind) {
+    case SPIREC_PHI_HUBER: direction_k<SPIREC_PHI_HUBER>(p, k); break;
+    case SPIREC_PHI_HYPERBOLIC: direction_k<SPIREC_PHI_HYPERBOLIC>(p, k); break;
+    default: direction_k<SPIREC_PHI_QUADRATIC>(p, k); break;
+    }
+    SPIREC_CK(cudaGetLastError());
+    p->launches += 1;
+    return SPIREC_OK;
+}
+}  // namespace
+
 // q2 = Re<d, T d> and the first line-search step
 //   t1 = -(q1 + num0) / (2 q2 + den0)   (0 when the curvature is not > 0),
 // as the fused row pass 3 of the FFT path computes them.
@@ -261,33 +378,16 @@ int launch_normal_direct(spirec_plan p, const float2* x, float2* Tx, bool dot_q2
 
 int cg_iteration(spirec_plan p, int k, double* Jdev)
 {
-    const int N = p->N;
     const float2* fin = p->f[k & 1];
     float2* fout = p->f[(k + 1) & 1];
     float2* dk = p->dbuf[k & 1];
     int rc;
-    CgPass a{};
-    a.g = p->g;
-    a.d_old = p->dbuf[(k + 1) & 1];
-    a.d_new = dk;
-    a.f = fin;
-    a.res = p->res;
-    a.D = p->D;
-    a.reg = p->reg;
-    a.parts = slot(p, P_ROWA);
-    a.counter = p->counters + C_ROWA;
-    a.scal = p->scal;
-    // the new direction d, q1 and the t = 0 line-search sums (with the row
-    // FFTs of d, which only the FFT path uses)
-    if ((rc = launch_rows_fwd(p, nullptr, N, N, N, 1, &a)) != SPIREC_OK) return rc;
+    if ((rc = launch_direction(p, k)) != SPIREC_OK) return rc;
     if (p->mode == SPIREC_MODE_DIRECT) {
         if ((rc = launch_normal_direct(p, dk, p->Td, true)) != SPIREC_OK) return rc;
     } else {
-        if ((rc = launch_cols(p, N, N)) != SPIREC_OK) return rc;
-        CgPass c = a;
-        c.parts = slot(p, P_ROWC);
-        c.counter = p->counters + C_ROWC;
-        if ((rc = launch_rows_inv(p, p->Td, 1, dk, &c, 0)) != SPIREC_OK) return rc;
+        const CgPass c{slot(p, P_ROWC), p->counters + C_ROWC, p->scal};
+        if ((rc = launch_toeplitz(p, dk, p->Td, &c)) != SPIREC_OK) return rc;
     }
     for (int j = 1; j <= 2; ++j)
         if ((rc = launch_line_search(p, fin, dk, j)) != SPIREC_OK) return rc;

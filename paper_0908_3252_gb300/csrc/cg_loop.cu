@@ -1268,7 +1268,7 @@ struct LaunchLoop {
 
 }  // namespace
 
-bool loop_supported(int M) { return M >= 64 && M <= 2048 && (M & (M - 1)) == 0; }
+bool loop_supported(int M) { return M >= 64 && M <= 1024 && (M & (M - 1)) == 0; }
 
 namespace {
 struct Shapes {
@@ -1313,7 +1313,6 @@ int shapes_for(const spirec_plan_s* p, int* RB, int* grid, int max, bool current
     case 256: return s.run<256>();
     case 512: return s.run<512>();
     case 1024: return s.run<1024>();
-    case 2048: return s.run<2048>();
     default: return s.run<0>();
     }
 }
@@ -1340,7 +1339,6 @@ int launch_cg_loop(spirec_plan p, int iters)
     case 256: return LaunchLoop{p, iters}.operator()<256>();
     case 512: return LaunchLoop{p, iters}.operator()<512>();
     case 1024: return LaunchLoop{p, iters}.operator()<1024>();
-    case 2048: return LaunchLoop{p, iters}.operator()<2048>();
     default: return LaunchLoop{p, iters}.operator()<0>();
     }
 }

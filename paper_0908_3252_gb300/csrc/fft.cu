@@ -10,10 +10,8 @@
 //   rows:    N row FFTs of the zero-padded rows (N inputs, M outputs),
 //   columns: per column FFT (N nonzero inputs) -> * Chat -> IFFT, rows < N,
 //   rows:    N row IFFTs, columns < N kept.
-// Inside the CG iteration the first row pass also forms the new direction
-// d = -g + beta d_old and the first line-search sums, and the last row pass
-// forms q2 = Re<d, T d> and the first line-search step.  The bodies of the
-// passes live in fft_device.cuh (shared with the persistent loop of
+// Inside the CG iteration the last row pass (the column pass at M >= 2048) also
+// forms q2 = Re<d, T d> and the first line-search step.  The bodies of the passes live in fft_device.cuh (shared with the persistent loop of
 // cg_loop.cu); this file holds the stand-alone kernels and their launchers.
 //
 // FFTs are self-sorting Stockham transforms in shared memory.  For
@@ -23,11 +21,8 @@
 // log2 M), values in registers between a read and a write phase.  Any other
 // M = 2^a 3^b 5^c (a caller's spectrum on such a grid, spirec_toeplitz_noalloc)
 // runs the runtime mixed-radix path with a ping-pong buffer.
-// At M = 2048 and 4096, where every transform of the apply has at most M/2
-// nonzero inputs and keeps at most M/2 outputs, the three passes instead
-// split each transform into S = M / 1024 warp-sized 1024-point DFTs, one per
-// output class k = r mod S (k_rows_fwd_split, k_cols_split,
-// k_rows_inv_split).
+// At M = 2048 and 4096 the three passes split every transform into warp-sized
+// 1024-point DFTs (k_rows_fwd_split, k_cols_split, k_rows_inv_split).
 #include <stdint.h>
 
 #include <atomic>
@@ -66,54 +61,47 @@ using namespace fftd;
 
 // ------------------------------------------------------------- row pass 1
 
-// MODE 0: row FFTs of `in` into X.  MODE 1 (CG): the rows of the new
-// direction, with q1 and the first line-search sums reduced over the grid
-// and finished by the last block into scal (see fft_device.cuh).
-template <int MC, int MODE, int KIND = -1>
+// Row FFTs of `in` (n_in nonzero entries a row) into X.
+template <int MC>
 __global__ void __launch_bounds__(1024) k_rows_fwd(const float2* in, int ld_in, int n_in, int rows, float2* X, FftPlan fp,
-                           const float2* __restrict__ tw, int rpc, CgPass c)
+                           const float2* __restrict__ tw, int rpc)
 {
     extern __shared__ float2 sm[];
     float2* a = sm;
     float2* b = sm + rpc * seq_len<MC>(fp.M);
     const int r0 = blockIdx.x * rpc;
     const int nr = min(rpc, rows - r0);
-    float beta = 0.f;
-    bool restart = true;
-    if (MODE == 1) {
-        const double bd = c.scal[S_BETA];
-        beta = (float)bd;
-        restart = bd == 0.0;
-    }
-    float acc[3] = {0.f, 0.f, 0.f};
-    rows_fwd_group<MC, MODE, KIND>(in, ld_in, n_in, r0, nr, rpc, X, fp, tw, c, beta, restart, a, b, acc);
-    if (MODE == 1) {
-        FF bt[3];
-        block_partial<3>(acc, bt);
-        store_parts<3>(bt, c.parts, kMaxParts);
-        if (last_block(c.counter)) {
-            FF t[3];
-            sum_parts_ff<3>(c.parts, kMaxParts, gridDim.x, t);
-            if (threadIdx.x == 0) {
-                c.scal[S_Q1] = ff_to_double(t[0]);
-                c.scal[S_NUM0] = ff_to_double(t[1]);
-                c.scal[S_DEN0] = ff_to_double(t[2]);
-                *c.counter = 0u;
-            }
-        }
-    }
+    rows_fwd_group<MC>(in, ld_in, n_in, r0, nr, rpc, X, fp, tw, a, b);
 }
 
 // ------------------------------------------------------------- row pass 3
 
-// Row IFFTs of X, first n_out columns to out.  With dotx: s = Re<dotx, out>
-// over the grid; MODE 0 stores it in scal[dot_scalar]; MODE 1 (CG) stores
-// q2 = s and the first line-search step
-//   t1 = -(q1 + num0) / (2 q2 + den0)   (0 when the curvature is not > 0).
-template <int MC, int MODE>
+// The grid sum q2 = Re<d, T d> of every thread's acc, and from it the first
+// line-search step t1 = -(q1 + num0) / (2 q2 + den0) (0 when the curvature is not
+// > 0), by the last block.
+__device__ __forceinline__ void finish_q2(float acc, const CgPass& c)
+{
+    float v[1] = {acc};
+    FF bt[1];
+    block_partial<1>(v, bt);
+    store_parts<1>(bt, c.parts, kMaxParts);
+    if (last_block(c.counter)) {
+        FF t[1];
+        sum_parts_ff<1>(c.parts, kMaxParts, gridDim.x, t);
+        if (threadIdx.x == 0) {
+            const double q2 = ff_to_double(t[0]);
+            c.scal[S_Q2] = q2;
+            const double curv = 2.0 * q2 + c.scal[S_DEN0];
+            c.scal[S_T1] = curv > 0.0 ? -(c.scal[S_Q1] + c.scal[S_NUM0]) / curv : 0.0;
+            *c.counter = 0u;
+        }
+    }
+}
+
+// Row IFFTs of X, first n_out columns to out; CG: also Re<dotx, out> and finish_q2.
+template <int MC, bool CG>
 __global__ void __launch_bounds__(1024) k_rows_inv(const float2* X, int rows, float2* out, int n_out, FftPlan fp,
-                           const float2* __restrict__ tw, int rpc, const float2* dotx, CgPass c,
-                           int dot_scalar)
+                           const float2* __restrict__ tw, int rpc, const float2* dotx, CgPass c)
 {
     extern __shared__ float2 sm[];
     float2* a = sm;
@@ -122,27 +110,7 @@ __global__ void __launch_bounds__(1024) k_rows_inv(const float2* X, int rows, fl
     const int nr = min(rpc, rows - r0);
     float acc = 0.f;
     rows_inv_group<MC>(X, r0, nr, rpc, out, n_out, fp, tw, dotx, a, b, acc);
-    if (dotx) {
-        float v[1] = {acc};
-        FF bt[1];
-        block_partial<1>(v, bt);
-        store_parts<1>(bt, c.parts, kMaxParts);
-        if (last_block(c.counter)) {
-            FF t[1];
-            sum_parts_ff<1>(c.parts, kMaxParts, gridDim.x, t);
-            if (threadIdx.x == 0) {
-                const double s = ff_to_double(t[0]);
-                if (MODE == 0) {
-                    c.scal[dot_scalar] = s;
-                } else {
-                    c.scal[S_Q2] = s;
-                    const double curv = 2.0 * s + c.scal[S_DEN0];
-                    c.scal[S_T1] = curv > 0.0 ? -(c.scal[S_Q1] + c.scal[S_NUM0]) / curv : 0.0;
-                }
-                *c.counter = 0u;
-            }
-        }
-    }
+    if (CG) finish_q2(acc, c);
 }
 
 // ------------------------------------------------------------- column pass
@@ -157,7 +125,30 @@ __global__ void __launch_bounds__(1024) k_cols_filter(float2* X, int n_in, int n
     cols_group<MC>(X, n_in, n_out, x0, min(cpc, fp.M - x0), cpc, fp, tw, Chat, sm, sm + cpc * ld);
 }
 
-// ----------------------------------------- column pass, M = 1024 S >= 2048
+// ------------------------------------------------- passes at M = 1024 S >= 2048
+//
+// The transforms of the apply have at most M/2 nonzero inputs and keep at most
+// M/2 outputs, so each splits into S warp-sized 1024-point DFTs, one per
+// output class r = k mod S:
+//   forward: X[S k + r] = DFT1024(z_r)[k],
+//            z_r[m] = w_M^(r m) sum_{t < S/2} x[m + 1024 t] w_S^(r t);
+//   inverse: u_r = IDFT1024 of class r, out[n] = sum_r w_M^(-r n) u_r[n mod 1024],
+//            n and n + 1024 from the same S values.
+// The columns of X are in class order, c = 1024 r + k for the frequency S k + r,
+// and so is Chat in both indices (split_pos).  X lies in pairs of columns, each
+// in tiles of two rows and two columns, one 32-byte sector: element (y, c) at
+//      ((c / 2) ldx + 2 (y / 2)) 2 + 2 (c % 2) + y % 2,
+// ldx = N rounded up to even (split_ld).  The column pass, the heaviest, moves a
+// pair of columns as one contiguous run; the row passes, two rows at a time,
+// move whole sectors, each as one 32-byte access.
+//
+// At 2048^2, M = 4096 (us, the same with 16-byte pieces of a row-major X and two
+// or three columns or rows a block, staged by loads): row pass 1 48 (about 60),
+// column pass 103 (155), row pass 3 47 (49 with its dot product, which is now a
+// few multiply-adds of the column pass); one T apply 254 -> 180.  The column
+// pass is bound by its instructions (55% of the issue slots at 16 warps an SM,
+// 62 M instructions) and by shared memory; with X by columns and the row passes
+// writing and reading 16-byte pieces it takes 93, but they take 102 and 81.
 
 // One warp, the 1024-point DFT (conjugate twiddles when INV) of the sequence
 // whose element lane + 32 j is in x[j], as four steps: DFT over the
@@ -195,340 +186,326 @@ __device__ __forceinline__ void unreverse32(float2 (&x)[32])
     }
 }
 
-// The split passes run 8 warps a CTA and two CTAs an SM, so that one CTA's
-// loads overlap the other's transforms.
 constexpr int kSplitWarps = 8;
 constexpr int kSplitThreads = 32 * kSplitWarps;
-constexpr int kSplitCtasPerSm = 16 / kSplitWarps;
-// The inverse row pass has no staging buffer (76 KB of shared memory a CTA),
-// so three CTAs fit an SM; its DFTs fit 85 registers a thread without spills.
-constexpr int kSplitInvCtasPerSm = 3;
-// Warp area of the column pass: 32 x 33 for the four-step DFT plus 2, so that
-// the S areas of one column start 8 (S = 4) or 4 (S = 2) float2 banks after
-// those of the previous column, and the combine step, whose neighbouring
-// threads read neighbouring columns, hits distinct banks.
-constexpr int kSplitArea = 1058;
+constexpr int kSplitCtasPerSm = 2;  // 128 registers a thread, up to 108 KB of shared memory
+constexpr int kSplitArea = 32 * 33;
 
-// Input m (m < 1024) of the 1024-point DFT that gives the outputs k = r mod S
-// of an M = 1024 S point DFT of x (x zero from M/2 on):
-//   z_r[m] = w_M^(r m) sum_{t < S/2} x[m + 1024 t] w_S^(r t),
-// as w_M^(r (m + 1024 t)) = w_M^(r m) w_S^(r t).  For S = 4 the factor
-// w_4^r = (-i)^r is applied exactly (a swap and sign changes).
+// Shared memory of the split passes: the warps' areas, the 32 x 32 twiddles
+// and the fold's twiddles w_{32 S}^e.
+struct SplitSmem {
+    float2 area[kSplitWarps][kSplitArea];
+    float2 t2[1024];
+    float2 fold[128];
+};
+
 template <int S>
-__device__ __forceinline__ float2 fold_input(const float2* x, int m, int r, const float2* __restrict__ tw)
+__device__ __forceinline__ void split_tables(SplitSmem& sm, const float2* __restrict__ tw)
 {
-    float2 z = x[m];
-    if constexpr (S == 4) {
-        const float2 v = x[m + 1024];
-        const float2 rv = r == 0 ? v : r == 1 ? make_float2(v.y, -v.x) : r == 2 ? make_float2(-v.x, -v.y)
-                                                                                : make_float2(-v.y, v.x);
-        z = freg::add(z, rv);
+    constexpr int M = 1024 * S;
+    for (int e = threadIdx.x; e < 1024; e += kSplitThreads) sm.t2[e] = __ldg(tw + ((S * (e >> 5) * (e & 31)) & (M - 1)));
+    for (int e = threadIdx.x; e < 32 * S; e += kSplitThreads) sm.fold[e] = __ldg(tw + 32 * e);
+    __syncthreads();
+}
+
+// One 32-byte sector (p 32-byte aligned) as one access.
+__device__ __forceinline__ void store_sector(float2* p, float2 a, float2 b, float2 c, float2 d)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(b.x),
+                 "f"(b.y), "f"(c.x), "f"(c.y), "f"(d.x), "f"(d.y)
+                 : "memory");
+}
+__device__ __forceinline__ void load_sector(const float2* p, float2 (&v)[4])
+{
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y)
+        : "l"(p));
+}
+
+// Barrier of `threads` threads of the block (whole warps), id 1 .. 15.
+__device__ __forceinline__ void team_sync(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// The folded input of class r: z_r[m], m = lane + 32 j, from src[0 .. n) in
+// shared memory, with
+// the factor w_4^r = (-i)^r exact (a swap and sign changes) and w_M^(r m) =
+// w_M^(r lane) w_{32 S}^(r j).
+template <int S>
+__device__ __forceinline__ void load_folded(float2 (&x)[32], const float2* src, int n, int r, int lane,
+                                            const float2* fold, float2 wl)
+{
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const int m = lane + 32 * j;
+        x[j] = m < n ? src[m] : make_float2(0.f, 0.f);
     }
-    return r == 0 ? z : cmul(z, __ldg(tw + r * m));
-}
-
-// Output n (n < M/2) of the inverse M-point DFT from the S inverse 1024-point
-// DFTs u_r of the classes k = r mod S (u_r at u + r * stride, index n mod
-// 1024 applied by the caller): sum_r w_M^(-r n) u_r, by Horner's rule in
-// conj(w_M^n).
-template <int S>
-__device__ __forceinline__ float2 combine_output(const float2* u, int stride, int n, const float2* __restrict__ tw)
-{
-    const float2 c = conjf2(__ldg(tw + n));
-    float2 y = u[(S - 1) * stride];
+    if constexpr (S == 4) {
 #pragma unroll
-    for (int r = S - 2; r >= 0; --r) y = freg::add(u[r * stride], cmul(c, y));
-    return y;
-}
-
-// Stride of a staged column of k_cols_split<S>: the 8 / S columns of one
-// row piece land on distinct banks (offsets 8 float2 apart for two columns,
-// 4 for four).
-template <int S>
-__host__ __device__ constexpr int cols_split_ld() { return 512 * S + (S == 4 ? 8 : 4); }
-
-// Shared memory of k_cols_split<S>: the warps' areas, whose start the staged
-// columns share (they are dead once every warp has folded its column into
-// registers), then the 32 x 32 twiddles: 76 KB, three CTAs an SM.
-template <int S>
-constexpr size_t cols_split_smem()
-{
-    const size_t stage = (size_t)(kSplitWarps / S) * cols_split_ld<S>(), areas = (size_t)kSplitWarps * kSplitArea;
-    return ((stage > areas ? stage : areas) + 1024) * sizeof(float2);
-}
-constexpr int kSplitColCtasPerSm = 3;
-
-// The Toeplitz column pass for M = 1024 S (S = 2, 4) when at most M/2 rows
-// are nonzero and at most M/2 are kept (n_in, n_out <= M/2, always the case
-// for N x N images): column FFT * Chat * IFFT with every 1024-point DFT in
-// one warp's registers.  X[S k + r] = DFT1024(z_r)[k] with
-// z_r[m] = sum_t x[m + 1024 t] w_M^(r (m + 1024 t)) (t < S/2, the input
-// folded to 1024 points), so warp r of a column computes the outputs
-// k = r mod S; after the spectrum and the inverse 1024-point DFT u_r, the
-// column's rows are y[n] = sum_r w_M^(-r n) u_r[n mod 1024], summed in a fixed
-// order.  8 / S columns a group, staged from X as row pieces of 8 / S
-// neighbouring columns; CTAs loop over the groups.  tw[e] = w_M^e.
-template <int S>
-__global__ void __launch_bounds__(kSplitThreads, kSplitColCtasPerSm)
-k_cols_split(float2* X, int n_in, int n_out, const float2* __restrict__ tw, const float* __restrict__ Chat)
-{
-    constexpr int M = 1024 * S, C = kSplitWarps / S, H = M / 2, LDS = cols_split_ld<S>();
-    static_assert(C * LDS <= kSplitWarps * kSplitArea, "the staged columns fit in the areas");
-    extern __shared__ float2 sm[];
-    float2* areas = sm;
-    float2* stage = sm;  // shares the areas' start
-    float2* t2 = areas + kSplitWarps * kSplitArea;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cc = warp / S, r = warp - cc * S;
-    for (int e = tid; e < 1024; e += kSplitThreads) t2[e] = __ldg(tw + ((S * (e >> 5) * (e & 31)) & (M - 1)));
-    for (int x0 = blockIdx.x * C; x0 < M; x0 += gridDim.x * C) {
-#pragma unroll 8
-        for (int e = tid; e < C * H; e += kSplitThreads) {
-            const int y = e / C, c = e - y * C;
-            stage[c * LDS + y] = y < n_in ? __ldcg(X + (int64_t)y * M + x0 + c) : make_float2(0.f, 0.f);
+        for (int j = 0; j < 32; ++j) {
+            const int m = lane + 32 * j + 1024;
+            const float2 v = m < n ? src[m] : make_float2(0.f, 0.f);
+            const float2 rv = r == 0 ? v : r == 1 ? make_float2(v.y, -v.x) : r == 2 ? make_float2(-v.x, -v.y)
+                                                                                    : make_float2(-v.y, v.x);
+            x[j] = freg::add(x[j], rv);
         }
-        __syncthreads();
-        // the warp's folded, twiddled input into registers; then every warp
-        // has read the stage, and the areas may overwrite it
+    }
+    if (r > 0) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) x[j] = cmul(x[j], cmul(fold[r * j], wl));
+    }
+}
+
+// Outputs m and m + 1024 (S = 4) of the inverse transform from the classes'
+// values u[r] = u_r[m]: v_r = w_M^(-r m) u_r, y[m] = sum v_r, y[m + 1024] =
+// sum i^r v_r.
+template <int S>
+__device__ __forceinline__ void combine_classes(const float2 (&u)[S], const float2 (&w)[S], float2& y0, float2& y1)
+{
+    const float2 v1 = cmul(u[1], conjf2(w[1]));
+    if constexpr (S == 2) {
+        y0 = freg::add(u[0], v1);
+        y1 = make_float2(0.f, 0.f);
+    } else {
+        const float2 v2 = cmul(u[2], conjf2(w[2])), v3 = cmul(u[3], conjf2(w[3]));
+        const float2 a = freg::add(u[0], v2), b = freg::sub(u[0], v2), c = freg::add(v1, v3), d = freg::sub(v1, v3);
+        y0 = freg::add(a, c);
+        y1 = make_float2(b.x - d.y, b.y + d.x);
+    }
+}
+
+// w[r] = w_M^(r m), r = 1 .. S - 1.
+template <int S>
+__device__ __forceinline__ void class_twiddles(float2 (&w)[S], int m, const float2* __restrict__ tw)
+{
+#pragma unroll
+    for (int r = 1; r < S; ++r) w[r] = __ldg(tw + r * m);
+}
+
+// The split passes' shared memory with what comes next on its way: a column a
+// team (4 of 1024 rows at S = 2, 2 of 2048 at S = 4) or 8/S rows.
+struct StagedSmem {
+    SplitSmem s;
+    float2 stage[4096];
+};
+
+__device__ __forceinline__ void cp_async16(float2* dst, const float2* src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(float2* dst, const float2* src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Column pass: FFT * Chat * IFFT of every column of X (N rows), a team of 2S
+// warps a pair of columns, S a column, teams looping over the pairs on their
+// own.  A team's next pair is copied into its stage as soon as the fold has read
+// it, and a column's spectrum is loaded before its first DFT.  CG: also Re<d, T
+// d> = sum Chat |FFT2(d)|^2 (Parseval: the row pass then reads no d) and finish_q2.
+template <int S, bool CG>
+__global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
+k_cols_split(float2* X, int N, int ldx, const float2* __restrict__ tw, const float* __restrict__ Chat, CgPass dot)
+{
+    constexpr int M = 1024 * S, C = kSplitWarps / (2 * S), T = 64 * S;  // pairs a block, threads a team
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StagedSmem& ss = *reinterpret_cast<StagedSmem*>(smem_raw);
+    SplitSmem& sm = ss.s;
+    split_tables<S>(sm, tw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int team = warp / (2 * S), cc = (warp / S) & 1, r = warp % S, t = threadIdx.x % T;
+    const float2 wl = __ldg(tw + r * lane);
+    float2* area = sm.area[warp];
+    float2* stage = ss.stage + team * (1024 * S);  // column cc at 512 S cc
+    // 16-byte chunk e of the pair: rows 2 (e / 2), + 1 of column e % 2
+    auto fetch = [&](int pair) {
+        const float2* src = X + (int64_t)pair * 2 * ldx;
+        for (int e = t; e < ldx; e += T) cp_async16(stage + (e & 1) * (512 * S) + (e & ~1), src + 2 * e);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc = 0.f;
+    int pair = blockIdx.x * C + team;
+    if (pair < M / 2) fetch(pair);
+    for (; pair < M / 2; pair += gridDim.x * C) {
+        const int c = 2 * pair + cc;
+        float h[32];
+        {
+            const float* ch = Chat + (int64_t)c * M + 1024 * r + lane;
+#pragma unroll
+            for (int k2 = 0; k2 < 32; ++k2) h[k2] = __ldg(ch + 32 * k2);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        team_sync(1 + team, T);  // the pair has landed; the team's areas are read
         float2 x[32];
-        {
-            const float2* col = stage + cc * LDS;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) x[j] = fold_input<S>(col, lane + 32 * j, r, tw);
-        }
-        __syncthreads();
-        float2* area = areas + warp * kSplitArea;
-        dft1024_warp<false>(x, area, t2, lane);  // X[S (lane + 32 k2) + r] in x[bitrev5(k2)]
+        load_folded<S>(x, stage + cc * (512 * S), N, r, lane, sm.fold, wl);
+        team_sync(1 + team, T);  // the stage is read
+        if (pair + (int)gridDim.x * C < M / 2) fetch(pair + (int)gridDim.x * C);
+        dft1024_warp<false>(x, area, sm.t2, lane);  // frequency S (lane + 32 k2) + r in x[bitrev5(k2)]
         unreverse32(x);
-        {
-            const float* ch = Chat + (int64_t)(x0 + cc) * M + r + S * lane;
 #pragma unroll
-            for (int k2 = 0; k2 < 32; ++k2) {
-                const float h = __ldg(ch + 32 * S * k2);
-                x[k2] = make_float2(x[k2].x * h, x[k2].y * h);
-            }
+        for (int k2 = 0; k2 < 32; ++k2) {
+            const float2 y = make_float2(x[k2].x * h[k2], x[k2].y * h[k2]);
+            if (CG) acc += redot(x[k2], y);
+            x[k2] = y;
         }
-        dft1024_warp<true>(x, area, t2, lane);  // u_r[lane + 32 m2] in x[bitrev5(m2)]
+        dft1024_warp<true>(x, area, sm.t2, lane);  // u_r[lane + 32 m2] in x[bitrev5(m2)]
 #pragma unroll
         for (int m2 = 0; m2 < 32; ++m2) area[lane + 32 * m2] = x[freg::bitrev5(m2)];
-        __syncthreads();
-#pragma unroll 4
-        for (int e = tid; e < C * n_out; e += kSplitThreads) {
-            const int y = e / C, c = e - y * C;
-            X[(int64_t)y * M + x0 + c] = combine_output<S>(areas + c * S * kSplitArea + (y & 1023), kSplitArea, y, tw);
+        team_sync(1 + team, T);
+        // rows m, m + 1 (and + 1024) of both columns: one sector each
+        const float2(*u)[kSplitArea] = &sm.area[team * 2 * S];
+#pragma unroll 1
+        for (int m = 2 * t; m < 1024; m += 2 * T) {
+            float2 w0[S], w1[S], y0[4], y1[4];
+            class_twiddles<S>(w0, m, tw);
+            class_twiddles<S>(w1, m + 1, tw);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float2 a[S], b[S];
+#pragma unroll
+                for (int i = 0; i < S; ++i) {
+                    const float4 v = *reinterpret_cast<const float4*>(&u[k * S + i][m]);
+                    a[i] = make_float2(v.x, v.y);
+                    b[i] = make_float2(v.z, v.w);
+                }
+                combine_classes<S>(a, w0, y0[2 * k], y1[2 * k]);
+                combine_classes<S>(b, w1, y0[2 * k + 1], y1[2 * k + 1]);
+            }
+            float2* o = X + (int64_t)pair * 2 * ldx + 2 * m;
+            if (m < N) store_sector(o, y0[0], y0[1], y0[2], y0[3]);
+            if (S == 4 && m + 1024 < N) store_sector(o + 2048, y1[0], y1[1], y1[2], y1[3]);
         }
-        __syncthreads();  // the next group refills the stage and the areas
     }
+    if (CG) finish_q2(acc, dot);
 }
 
-// ------------------------------------------- row passes, M = 1024 S >= 2048
-
-// Warp areas of the split row passes: 32 x 33 for the four-step DFT, padded
-// so that whole-row copies, whose neighbouring elements k = S j + r live in
-// the S areas of a row at j, hit distinct banks (area stride = 4 or 8 mod 16).
+// Row pass 1: the row FFTs of `in` (N x N) into X, R = 8/S rows a block at a
+// time, the next ones copied into the stage meanwhile.  Warp (q, r) transforms
+// class r of row q; the R warps of a class then write its columns, a sector of
+// two rows and two columns at a time (rows past N: zeros).
 template <int S>
-__host__ __device__ constexpr int row_area() { return 1056 + (S == 4 ? 4 : 8); }
-
-// Shared memory of the split row passes: (pass 1 only) the staged rows, then
-// the warps' areas and the 32 x 32 twiddles.
-template <int S, bool STAGE>
-constexpr size_t rows_split_smem()
-{
-    return ((STAGE ? (size_t)(kSplitWarps / S) * (512 * S + 4) : 0) + kSplitWarps * row_area<S>() + 1024) * sizeof(float2);
-}
-
-// Row pass 1 for M = 1024 S (S = 2, 4) with at most M/2 nonzero inputs
-// (n_in <= M/2): the rows (MODE 1: the new direction d = -g + beta d_old,
-// written to d_new, with q1 and the first line-search sums as in
-// rows_fwd_group) staged in shared memory, then warp r of a row computes the
-// outputs k = r mod S of its 1024-point DFT from the folded input
-// sum_t x[m + 1024 t] w_M^(r (m + 1024 t)), and the block writes whole rows
-// of X.  8 / S rows a group; CTAs loop over the groups.
-template <int S, int MODE, int KIND>
 __global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
-k_rows_fwd_split(const float2* in, int ld_in, int n_in, int rows, float2* X, const float2* __restrict__ tw,
-                 CgPass c)
+k_rows_fwd_split(const float2* __restrict__ in, int N, float2* X, int ldx, const float2* __restrict__ tw)
 {
-    constexpr int M = 1024 * S, R = kSplitWarps / S, H = M / 2, LDS = H + 4, A = row_area<S>();
-    extern __shared__ float2 sm[];
-    float2* stage = sm;
-    float2* areas = stage + R * LDS;
-    float2* t2 = areas + kSplitWarps * A;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int R = kSplitWarps / S, T = 32 * S;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StagedSmem& ss = *reinterpret_cast<StagedSmem*>(smem_raw);
+    SplitSmem& sm = ss.s;
+    split_tables<S>(sm, tw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = warp / S, r = warp - q * S;
-    for (int e = tid; e < 1024; e += kSplitThreads) t2[e] = __ldg(tw + ((S * (e >> 5) * (e & 31)) & (M - 1)));
-    float beta = 0.f;
-    bool restart = true;
-    if (MODE == 1) {
-        const double bd = c.scal[S_BETA];
-        beta = (float)bd;
-        restart = bd == 0.0;
-    }
-    const int N = n_in;
-    float acc[3] = {0.f, 0.f, 0.f};
-    for (int r0 = blockIdx.x * R; r0 < rows; r0 += gridDim.x * R) {
-        const int nr = min(R, rows - r0);
-#pragma unroll 4
-        for (int e = tid; e < R * H; e += kSplitThreads) {
-            const int qq = e / H, m = e - qq * H;
-            float2 v = make_float2(0.f, 0.f);
-            if (qq < nr && m < N) {
-                const int64_t o = (int64_t)(r0 + qq) * ld_in + m;
-                if (MODE == 0) {
-                    v = __ldcg(in + o);
-                } else {
-                    v = new_direction(__ldcg(c.g + o), __ldcg(c.d_old + o), beta, restart);
-                    c.d_new[o] = v;
-                }
-            }
-            stage[qq * LDS + m] = v;
+    const float2 wl = __ldg(tw + r * lane);
+    float2* area = sm.area[warp];
+    float2* stage = ss.stage + q * (512 * S);
+    const bool al16 = (N & 1) == 0 && ((uintptr_t)in & 15) == 0;  // 16-byte copies of a row
+    auto fetch = [&](int row) {
+        if (row < N) {
+            const float2* src = in + (int64_t)row * N;
+            if (al16)
+                for (int e = 2 * (32 * r + lane); e < N; e += 2 * T) cp_async16(stage + e, src + e);
+            else
+                for (int e = 32 * r + lane; e < N; e += T) cp_async8(stage + e, src + e);
         }
-        __syncthreads();
-        if (MODE == 1) {
-            const Reg reg = c.reg;
-#pragma unroll 4
-            for (int e = tid; e < nr * N; e += kSplitThreads) {
-                const int qq = e / N, m = e - qq * N;
-                const int n = r0 + qq;
-                const int64_t o = (int64_t)n * N + m;
-                const bool has_r = m + 1 < N, has_d = n + 1 < N;
-                const int64_t od = has_d ? o + N : o;
-                const float2 dn = stage[qq * LDS + m];
-                const float2 dr = stage[qq * LDS + (has_r ? m + 1 : m)];
-                const float2 fp_ = __ldcg(c.f + o), fr = __ldcg(c.f + (has_r ? o + 1 : o)), fd = __ldcg(c.f + od);
-                const float2 gd = __ldcg(c.g + od), dold_d = __ldcg(c.d_old + od);
-                acc[0] += 2.f * redot(dn, __ldcg(c.res + o));
-                if (reg.lambda1 != 0.f) {
-                    {
-                        const float2 w = f2sub(dr, dn);
-                        const float2 z = f2sub(fr, fp_);
-                        const float bw =
-                            has_r ? reg.lambda1 * phi_weight_k<KIND>(reg.kind, reg.alpha1, redot(z, z)) : 0.f;
-                        acc[1] = fmaf(bw, redot(z, w), acc[1]);
-                        acc[2] = fmaf(bw, redot(w, w), acc[2]);
-                    }
-                    {
-                        const float2 dd = new_direction(gd, dold_d, beta, restart);
-                        const float2 w = f2sub(dd, dn);
-                        const float2 z = f2sub(fd, fp_);
-                        const float bw =
-                            has_d ? reg.lambda1 * phi_weight_k<KIND>(reg.kind, reg.alpha1, redot(z, z)) : 0.f;
-                        acc[1] = fmaf(bw, redot(z, w), acc[1]);
-                        acc[2] = fmaf(bw, redot(w, w), acc[2]);
-                    }
-                }
-                if (reg.lambda0 != 0.f) {
-                    const float bw = reg.lambda0 * phi_weight_k<KIND>(reg.kind, reg.alpha0, redot(fp_, fp_));
-                    acc[1] = fmaf(bw, redot(fp_, dn), acc[1]);
-                    acc[2] = fmaf(bw, redot(dn, dn), acc[2]);
-                }
-            }
-        }
-        if (q < nr) {
-            float2* area = areas + warp * A;
-            const float2* row = stage + q * LDS;
-#pragma unroll 4
-            for (int m = lane; m < 1024; m += 32) area[m] = fold_input<S>(row, m, r, tw);
-            __syncwarp();
-            float2 x[32];
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int r0 = blockIdx.x * R;
+    fetch(r0 + q);
+    for (; r0 < N; r0 += gridDim.x * R) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        team_sync(8 + q, T);  // the row has landed
+        float2 x[32];
+        load_folded<S>(x, stage, r0 + q < N ? N : 0, r, lane, sm.fold, wl);
+        team_sync(8 + q, T);  // the stage is read
+        fetch(r0 + (int)gridDim.x * R + q);
+        dft1024_warp<false>(x, area, sm.t2, lane);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) x[j] = area[lane + 32 * j];
-            __syncwarp();
-            dft1024_warp<false>(x, area, t2, lane);
+        for (int k2 = 0; k2 < 32; ++k2) area[lane + 32 * k2] = x[freg::bitrev5(k2)];
+        team_sync(1 + r, 32 * R);
+#pragma unroll 4
+        for (int k = 2 * (32 * q + lane); k < 1024; k += 64 * R) {
 #pragma unroll
-            for (int k2 = 0; k2 < 32; ++k2) area[lane + 32 * k2] = x[freg::bitrev5(k2)];
-        }
-        __syncthreads();
-        for (int e = tid; e < nr * M; e += kSplitThreads) {
-            const int qq = e / M, kk = e - qq * M;
-            X[(int64_t)(r0 + qq) * M + kk] = areas[(qq * S + (kk & (S - 1))) * A + kk / S];
-        }
-        __syncthreads();  // the next group refills the stage and the areas
-    }
-    if (MODE == 1) {
-        FF bt[3];
-        block_partial<3>(acc, bt);
-        store_parts<3>(bt, c.parts, kMaxParts);
-        if (last_block(c.counter)) {
-            FF t[3];
-            sum_parts_ff<3>(c.parts, kMaxParts, gridDim.x, t);
-            if (threadIdx.x == 0) {
-                c.scal[S_Q1] = ff_to_double(t[0]);
-                c.scal[S_NUM0] = ff_to_double(t[1]);
-                c.scal[S_DEN0] = ff_to_double(t[2]);
-                *c.counter = 0u;
+            for (int h = 0; h < R; h += 2) {
+                const float4 a = *reinterpret_cast<const float4*>(&sm.area[h * S + r][k]);
+                const float4 b = *reinterpret_cast<const float4*>(&sm.area[(h + 1) * S + r][k]);
+                if (r0 + h < N)
+                    store_sector(X + ((int64_t)(512 * r + (k >> 1)) * ldx + r0 + h) * 2, make_float2(a.x, a.y),
+                                 make_float2(b.x, b.y), make_float2(a.z, a.w), make_float2(b.z, b.w));
             }
         }
+        team_sync(1 + r, 32 * R);  // the class's areas are read
     }
 }
 
-// Row pass 3 for M = 1024 S (S = 2, 4), n_out <= M/2: each row of X copied
-// whole into the S warp areas (element S j + r to area r at j), warp r's
-// inverse 1024-point DFT u_r, and out[m] = sum_r w_M^(-r m) u_r[m mod 1024]
-// in a fixed order; with dotx the same grid sum and scalars as k_rows_inv.
-template <int S, int MODE>
-__global__ void __launch_bounds__(kSplitThreads, kSplitInvCtasPerSm)
-k_rows_inv_split(const float2* X, int rows, float2* out, int n_out, const float2* __restrict__ tw,
-                 const float2* dotx, CgPass c, int dot_scalar)
+// Row pass 3: the row IFFTs of X to out (N x N), R = 8/S rows a block at a time.
+// The R warps of a class bring its part of the rows into the areas (every
+// sector of a thread in flight at once), warp (q, r) transforms class r of row
+// q, and the S warps of a row combine its classes.
+template <int S>
+__global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
+k_rows_inv_split(const float2* __restrict__ X, int N, int ldx, float2* __restrict__ out, const float2* __restrict__ tw)
 {
-    constexpr int M = 1024 * S, R = kSplitWarps / S, A = row_area<S>();
-    extern __shared__ float2 sm[];
-    float2* areas = sm;
-    float2* t2 = areas + kSplitWarps * A;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp / S;
-    for (int e = tid; e < 1024; e += kSplitThreads) t2[e] = __ldg(tw + ((S * (e >> 5) * (e & 31)) & (M - 1)));
-    float acc = 0.f;
-    for (int r0 = blockIdx.x * R; r0 < rows; r0 += gridDim.x * R) {
-        const int nr = min(R, rows - r0);
-#pragma unroll 8
-        for (int e = tid; e < nr * M; e += kSplitThreads) {
-            const int qq = e / M, kk = e - qq * M;
-            areas[(qq * S + (kk & (S - 1))) * A + kk / S] = __ldcg(X + (int64_t)(r0 + qq) * M + kk);
-        }
-        __syncthreads();
-        if (q < nr) {
-            float2* area = areas + warp * A;
-            float2 x[32];
+    constexpr int R = kSplitWarps / S;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SplitSmem& sm = *reinterpret_cast<SplitSmem*>(smem_raw);
+    split_tables<S>(sm, tw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = warp / S, r = warp - q * S;
+    float2* area = sm.area[warp];
+    for (int r0 = blockIdx.x * R; r0 < N; r0 += gridDim.x * R) {
+        {
+            constexpr int V = 512 / (32 * R);  // sectors of a row pair a thread
+            float2 v[R / 2 * V][4];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) x[j] = area[lane + 32 * j];
-            __syncwarp();
-            dft1024_warp<true>(x, area, t2, lane);  // u_r[lane + 32 m2] in x[bitrev5(m2)]
+            for (int i = 0; i < R / 2 * V; ++i) {
+                const int h = 2 * (i / V), k2 = 32 * q + lane + 32 * R * (i % V);
 #pragma unroll
-            for (int m2 = 0; m2 < 32; ++m2) area[lane + 32 * m2] = x[freg::bitrev5(m2)];
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int e = tid; e < nr * n_out; e += kSplitThreads) {
-            const int qq = e / n_out, m = e - qq * n_out;
-            const float2 y = combine_output<S>(areas + qq * S * A + (m & 1023), A, m, tw);
-            const int64_t o = (int64_t)(r0 + qq) * n_out + m;
-            out[o] = y;
-            if (dotx) acc += redot(__ldcg(dotx + o), y);
-        }
-        __syncthreads();
-    }
-    if (dotx) {
-        float v[1] = {acc};
-        FF bt[1];
-        block_partial<1>(v, bt);
-        store_parts<1>(bt, c.parts, kMaxParts);
-        if (last_block(c.counter)) {
-            FF t[1];
-            sum_parts_ff<1>(c.parts, kMaxParts, gridDim.x, t);
-            if (threadIdx.x == 0) {
-                const double sv = ff_to_double(t[0]);
-                if (MODE == 0) {
-                    c.scal[dot_scalar] = sv;
-                } else {
-                    c.scal[S_Q2] = sv;
-                    const double curv = 2.0 * sv + c.scal[S_DEN0];
-                    c.scal[S_T1] = curv > 0.0 ? -(c.scal[S_Q1] + c.scal[S_NUM0]) / curv : 0.0;
-                }
-                *c.counter = 0u;
+                for (int e = 0; e < 4; ++e) v[i][e] = make_float2(0.f, 0.f);
+                if (r0 + h < N) load_sector(X + ((int64_t)(512 * r + k2) * ldx + r0 + h) * 2, v[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < R / 2 * V; ++i) {
+                const int h = 2 * (i / V), k = 2 * (32 * q + lane + 32 * R * (i % V));
+                *reinterpret_cast<float4*>(&sm.area[h * S + r][k]) = make_float4(v[i][0].x, v[i][0].y, v[i][2].x, v[i][2].y);
+                *reinterpret_cast<float4*>(&sm.area[(h + 1) * S + r][k]) =
+                    make_float4(v[i][1].x, v[i][1].y, v[i][3].x, v[i][3].y);
             }
         }
+        team_sync(1 + r, 32 * R);
+        float2 x[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) x[j] = area[lane + 32 * j];
+        __syncwarp();
+        dft1024_warp<true>(x, area, sm.t2, lane);  // u_r[lane + 32 m2] in x[bitrev5(m2)]
+#pragma unroll
+        for (int m2 = 0; m2 < 32; ++m2) area[lane + 32 * m2] = x[freg::bitrev5(m2)];
+        team_sync(8 + q, 32 * S);
+        if (r0 + q < N) {
+            float2* o = out + (int64_t)(r0 + q) * N;
+#pragma unroll 4
+            for (int m = 32 * r + lane; m < 1024; m += 32 * S) {
+                float2 w[S], u[S], y0, y1;
+                class_twiddles<S>(w, m, tw);
+#pragma unroll
+                for (int i = 0; i < S; ++i) u[i] = sm.area[q * S + i][m];
+                combine_classes<S>(u, w, y0, y1);
+                if (m < N) o[m] = y0;
+                if (S == 4 && m + 1024 < N) o[m + 1024] = y1;
+            }
+        }
+        __syncthreads();  // the next rows refill the areas
     }
+}
+
+// Position of frequency k in the columns of X and in Chat at M = MC: the class
+// order of the split passes, else k itself.
+template <int MC>
+__host__ __device__ __forceinline__ int split_pos(int k)
+{
+    constexpr int S = MC >= 2048 ? MC / 1024 : 1;
+    return S > 1 ? (k & (S - 1)) * 1024 + k / S : k;
 }
 
 // ------------------------------------------------------- kernel spectrum
@@ -541,7 +518,7 @@ k_rows_inv_split(const float2* X, int rows, float2* out, int n_out, const float2
 // and column transforms of N inputs, instead of M and M over an embedded
 // M x M array (embedding, rows and columns at M = 1024, N = 512: 34 -> 25 us).
 
-// Rows u of G's half, conjugated, at v mod M: T[u][ky] to X[u * M + ky].
+// Rows u of G's half, conjugated, at v mod M: T[u][ky] to X[u * M + split_pos(ky)].
 template <int MC>
 __global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict__ G, int N, float2* X, FftPlan fp,
                                                         const float2* __restrict__ tw, int rpc)
@@ -565,12 +542,13 @@ __global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict
     float2* res = fft_block<MC, false>(a, b, fp, rpc, ld, tw);
     for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
         const int q = e / M, m = e - q * M;
-        X[(int64_t)(u0 + q) * M + m] = res[q * ld + sidx<MC>(m)];
+        X[(int64_t)(u0 + q) * M + split_pos<MC>(m)] = res[q * ld + sidx<MC>(m)];
     }
 }
 
 // Column transforms of X (rows u < N) and the real spectrum: to
-// out[kx * M + ky] (Chat), or out[ky * M + kx] (ROWS_KY).
+// out[kx * M + ky], both by split_pos (Chat), or out[ky * M + kx] (ROWS_KY, the
+// caller's grid when it is not a power of two).
 template <int MC, bool ROWS_KY>
 __global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* __restrict__ X, int N, FftPlan fp, const float2* __restrict__ tw,
                                 float* out, int cpc)
@@ -597,13 +575,16 @@ __global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* __restrict
     for (int e = threadIdx.x; e < nc * M; e += blockDim.x) {
         const int cc = ROWS_KY ? e / M : e % nc, kx = ROWS_KY ? e - cc * M : e / nc;
         const float v = res[cc * ld + sidx<MC>(kx)].x * inv;
-        out[ROWS_KY ? (int64_t)(x0 + cc) * M + kx : (int64_t)kx * M + x0 + cc] = v;
+        out[ROWS_KY ? (int64_t)(x0 + cc) * M + kx : (int64_t)split_pos<MC>(kx) * M + x0 + cc] = v;
     }
 }
 
 // ------------------------------------------------------------- launch shapes
 
 constexpr int kFftSmemCap = 200 * 1024;
+
+// Rows of X at M >= 2048 (the split passes): N rounded up to even.
+int split_ld(int N) { return (N + 1) & ~1; }
 
 struct Shape {
     int per_cta;  // rows or columns per CTA
@@ -643,14 +624,9 @@ template <int MC>
 int set_attrs()
 {
     const int bytes = kFftSmemCap;
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd<MC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd<MC, 1, SPIREC_PHI_HUBER>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd<MC, 1, SPIREC_PHI_HYPERBOLIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd<MC, 1, SPIREC_PHI_QUADRATIC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv<MC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     SPIREC_CK(cudaFuncSetAttribute(k_cols_filter<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     SPIREC_CK(cudaFuncSetAttribute(k_rows_spectrum<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     SPIREC_CK(cudaFuncSetAttribute(k_cols_spectrum<MC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -659,18 +635,13 @@ int set_attrs()
 }
 
 template <int S>
-int set_split_row_attrs()
+int set_split_attrs()
 {
-    const int fb = (int)rows_split_smem<S, true>(), ib = (int)rows_split_smem<S, false>();
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd_split<S, 0, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, fb));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd_split<S, 1, SPIREC_PHI_HUBER>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, fb));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd_split<S, 1, SPIREC_PHI_HYPERBOLIC>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, fb));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd_split<S, 1, SPIREC_PHI_QUADRATIC>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, fb));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv_split<S, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, ib));
-    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv_split<S, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, ib));
+    const int bytes = (int)sizeof(SplitSmem);
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_fwd_split<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StagedSmem)));
+    SPIREC_CK(cudaFuncSetAttribute(k_cols_split<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StagedSmem)));
+    SPIREC_CK(cudaFuncSetAttribute(k_cols_split<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StagedSmem)));
+    SPIREC_CK(cudaFuncSetAttribute(k_rows_inv_split<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     return SPIREC_OK;
 }
 
@@ -695,63 +666,38 @@ int with_size(int M, F&& f)
 
 bool is_pow2_specialised(int M) { return M >= 16 && M <= 4096 && (M & (M - 1)) == 0; }
 
-CgPass plain_pass(spirec_plan p, int slot, unsigned* counter)
-{
-    CgPass c{};
-    c.parts = reinterpret_cast<float2*>(p->part) + (size_t)slot * kMaxParts;
-    c.counter = counter;
-    c.scal = p->scal;
-    c.reg = p->reg;
-    return c;
-}
-
 struct AttrAll {
     template <int MC>
     int operator()() { return MC > 0 ? set_attrs<MC>() : SPIREC_OK; }
 };
 
+// Grid of a split pass over `items` rows or columns, `per` a block.
+int split_grid(int items, int per, int* grid)
+{
+    int sms = 0;
+    if (device_sms(&sms) != SPIREC_OK) return SPIREC_ECUDA;
+    const int groups = (items + per - 1) / per, cap = kSplitCtasPerSm * sms;
+    *grid = groups < cap ? groups : cap;
+    return SPIREC_OK;
+}
+
 struct LaunchRowsFwd {
     spirec_plan p;
     const float2* in;
-    int ld_in, n_in, rows, mode, blocks;
-    Shape s;
-    CgPass c;
-    int split_grid;  // CTAs of the split passes (M = 2048, 4096): two an SM
-    template <int S, int MODE, int KIND>
-    void split(int grid)
-    {
-        k_rows_fwd_split<S, MODE, KIND><<<grid, kSplitThreads, rows_split_smem<S, true>(), p->stream>>>(
-            in, ld_in, n_in, rows, p->X, p->twiddle, c);
-    }
     template <int MC>
     int operator()()
     {
-        if constexpr (MC == 2048 || MC == 4096) {
+        const int N = p->N;
+        if constexpr (MC >= 2048) {
             constexpr int S = MC / 1024;
-            if (2 * n_in <= MC) {
-                const int groups = (rows + kSplitWarps / S - 1) / (kSplitWarps / S);
-                const int grid = groups < split_grid ? groups : split_grid;
-                if (mode == 0) split<S, 0, -1>(grid);
-                else if (c.reg.kind == SPIREC_PHI_HUBER) split<S, 1, SPIREC_PHI_HUBER>(grid);
-                else if (c.reg.kind == SPIREC_PHI_HYPERBOLIC) split<S, 1, SPIREC_PHI_HYPERBOLIC>(grid);
-                else split<S, 1, SPIREC_PHI_QUADRATIC>(grid);
-                SPIREC_CK(cudaGetLastError());
-                p->launches += 1;
-                return SPIREC_OK;
-            }
+            int grid = 0, rc;
+            if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
+            k_rows_fwd_split<S><<<grid, kSplitThreads, sizeof(StagedSmem), p->stream>>>(in, N, p->X, split_ld(N), p->twiddle);
+        } else {
+            const Shape s = row_shape(p->MF, MC > 0);
+            k_rows_fwd<MC><<<(N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+                in, N, N, N, p->X, p->fft, p->twiddle, s.per_cta);
         }
-        if (mode == 0)
-            k_rows_fwd<MC, 0><<<blocks, s.threads, s.smem, p->stream>>>(in, ld_in, n_in, rows, p->X, p->fft,
-                                                                        p->twiddle, s.per_cta, c);
-        else if (c.reg.kind == SPIREC_PHI_HUBER)  // phi fixed at compile time in the line-search sums
-            k_rows_fwd<MC, 1, SPIREC_PHI_HUBER><<<blocks, s.threads, s.smem, p->stream>>>(
-                in, ld_in, n_in, rows, p->X, p->fft, p->twiddle, s.per_cta, c);
-        else if (c.reg.kind == SPIREC_PHI_HYPERBOLIC)
-            k_rows_fwd<MC, 1, SPIREC_PHI_HYPERBOLIC><<<blocks, s.threads, s.smem, p->stream>>>(
-                in, ld_in, n_in, rows, p->X, p->fft, p->twiddle, s.per_cta, c);
-        else
-            k_rows_fwd<MC, 1, SPIREC_PHI_QUADRATIC><<<blocks, s.threads, s.smem, p->stream>>>(
-                in, ld_in, n_in, rows, p->X, p->fft, p->twiddle, s.per_cta, c);
         SPIREC_CK(cudaGetLastError());
         p->launches += 1;
         return SPIREC_OK;
@@ -760,27 +706,23 @@ struct LaunchRowsFwd {
 
 struct LaunchCols {
     spirec_plan p;
-    int n_in, n_out, blocks;
-    Shape s;
+    const CgPass* cg;
     template <int MC>
     int operator()()
     {
-        if constexpr (MC == 2048 || MC == 4096) {
+        const int N = p->N;
+        if constexpr (MC >= 2048) {
             constexpr int S = MC / 1024;
-            if (2 * n_in <= MC && 2 * n_out <= MC) {
-                int sms = 0;
-                if (device_sms(&sms) != SPIREC_OK) return SPIREC_ECUDA;
-                const int groups = MC / (kSplitWarps / S);
-                const int cap = kSplitColCtasPerSm * sms;
-                k_cols_split<S><<<groups < cap ? groups : cap, kSplitThreads, cols_split_smem<S>(), p->stream>>>(
-                    p->X, n_in, n_out, p->twiddle, p->Chat);
-                SPIREC_CK(cudaGetLastError());
-                p->launches += 1;
-                return SPIREC_OK;
-            }
+            int grid = 0, rc;
+            if ((rc = split_grid(MC / 2, kSplitWarps / (2 * S), &grid)) != SPIREC_OK) return rc;
+            auto kern = cg ? k_cols_split<S, true> : k_cols_split<S, false>;
+            kern<<<grid, kSplitThreads, sizeof(StagedSmem), p->stream>>>(p->X, N, split_ld(N), p->twiddle, p->Chat,
+                                                                        cg ? *cg : CgPass{});
+        } else {
+            const Shape s = col_shape(p->MF, MC > 0);
+            k_cols_filter<MC><<<(p->MF + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+                p->X, N, N, p->fft, p->twiddle, p->Chat, s.per_cta);
         }
-        k_cols_filter<MC><<<blocks, s.threads, s.smem, p->stream>>>(p->X, n_in, n_out, p->fft, p->twiddle,
-                                                                    p->Chat, s.per_cta);
         SPIREC_CK(cudaGetLastError());
         p->launches += 1;
         return SPIREC_OK;
@@ -790,37 +732,23 @@ struct LaunchCols {
 struct LaunchRowsInv {
     spirec_plan p;
     float2* out;
-    int mode;
-    const float2* dotx;
-    int dot_scalar, blocks;
-    Shape s;
-    CgPass c;
-    int split_grid;
+    const float2* x;
+    const CgPass* cg;
     template <int MC>
     int operator()()
     {
-        if constexpr (MC == 2048 || MC == 4096) {
+        const int N = p->N;
+        if constexpr (MC >= 2048) {
             constexpr int S = MC / 1024;
-            if (2 * p->N <= MC) {
-                const int groups = (p->N + kSplitWarps / S - 1) / (kSplitWarps / S);
-                const int grid = groups < split_grid ? groups : split_grid;
-                if (mode == 0)
-                    k_rows_inv_split<S, 0><<<grid, kSplitThreads, rows_split_smem<S, false>(), p->stream>>>(
-                        p->X, p->N, out, p->N, p->twiddle, dotx, c, dot_scalar);
-                else
-                    k_rows_inv_split<S, 1><<<grid, kSplitThreads, rows_split_smem<S, false>(), p->stream>>>(
-                        p->X, p->N, out, p->N, p->twiddle, dotx, c, dot_scalar);
-                SPIREC_CK(cudaGetLastError());
-                p->launches += 1;
-                return SPIREC_OK;
-            }
+            int grid = 0, rc;
+            if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
+            k_rows_inv_split<S><<<grid, kSplitThreads, sizeof(SplitSmem), p->stream>>>(p->X, N, split_ld(N), out, p->twiddle);
+        } else {
+            const Shape s = row_shape(p->MF, MC > 0);
+            auto kern = cg ? k_rows_inv<MC, true> : k_rows_inv<MC, false>;
+            kern<<<(N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+                p->X, N, out, N, p->fft, p->twiddle, s.per_cta, cg ? x : nullptr, cg ? *cg : CgPass{});
         }
-        if (mode == 0)
-            k_rows_inv<MC, 0><<<blocks, s.threads, s.smem, p->stream>>>(p->X, p->N, out, p->N, p->fft,
-                                                                        p->twiddle, s.per_cta, dotx, c, dot_scalar);
-        else
-            k_rows_inv<MC, 1><<<blocks, s.threads, s.smem, p->stream>>>(p->X, p->N, out, p->N, p->fft,
-                                                                        p->twiddle, s.per_cta, dotx, c, dot_scalar);
         SPIREC_CK(cudaGetLastError());
         p->launches += 1;
         return SPIREC_OK;
@@ -854,7 +782,8 @@ struct LaunchSpectrum {
     }
 };
 
-// out[e'] of the transposed real in[e] (M x M)
+// out[ky * M + kx] = Chat[kx][ky] for a power-of-two M (the caller's layout).
+template <int MC>
 __global__ void __launch_bounds__(256) k_transpose_real(const float* __restrict__ in, int M, float* __restrict__ out)
 {
     __shared__ float tile[32][33];
@@ -862,16 +791,30 @@ __global__ void __launch_bounds__(256) k_transpose_real(const float* __restrict_
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int x = x0 + tx, y = y0 + ty + 8 * k;
-        if (x < M && y < M) tile[ty + 8 * k][tx] = __ldg(in + (int64_t)y * M + x);
+        const int ky = x0 + tx, kx = y0 + ty + 8 * k;
+        if (ky < M && kx < M) tile[ty + 8 * k][tx] = __ldg(in + (int64_t)split_pos<MC>(kx) * M + split_pos<MC>(ky));
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int x = x0 + ty + 8 * k, y = y0 + tx;
-        if (x < M && y < M) out[(int64_t)x * M + y] = tile[tx][ty + 8 * k];
+        const int ky = x0 + ty + 8 * k, kx = y0 + tx;
+        if (ky < M && kx < M) out[(int64_t)ky * M + kx] = tile[tx][ty + 8 * k];
     }
 }
+
+struct LaunchSpectrumOut {
+    spirec_plan p;
+    float* out;
+    template <int MC>
+    int operator()()
+    {
+        const unsigned t = (unsigned)((p->M + 31) / 32);
+        k_transpose_real<MC><<<dim3(t, t), dim3(32, 8), 0, p->stream>>>(p->Chat, p->M, out);
+        SPIREC_CK(cudaGetLastError());
+        p->launches += 1;
+        return SPIREC_OK;
+    }
+};
 
 }  // namespace
 
@@ -879,67 +822,22 @@ int fft_setup_attributes(int)
 {
     int rc;
     if ((rc = set_attrs<0>()) != SPIREC_OK) return rc;
-    SPIREC_CK(cudaFuncSetAttribute(k_cols_split<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)cols_split_smem<2>()));
-    SPIREC_CK(cudaFuncSetAttribute(k_cols_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)cols_split_smem<4>()));
-    if ((rc = set_split_row_attrs<2>()) != SPIREC_OK) return rc;
-    if ((rc = set_split_row_attrs<4>()) != SPIREC_OK) return rc;
+    if ((rc = set_split_attrs<2>()) != SPIREC_OK) return rc;
+    if ((rc = set_split_attrs<4>()) != SPIREC_OK) return rc;
     for (int M = 16; M <= 4096; M *= 2)
         if ((rc = with_size(M, AttrAll{})) != SPIREC_OK) return rc;
     return SPIREC_OK;
 }
 
-int launch_rows_fwd(spirec_plan p, const float2* in, int ld_in, int n_in, int rows, int mode,
-                    const CgPass* cg)
-{
-    const int M = p->MF;
-    const Shape s = row_shape(M, is_pow2_specialised(M));
-    const int blocks = (rows + s.per_cta - 1) / s.per_cta;
-    if (mode == 1 && blocks > kMaxParts) {
-        set_error("too many row blocks");
-        return SPIREC_EUNSUPPORTED;
-    }
-    const CgPass c = cg ? *cg : plain_pass(p, 0, nullptr);
-    int sms = 0;
-    if (device_sms(&sms) != SPIREC_OK) return SPIREC_ECUDA;
-    return with_size(M, LaunchRowsFwd{p, in, ld_in, n_in, rows, mode, blocks, s, c, kSplitCtasPerSm * sms});
-}
-
-int launch_cols(spirec_plan p, int n_in, int n_out)
-{
-    const int M = p->MF;
-    const Shape s = col_shape(M, is_pow2_specialised(M));
-    const int blocks = (M + s.per_cta - 1) / s.per_cta;
-    return with_size(M, LaunchCols{p, n_in, n_out, blocks, s});
-}
-
-int launch_rows_inv(spirec_plan p, float2* out, int mode, const float2* dotx, const CgPass* cg,
-                    int dot_scalar)
-{
-    const int M = p->MF, N = p->N;
-    const Shape s = row_shape(M, is_pow2_specialised(M));
-    const int blocks = (N + s.per_cta - 1) / s.per_cta;
-    if (dotx && blocks > kMaxParts) {
-        set_error("too many row blocks");
-        return SPIREC_EUNSUPPORTED;
-    }
-    const CgPass c = cg ? *cg : plain_pass(p, P_MISC, p->counters + C_MISC);
-    int sms = 0;
-    if (device_sms(&sms) != SPIREC_OK) return SPIREC_ECUDA;
-    return with_size(M, LaunchRowsInv{p, out, mode, dotx, dot_scalar, blocks, s, c, kSplitInvCtasPerSm * sms});
-}
-
-int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, int dot_scalar)
+int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, const CgPass* cg)
 {
     int rc;
-    const int N = p->N;
-    if ((rc = launch_rows_fwd(p, x, N, N, N, 0, nullptr)) != SPIREC_OK) return rc;
-    if ((rc = launch_cols(p, N, N)) != SPIREC_OK) return rc;
-    return launch_rows_inv(p, Tx, 0, dot_scalar >= 0 ? x : nullptr, nullptr, dot_scalar);
+    if ((rc = with_size(p->MF, LaunchRowsFwd{p, x})) != SPIREC_OK) return rc;
+    if ((rc = with_size(p->MF, LaunchCols{p, cg})) != SPIREC_OK) return rc;
+    return with_size(p->MF, LaunchRowsInv{p, Tx, x, cg});
 }
 
-// A power of two as it is; anything else (the 2^a 3^b 5^c grids a plan picks
+// A power of two from 64 on as it is; anything else (the 2^a 3^b 5^c grids a plan picks
 // by default among them) is embedded in the next power of two that holds the
 // lags: T is the same linear convolution on any grid of at least 2N - 1, and
 // the power-of-two passes are the faster ones at every N although the grid
@@ -952,8 +850,8 @@ int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, int dot_scalar)
 //   N = 1030, M = 2160 / 4096   250   / 169    342 / 227
 int fft_grid(int N, int M)
 {
-    if (is_pow2_specialised(M)) return M;
-    int g = 16;
+    if (M >= 64 && is_pow2_specialised(M)) return M;
+    int g = 64;  // the persistent loop's smallest
     while (g < 2 * N - 1) g *= 2;
     return g;
 }
@@ -964,6 +862,9 @@ int launch_spectrum(spirec_plan p)
     const bool pow2 = is_pow2_specialised(M);
     return with_size(M, LaunchSpectrum{p, &p->fft, p->twiddle, false, p->Chat, row_shape(M, pow2), col_shape(M, pow2)});
 }
+
+// Complex values of X.
+size_t x_elems(int N, int MF) { return (size_t)(MF >= 2048 ? split_ld(N) : N) * MF; }
 
 // Complex values of cwork: the N x M rows of a spectrum build on either grid,
 // and the persistent loop's split-order spectrum at MF = 1024 (k_chat_split).
@@ -980,11 +881,7 @@ int launch_spectrum_out(spirec_plan p, float* out)
         const bool pow2 = is_pow2_specialised(M);
         return with_size(M, LaunchSpectrum{p, &p->fft_M, p->twiddle_M, true, out, row_shape(M, pow2), col_shape(M, pow2)});
     }
-    const unsigned t = (unsigned)((p->M + 31) / 32);
-    k_transpose_real<<<dim3(t, t), dim3(32, 8), 0, p->stream>>>(p->Chat, p->M, out);
-    SPIREC_CK(cudaGetLastError());
-    p->launches += 1;
-    return SPIREC_OK;
+    return with_size(p->M, LaunchSpectrumOut{p, out});
 }
 
 }  // namespace spirec
@@ -1057,14 +954,12 @@ struct LaunchNoAlloc {
         const bool pow2 = MC > 0;
         const Shape rs = row_shape(M, pow2), cs = col_shape(M, pow2);
         const int rblocks = (N + rs.per_cta - 1) / rs.per_cta;
-        const CgPass c{};
-        k_rows_fwd<MC, 0><<<rblocks, rs.threads, rs.smem, st>>>(x, N, N, N, rows, fp, tw, rs.per_cta, c);
+        k_rows_fwd<MC><<<rblocks, rs.threads, rs.smem, st>>>(x, N, N, N, rows, fp, tw, rs.per_cta);
         SPIREC_CK(cudaGetLastError());
         k_cols_filter<MC><<<(M + cs.per_cta - 1) / cs.per_cta, cs.threads, cs.smem, st>>>(rows, N, N, fp, tw,
                                                                                           chat, cs.per_cta);
         SPIREC_CK(cudaGetLastError());
-        k_rows_inv<MC, 0><<<rblocks, rs.threads, rs.smem, st>>>(rows, N, Tx, N, fp, tw, rs.per_cta, nullptr,
-                                                                 c, 0);
+        k_rows_inv<MC, false><<<rblocks, rs.threads, rs.smem, st>>>(rows, N, Tx, N, fp, tw, rs.per_cta, nullptr, CgPass{});
         SPIREC_CK(cudaGetLastError());
         return SPIREC_OK;
     }

@@ -1,6 +1,6 @@
 // fft_device.cuh -- device code of the Toeplitz apply (see fft.cu for the
 // math): shared-memory Stockham FFTs and the per-group bodies of the three
-// passes, including the CG work fused into the row passes.  Used by the
+// passes.  Used by the
 // stand-alone pass kernels (fft.cu) and by the persistent CG loop
 // (cg_loop.cu).
 //
@@ -269,111 +269,38 @@ __device__ __forceinline__ float2 new_direction(float2 g, float2 dold, float bet
 
 // ------------------------------------------------------ row pass 1, a group
 
-// Rows [r0, r0 + rpc) (nr of them real).  MODE 0: the rows of `in` (n_in
-// nonzero entries, stride ld_in).  MODE 1 (CG): the rows of the new direction
-// d = -g + beta d_old, written to c.d_new, with the per-thread sums
-//   acc[0] += Re<d, 2 res>, res = T f - D             (q1)
-//   acc[1] += sum_e lambda b(|z_e|) Re(conj(z_e) w_e)  (h'(0) penalty part)
-//   acc[2] += sum_e lambda b(|z_e|) |w_e|^2            (curvature at t = 0)
-// over the right/down edges and pixels of these rows.  Then the FFTs and the
-// M outputs of each row into X.
-template <int MC, int MODE, int KIND = -1>
+// Rows [r0, r0 + rpc) (nr of them real) of `in` (n_in nonzero entries, stride
+// ld_in): the FFTs and the M outputs of each row into X.
+template <int MC>
 __device__ __forceinline__ void rows_fwd_group(const float2* in, int ld_in, int n_in, int r0, int nr,
                                                int rpc, float2* X, const FftPlan& fp,
-                                               const float2* __restrict__ tw, const CgPass& c,
-                                               float beta, bool restart, float2* a, float2* b,
-                                               float (&acc)[3])
+                                               const float2* __restrict__ tw, float2* a, float2* b)
 {
     const int M = fp.M;
     const int ld = seq_len<MC>(M);
-    const int N = n_in;
     if constexpr (MC > 0) {
         // rpc * M == 4 * blockDim.x: four elements per thread, loads first
-        float2 ga[4], gb[4];
-        bool live[4];
+        float2 v[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int e = threadIdx.x + i * blockDim.x;
             const int q = e / M, m = e - q * M;
-            live[i] = q < nr && m < N;
-            const int64_t o = live[i] ? (int64_t)(r0 + q) * ld_in + m : 0;
-            if (MODE == 0) {
-                ga[i] = live[i] ? __ldcg(in + o) : make_float2(0.f, 0.f);
-            } else {
-                ga[i] = live[i] ? __ldcg(c.g + o) : make_float2(0.f, 0.f);
-                gb[i] = live[i] ? __ldcg(c.d_old + o) : make_float2(0.f, 0.f);
-            }
+            v[i] = q < nr && m < n_in ? __ldcg(in + (int64_t)(r0 + q) * ld_in + m) : make_float2(0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int e = threadIdx.x + i * blockDim.x;
             const int q = e / M, m = e - q * M;
-            float2 v = make_float2(0.f, 0.f);
-            if (live[i]) {
-                if (MODE == 0) {
-                    v = ga[i];
-                } else {
-                    v = new_direction(ga[i], gb[i], beta, restart);
-                    c.d_new[(int64_t)(r0 + q) * ld_in + m] = v;
-                }
-            }
-            a[q * ld + sidx<MC>(m)] = v;
+            a[q * ld + sidx<MC>(m)] = v[i];
         }
     } else {
         for (int e = threadIdx.x; e < rpc * M; e += blockDim.x) {
             const int q = e / M, m = e - q * M;
-            float2 v = make_float2(0.f, 0.f);
-            if (q < nr && m < N) {
-                const int64_t o = (int64_t)(r0 + q) * ld_in + m;
-                if (MODE == 0) {
-                    v = __ldcg(in + o);
-                } else {
-                    v = new_direction(__ldcg(c.g + o), __ldcg(c.d_old + o), beta, restart);
-                    c.d_new[o] = v;
-                }
-            }
-            a[q * ld + sidx<MC>(m)] = v;
+            a[q * ld + sidx<MC>(m)] =
+                q < nr && m < n_in ? __ldcg(in + (int64_t)(r0 + q) * ld_in + m) : make_float2(0.f, 0.f);
         }
     }
     __syncthreads();
-    if (MODE == 1) {
-        const Reg reg = c.reg;
-#pragma unroll 2
-        for (int e = threadIdx.x; e < nr * N; e += blockDim.x) {            const int q = e / N, m = e - q * N;
-            const int n = r0 + q;
-            const int64_t o = (int64_t)n * N + m;
-            const bool has_r = m + 1 < N, has_d = n + 1 < N;
-            const int64_t od = has_d ? o + N : o;
-            // every load first (clamped neighbours, masked contributions)
-            const float2 dn = a[q * ld + sidx<MC>(m)];
-            const float2 dr = a[q * ld + sidx<MC>(has_r ? m + 1 : m)];
-            const float2 fp_ = __ldcg(c.f + o), fr = __ldcg(c.f + (has_r ? o + 1 : o)), fd = __ldcg(c.f + od);
-            const float2 gd = __ldcg(c.g + od), dold_d = __ldcg(c.d_old + od);
-            acc[0] += 2.f * redot(dn, __ldcg(c.res + o));
-            if (reg.lambda1 != 0.f) {
-                {
-                    const float2 w = f2sub(dr, dn);
-                    const float2 z = f2sub(fr, fp_);
-                    const float bw = has_r ? reg.lambda1 * phi_weight_k<KIND>(reg.kind, reg.alpha1, redot(z, z)) : 0.f;
-                    acc[1] = fmaf(bw, redot(z, w), acc[1]);
-                    acc[2] = fmaf(bw, redot(w, w), acc[2]);
-                }
-                {
-                    const float2 dd = new_direction(gd, dold_d, beta, restart);
-                    const float2 w = f2sub(dd, dn);
-                    const float2 z = f2sub(fd, fp_);
-                    const float bw = has_d ? reg.lambda1 * phi_weight_k<KIND>(reg.kind, reg.alpha1, redot(z, z)) : 0.f;
-                    acc[1] = fmaf(bw, redot(z, w), acc[1]);
-                    acc[2] = fmaf(bw, redot(w, w), acc[2]);
-                }
-            }
-            if (reg.lambda0 != 0.f) {
-                const float bw = reg.lambda0 * phi_weight_k<KIND>(reg.kind, reg.alpha0, redot(fp_, fp_));
-                acc[1] = fmaf(bw, redot(fp_, dn), acc[1]);
-                acc[2] = fmaf(bw, redot(dn, dn), acc[2]);
-            }
-        }
-    }
     float2* res = fft_block<MC, false>(a, b, fp, rpc, ld, tw);
     for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
         const int q = e / M, m = e - q * M;

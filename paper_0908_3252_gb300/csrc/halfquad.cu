@@ -374,7 +374,7 @@ int hq_outer_step(spirec_plan p, int k, double* Jdev)
     p->launches += 1;
     for (int j = 0; j < p->hq_inner; ++j) {
         rc = p->mode == SPIREC_MODE_DIRECT ? launch_normal_direct(p, pv, p->Td, false)
-                                           : launch_toeplitz(p, pv, p->Td, -1);
+                                           : launch_toeplitz(p, pv, p->Td);
         if (rc != SPIREC_OK) return rc;
         k_hq_apply<false><<<blocks, kVecThreads, 0, p->stream>>>(pv, p->Td, W, nullptr, N, p->tmp, slot(p, P_UPD),
                                                                  p->counters + C_UPD, p->scal);
@@ -405,7 +405,7 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev)
     p->launches += 1;
     for (int j = 0; j < p->hq_inner; ++j) {
         rc = p->mode == SPIREC_MODE_DIRECT ? launch_normal_direct(p, pv, p->Td, false)
-                                           : launch_toeplitz(p, pv, p->Td, -1);
+                                           : launch_toeplitz(p, pv, p->Td);
         if (rc != SPIREC_OK) return rc;
         k_hq_apply<true><<<blocks, kVecThreads, 0, p->stream>>>(pv, p->Td, W, f, N, p->tmp, slot(p, P_UPD),
                                                                 p->counters + C_UPD, p->scal);

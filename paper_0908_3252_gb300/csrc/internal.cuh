@@ -37,8 +37,8 @@ bool make_fft_plan(int M, FftPlan* p);
 // one per block of the kernel that produced them).
 constexpr int kMaxParts = 4096;
 enum PartSlot {
-    P_ROWA = 0,   // row pass 1 of the CG: q1, num0, den0 (3 slots)
-    P_ROWC = 3,   // row pass 3: q2 (or a plain dot)
+    P_ROWA = 0,   // direction of the CG: q1, num0, den0 (3 slots)
+    P_ROWC = 3,   // Toeplitz apply: q2
     P_LS = 4,     // line-search step: num, den (2 slots)
     P_UPD = 6,    // gradient/update: 6 slots (see k_update)
     P_MISC = 12,  // one-off sums (2 slots)
@@ -83,15 +83,8 @@ struct Reg {
     int kind;
 };
 
-// Pointers of the fused CG passes (row pass 1 and 3 of the Toeplitz apply).
+// Where a Toeplitz apply of the CG puts its grid sum and scalars.
 struct CgPass {
-    const float2* g;
-    const float2* d_old;
-    float2* d_new;
-    const float2* f;
-    const float2* res;  // T f - D, the data term's image-domain residual
-    const float2* D;
-    Reg reg;
     float2* parts;
     unsigned* counter;
     double* scal;
@@ -136,7 +129,7 @@ struct spirec_plan_s {
     float2* G;     // N x (2N-1)
     float* Chat;   // MF x MF real, transposed: Chat[kx*MF + ky]
     float2* cwork; // cwork_elems: rows of the spectrum builds, the loop's split-order spectrum
-    float2* X;     // N x MF complex (Toeplitz rows)
+    float2* X;     // x_elems: N x MF complex (Toeplitz rows; by columns at MF >= 2048)
     float2* D;     // N x N
     float2* s;     // L (+32 padding)
     float2* ystage;  // L (+32 padding): a caller's y staged for the tensor-core adjoint
@@ -203,19 +196,13 @@ int launch_spectrum_out(spirec_plan p, float* out);
 // The grid side the transforms of an N x N image on the caller's grid M use.
 int fft_grid(int N, int M);
 size_t cwork_elems(int N, int M, int MF);
+size_t x_elems(int N, int MF);
 int launch_adjoint(spirec_plan p, const float2* y, float2* x);  // x = H^H y
 int launch_forward(spirec_plan p, const float2* x, float2* y);  // y = H x
 
-// Toeplitz T x -> Tx; with dot_scalar >= 0 also scal[dot_scalar] = Re<x, Tx>.
-int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, int dot_scalar);
+// Toeplitz T x -> Tx; with cg also q2 = Re<x, T x> and the first line-search step.
+int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, const CgPass* cg = nullptr);
 int fft_setup_attributes(int maxM);
-// Toeplitz passes; mode 1 = the fused CG forms (see fft.cu).
-int launch_rows_fwd(spirec_plan p, const float2* in, int ld_in, int n_in, int rows, int mode,
-                    const CgPass* cg);
-int launch_cols(spirec_plan p, int n_in, int n_out);
-int launch_rows_inv(spirec_plan p, float2* out, int mode, const float2* dotx, const CgPass* cg,
-                    int dot_scalar);
-
 // CG pieces (cg.cu).  Iteration k reads f[k & 1] and writes f[(k + 1) & 1].
 int launch_data_norm(spirec_plan p);
 // res = Tx - D where res holds T x (have_tx), else res = -D (x = 0)
@@ -237,7 +224,7 @@ int hq_outer_step(spirec_plan p, int k, double* Jdev);
 // Jdev[k], hq_inner CG steps on the Newton system, the line search, the step).
 int nt_outer_step(spirec_plan p, int k, double* Jdev);
 // The whole loop (first gradient + iters iterations) as one persistent
-// cooperative kernel (cg_loop.cu); power-of-two M in [64, 2048] only, and
+// cooperative kernel (cg_loop.cu); MF in [64, 1024] only, and
 // SPIREC_EUNSUPPORTED (nothing enqueued) when the image does not fit its
 // shared-memory caches.  The iterate ends in f[0].
 bool loop_supported(int M);

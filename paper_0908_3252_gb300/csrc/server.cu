@@ -104,7 +104,7 @@ size_t plan_bytes(int N, int64_t L, int M, int precision)
     b += (size_t)N * (2 * N - 1) * 8;            // G
     const size_t MF = (size_t)fft_grid(N, M);
     b += MF * MF * 4 + cwork_elems(N, M, (int)MF) * 8;  // spectrum + work
-    b += (size_t)N * MF * 8;                     // rows
+    b += x_elems(N, (int)MF) * 8;                // rows
     b += 3 * ((size_t)L + 32) * 8;               // data, its staging, the host upload buffer
     b += 10 * NN * 8;                            // iterates, directions, gradients, D, scratch
     b += (MF + M) * 8 + (size_t)P_NSLOTS * kMaxParts * 8 + 4096;

@@ -128,3 +128,28 @@ def test_spectrum_and_toeplitz_grids(sp, N, M):
         if N <= 512 and p.M <= 1024:
             sp.spirec_toeplitz_noalloc(to_dev(x), C, Tx, N, p.M, _stream())
             assert rel(from_dev(Tx), TC.toeplitz_apply(want, x)) < 1e-5
+
+
+# T on the grids of 2048 and 4096 points (rows and columns split into warp-sized
+# transforms, two rows and two columns a sector): odd and even sides, the last
+# rows of a block missing, rows that do not start on 16 bytes, sides up to the
+# grid's largest.  G by matrix products in 64 bits.
+@pytest.mark.parametrize("N,M", [(3, 2048), (6, 4096), (515, 0), (1023, 0), (1024, 0), (1025, 0), (1030, 0), (2047, 0)])
+def test_toeplitz_large_grids(sp, N, M):
+    import torch
+    from oracle import factored as F
+    from oracle import toeplitz_cpu as TC
+    g = synth.rng(N)
+    kx, ky = synth.uniform_k(40, g)
+    x = c64(synth.complex_normal((N, N), g))
+    with sp.Plan(N, 40, M, 0, _stream(), kx, ky) as p:
+        buf = torch.zeros(N * N + 1, dtype=torch.complex64, device="cuda")
+        Mp = max(1 << (2 * N - 1).bit_length(), M)
+        want = TC.toeplitz_apply(TC.kernel_spectrum(F.gram(kx, ky, N), N, Mp), x)
+        for shift in (0, 1):  # the second input starts 8 bytes past a 16-byte boundary
+            xd = buf[shift:shift + N * N].view(N, N)
+            xd.copy_(to_dev(x))
+            Tx = empty_c64((N, N))
+            sp.spirec_toeplitz_dev(p.h, xd, Tx)
+            sp.spirec_sync(p.h)
+            assert rel(from_dev(Tx), want) < 1e-5
