@@ -135,12 +135,11 @@ struct Geo {
     static constexpr int TW = TW_R4 + (FOURSTEP ? 1024 : 0);
 };
 
-// dynamic shared memory of a block owning RB rows of an N-wide image: the
-// FFT buffer, the staged twiddle table, the row caches
+// dynamic shared memory of one of `grid` blocks owning RB rows of an N-wide
+// image each: the FFT buffer, the staged twiddle table, the row caches
 template <int MC>
-size_t loop_smem(int N, int RB)
+size_t loop_smem(int N, int RB, size_t grid)
 {
-    const size_t grid = (size_t)((N + RB - 1) / RB);
     // FFT buffer, twiddles, f and d of RB + 2 rows, T f - D, D, g, T d of RB rows,
     // and the deferred update partials (kUpdVals x even (grid + 1), and one
     // float2 to align them to 16 bytes)
@@ -889,7 +888,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
     const int N = A.N, RB = A.RB;
     Rows R;
     R.N = N;
-    R.R0 = blockIdx.x * RB;
+    R.R0 = min((int)blockIdx.x * RB, N);  // a block past the rows (nown = 0) only works in the column pass
     R.nown = min(RB, N - R.R0);
     R.hlo = R.R0 > 0 ? R.R0 - 1 : R.R0;
     R.hhi = min(R.R0 + R.nown, N - 1);
@@ -1131,13 +1130,33 @@ bool loop_cap(size_t* cap_out)
     return true;
 }
 
-// Whether blocks of RB rows fit: shared memory within the cap and every
-// block of the grid co-resident (the grid synchronisations need that).
+// Columns of a group of the column pass, and their number.
 template <int MC>
-bool loop_fits(int N, int RB, size_t cap, int sms, int* grid_out, size_t* smem_out)
+constexpr int loop_col_groups() { return MC / (Geo<MC>::FOURSTEP ? Geo<MC>::FS_COLS : Geo<MC>::CPC); }
+
+// Rows per block of the i-th shape, i < kMaxGroupsPerBlock: whole row-FFT
+// groups, or at M = 1024, whose row FFTs take two warps a row, any number.
+template <int MC>
+int loop_rb(int i)
 {
-    const int grid = (N + RB - 1) / RB;
-    const size_t smem = loop_smem<MC>(N, RB);
+    constexpr int split[kMaxGroupsPerBlock] = {1, 2, 3, 4, 6, 8, 12, 16};
+    return Geo<MC>::FOURSTEP ? split[i] : (i + 1) * Geo<MC>::RPC;
+}
+
+// Whether blocks of RB rows fit: shared memory within the cap and every block
+// of the grid co-resident (the grid synchronisations need that).  With `wide`
+// the grid has a block for every column group too, as far as they fit: blocks
+// beyond the rows only work in the column pass, which otherwise takes two
+// rounds where there are fewer row blocks than column groups (N = 192, M =
+// 512, 48 row blocks for 64 groups: column pass 12.1 -> 6.2 us, an iteration 30.0 ->
+// 24.3; N = 384, M = 1024, 96 of 128 and rows of 4 or 3 a block: 30.0 -> 23.8).
+template <int MC>
+bool loop_fits(int N, int RB, size_t cap, int sms, bool wide, int* grid_out, size_t* smem_out)
+{
+    int grid = (N + RB - 1) / RB;
+    const int groups = loop_col_groups<MC>();
+    if (wide && grid < groups) grid = groups < sms ? groups : (grid < sms ? sms : grid);
+    const size_t smem = loop_smem<MC>(N, RB, (size_t)grid);
     if (smem > cap) return false;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_loop<MC>, kLoopThreads, smem) != cudaSuccess)
@@ -1148,24 +1167,18 @@ bool loop_fits(int N, int RB, size_t cap, int sms, int* grid_out, size_t* smem_o
     return true;
 }
 
-// The shapes RB = gpb * RPC, gpb = 1 .. kMaxGroupsPerBlock (up to the first
-// that holds the whole image), that fit; at most max.
+// The shapes loop_rb(0), loop_rb(1), ... (up to the first that holds the whole
+// image) that fit; at most max.  The first has a block for every column group.
 template <int MC>
-int loop_shapes(int N, int* RB, int* grid, int max)
+int loop_shapes(int N, int* RB, int* grid, size_t* smem, int max)
 {
     int sms = 0;
     size_t cap = 0;
     if (device_sms(&sms) != SPIREC_OK || !loop_cap<MC>(&cap)) return 0;
     int n = 0;
-    for (int gpb = 1; gpb <= kMaxGroupsPerBlock && n < max; ++gpb) {
-        const int rb = gpb * Geo<MC>::RPC;
-        int gr = 0;
-        size_t smem = 0;
-        if (loop_fits<MC>(N, rb, cap, sms, &gr, &smem)) {
-            RB[n] = rb;
-            grid[n] = gr;
-            ++n;
-        }
+    for (int i = 0; i < kMaxGroupsPerBlock && n < max; ++i) {
+        const int rb = loop_rb<MC>(i);
+        if (loop_fits<MC>(N, rb, cap, sms, n == 0, &grid[n], &smem[n])) RB[n++] = rb;
         if (rb >= N) break;
     }
     cudaGetLastError();
@@ -1173,29 +1186,25 @@ int loop_shapes(int N, int* RB, int* grid, int max)
 }
 
 // The block shape of a launch: the tuned rows per block of the plan's shape
-// when that fits, else the fewest groups per block gpb whose grid is
-// co-resident (every block on its own SM when the image allows).
+// when that fits, else the first shape (every block on its own SM when the
+// image allows).
 template <int MC>
 bool loop_shape(const spirec_plan_s* p, int* RB_out, int* grid_out, size_t* smem_out)
 {
     int sms = 0;
     size_t cap = 0;
-    if (device_sms(&sms) != SPIREC_OK || !loop_cap<MC>(&cap)) return false;
     const int N = p->N;
+    if (device_sms(&sms) != SPIREC_OK || !loop_cap<MC>(&cap)) return false;
+    if (loop_shapes<MC>(N, RB_out, grid_out, smem_out, 1) != 1) return false;
     const int tuned = tune_lookup(SPIREC_KNOB_LOOP_ROWS, p, sms);
-    if (tuned > 0 && loop_fits<MC>(N, tuned, cap, sms, grid_out, smem_out)) {
+    int grid = 0;
+    size_t smem = 0;
+    if (tuned > 0 && tuned != *RB_out && loop_fits<MC>(N, tuned, cap, sms, false, &grid, &smem)) {
         *RB_out = tuned;
-        return true;
+        *grid_out = grid;
+        *smem_out = smem;
     }
-    for (int gpb = 1; gpb <= kMaxGroupsPerBlock; ++gpb) {
-        const int RB = gpb * Geo<MC>::RPC;
-        if (loop_fits<MC>(N, RB, cap, sms, grid_out, smem_out)) {
-            *RB_out = RB;
-            return true;
-        }
-        if (RB >= N) return false;
-    }
-    return false;
+    return true;
 }
 
 // The spectrum in the split order of the M = 1024 column pass:
@@ -1299,7 +1308,8 @@ struct Shapes {
                 }
                 return 1;
             }
-            return loop_shapes<MC>(p->N, RB, grid, max);
+            size_t smem[kMaxGroupsPerBlock];
+            return loop_shapes<MC>(p->N, RB, grid, smem, max < kMaxGroupsPerBlock ? max : kMaxGroupsPerBlock);
         }
     }
 };

@@ -153,3 +153,23 @@ def test_toeplitz_large_grids(sp, N, M):
             sp.spirec_toeplitz_dev(p.h, xd, Tx)
             sp.spirec_sync(p.h)
             assert rel(from_dev(Tx), want) < 1e-5
+
+
+# The persistent loop with blocks beyond the rows (fewer row blocks than column
+# groups), with one row a block and with a last block of fewer rows, against
+# the kernel graph of the same plan's penalty and data (three iterations: the
+# FP32 rounding model's distance is below 1e-6, G and D are the same).
+@pytest.mark.parametrize("N,M", [(33, 0), (40, 128), (66, 0), (100, 256), (130, 0), (150, 1024), (200, 0), (260, 0), (303, 0),
+                                 (400, 0)])
+def test_loop_grids(sp, monkeypatch, N, M):
+    g = synth.rng(N)
+    kx, ky = synth.spiral(N, 4, 700, "variable")
+    s = synth.complex_normal(kx.shape[0], g).astype(np.complex64)
+    x0 = synth.complex_normal((N, N), g).astype(np.complex64)
+    with sp.Plan(N, kx.shape[0], M, 1, _stream(), kx, ky) as p:
+        sp.spirec_set_data(p.h, s)
+        sp.spirec_set_reg(p.h, 0.05, 0.05, 0.02, 0.1, 0)
+        x, J = sp.spirec_solve(p.h, x0, 3, N)
+        monkeypatch.setenv("SPIREC_NO_LOOP", "1")
+        y, Jy = sp.spirec_solve(p.h, x0, 3, N)
+    assert rel(x, y) < 1e-5 and rel(J, Jy) < 1e-5
