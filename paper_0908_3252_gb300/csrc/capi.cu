@@ -407,7 +407,9 @@ bool solve_uses_loop(spirec_plan p)
            !getenv("SPIREC_NO_LOOP");
 }
 
-int solve_core(spirec_plan p, const float* x0, bool x0_dev, int iters)
+// The solve's work on the plan's stream.  The iterate ends in
+// p->f[p->result_slot], or, when out is given (device), in out.
+int solve_core(spirec_plan p, const float* x0, bool x0_dev, int iters, float* out)
 {
     if (!p->have_traj || !p->have_data) {
         set_error("solve needs a trajectory and data (spirec_set_trajectory, spirec_set_data)");
@@ -426,10 +428,30 @@ int solve_core(spirec_plan p, const float* x0, bool x0_dev, int iters)
     const size_t img = (size_t)p->N * p->N * sizeof(float2);
     cudaEvent_t e;
     if ((rc = tstart(p, 3, &e)) != SPIREC_OK) return rc;
+    // the result moves to `out` where the solve has not written it there
+    auto deliver = [&](const float2* from) -> int {
+        if (out) SPIREC_CK(cudaMemcpyAsync(out, from, img, cudaMemcpyDeviceToDevice, p->stream));
+        return tstop(p, e);
+    };
+    auto aligned = [](const void* q) { return ((uintptr_t)q & (sizeof(float2) - 1)) == 0; };
+    const bool in_place = x0 && x0_dev && aligned(x0);  // readable where it is
+    const float2* start = in_place ? reinterpret_cast<const float2*>(x0) : x0 ? p->f[0] : nullptr;
+    if (x0 && !in_place)
+        SPIREC_CK(cudaMemcpyAsync(p->f[0], x0, img, x0_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                  p->stream));
+    int RB = 0, grid = 0;
+    if (solve_uses_loop(p) && loop_current(p, &RB, &grid)) {
+        // first gradient and every iteration in one persistent kernel, from x0
+        // to out where they are
+        float2* to = out && aligned(out) ? reinterpret_cast<float2*>(out) : p->f[0];
+        p->result_slot = 0;
+        if (start && (rc = launch_toeplitz(p, start, p->res)) != SPIREC_OK) return rc;
+        if ((rc = launch_cg_loop(p, iters, start, to)) != SPIREC_OK) return rc;
+        return to == p->f[0] ? deliver(to) : tstop(p, e);
+    }
     const bool direct = p->mode == SPIREC_MODE_DIRECT;
+    if (in_place) SPIREC_CK(cudaMemcpyAsync(p->f[0], x0, img, cudaMemcpyDeviceToDevice, p->stream));
     if (x0) {
-        SPIREC_CK(cudaMemcpyAsync(p->f[0], x0, img,
-                                  x0_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, p->stream));
         if ((rc = direct ? launch_normal_direct(p, p->f[0], p->res, false) : launch_toeplitz(p, p->f[0], p->res)) !=
             SPIREC_OK)
             return rc;
@@ -443,24 +465,13 @@ int solve_core(spirec_plan p, const float* x0, bool x0_dev, int iters)
         p->result_slot = 0;
         rc = iters == 0 ? launch_hq_objective(p, p->Jdev) : run_iterations(p, iters);
         if (rc != SPIREC_OK) return rc;
-        return tstop(p, e);
+        return deliver(p->f[0]);
     }
-    rc = SPIREC_EUNSUPPORTED;
-    if (solve_uses_loop(p)) {
-        // first gradient and every iteration in one persistent kernel
-        rc = launch_cg_loop(p, iters);
-        if (rc != SPIREC_OK && rc != SPIREC_EUNSUPPORTED) return rc;
-        p->result_slot = 0;
-    }
-    if (rc == SPIREC_EUNSUPPORTED) {
-        p->result_slot = iters & 1;
-        // gradient at x0, J(x0), beta = 0 (the first direction is -g)
-        if ((rc = launch_update(p, p->f[0], p->f[0], p->dbuf[1], p->res, nullptr, p->g, 1, p->Jdev)) !=
-            SPIREC_OK)
-            return rc;
-        if ((rc = run_iterations(p, iters)) != SPIREC_OK) return rc;
-    }
-    return tstop(p, e);
+    p->result_slot = iters & 1;
+    // gradient at x0, J(x0), beta = 0 (the first direction is -g)
+    if ((rc = launch_update(p, p->f[0], p->f[0], p->dbuf[1], p->res, nullptr, p->g, 1, p->Jdev)) != SPIREC_OK) return rc;
+    if ((rc = run_iterations(p, iters)) != SPIREC_OK) return rc;
+    return deliver(p->f[p->result_slot]);
 }
 
 }  // namespace
@@ -613,7 +624,6 @@ int tune_loop(spirec_plan p, int objective, int iters, int sms, int* chosen, dou
     if ((rc = tune_store(SPIREC_KNOB_LOOP_ROWS, p, sms, 0)) != SPIREC_OK) return rc;
     int RB[8], grid[8];
     const int n = loop_candidates(p, RB, grid, 8);
-    const size_t img = (size_t)p->N * p->N * sizeof(float2);
     double best_score = 0.0;
     int best = 0;
     for (int i = 0; i < n; ++i) {
@@ -622,10 +632,7 @@ int tune_loop(spirec_plan p, int objective, int iters, int sms, int* chosen, dou
         rc = time_median(
             p,
             [&]() -> int {
-                SPIREC_CK(cudaMemsetAsync(p->f[0], 0, img, p->stream));
-                const int rc1 = launch_res_init(p, p->res, false);
-                if (rc1 != SPIREC_OK) return rc1;
-                return launch_cg_loop(p, iters);
+                return launch_cg_loop(p, iters, nullptr, p->f[0]);
             },
             &ms);
         if (rc != SPIREC_OK) return rc;
@@ -1147,7 +1154,7 @@ int spirec_solve(spirec_plan p, const float* x0, int32_t iters, float* x_out, do
         return SPIREC_EINVAL;
     }
     Join j(p);
-    if ((rc = solve_core(p, x0, false, iters)) != SPIREC_OK) return rc;
+    if ((rc = solve_core(p, x0, false, iters, nullptr)) != SPIREC_OK) return rc;
     // every copy enqueued (the last J and the error word into the pinned
     // words), then one synchronisation
     const size_t img = (size_t)p->N * p->N * sizeof(float2);
@@ -1172,9 +1179,7 @@ int spirec_solve(spirec_plan p, const float* x0, int32_t iters, float* x_out, do
 static int solve_dev_enqueue(spirec_plan p, const float* x0, int32_t iters, float* x_out, double* J_hist)
 {
     int rc;
-    if ((rc = solve_core(p, x0, true, iters)) != SPIREC_OK) return rc;
-    const size_t img = (size_t)p->N * p->N * sizeof(float2);
-    SPIREC_CK(cudaMemcpyAsync(x_out, p->f[p->result_slot], img, cudaMemcpyDeviceToDevice, p->stream));
+    if ((rc = solve_core(p, x0, true, iters, x_out)) != SPIREC_OK) return rc;
     if (J_hist)
         SPIREC_CK(cudaMemcpyAsync(J_hist, p->Jdev, sizeof(double) * (iters + 1), cudaMemcpyDeviceToDevice,
                                   p->stream));

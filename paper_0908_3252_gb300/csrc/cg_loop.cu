@@ -43,7 +43,9 @@
 // memory during the next column pass and summed, with J and beta formed, at
 // that pass's synchronisation (deferred_parts_fetch, deferred_parts_sum).
 //
-// Every grid synchronisation is a reduction over block partials behind an
+// Grids of at most 16 blocks (M <= 256) run as one thread-block cluster, whose
+// hardware barrier takes the place of the arrival counter.  Every other grid
+// synchronisation is a reduction over block partials behind an
 // arrival counter (see grid_reduce).  Its wait is bounded in time (the
 // launch's wait limit, 2 s unless a test sets it): on expiry the block raises
 // an abort word and an error bit, every block returns at its next
@@ -72,13 +74,13 @@ constexpr int kProf = 10;
 
 struct LoopArgs {
     int N, iters, RB;  // RB: rows owned per block
-    float2* f0;        // x0 in, the last iterate out
+    const float2* x0;  // start (null: zeros)
+    float2* out;       // the last iterate (may be x0: read before the first grid synchronisation)
     float2* g;         // gradient rows (halo exchange)
-    float2* res;       // T x0 - D in, T f - D out (the data term's residual)
+    float2* res;       // T x0 in (with x0), T f - D out (the data term's residual)
     const float2* D;
     float2* X;
-    const float* Chat;
-    const float* ChatS;  // M = 1024: Chat in the split order of the column pass
+    const float* Chat;  // at split_pos in both indices
     const float2* tw;
     FftPlan fp;
     Reg reg;
@@ -187,15 +189,51 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned* counter, unsigned tar
     }
 }
 
+// ------------------------------------------------ the same within one cluster
+//
+// A grid of at most kClusterMax blocks runs as one thread-block cluster (CL):
+// the synchronisation is the cluster's hardware barrier (release / acquire at
+// cluster scope, which also orders the blocks' global writes), and every block
+// stores its partials straight into the shared memory of all of them.  The
+// barrier needs no bound: a cluster's blocks are always resident together, and
+// they leave the loop together.
+
+constexpr int kClusterMax = 16;  // blocks of a cluster (more than 8 need the opt-in)
+constexpr int kPartSlots = 14;   // L_A .. L_E
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// v to the float2 at p (this block's shared memory) of block `rank`.
+__device__ __forceinline__ void store_remote(float2* p, int rank, float2 v)
+{
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\t"
+        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
+        "st.shared::cluster.v2.f32 [ra], {%2, %3};\n\t}" ::"r"((uint32_t)__cvta_generic_to_shared(p)),
+        "r"(rank), "f"(v.x), "f"(v.y)
+        : "memory");
+}
+
+// Where the partials of a synchronisation are.
+struct Sync {
+    float2* parts;       // global, P_NSLOTS x kMaxParts
+    float2* cparts;      // CL: shared, kPartSlots x kClusterMax
+    unsigned* counter;
+    unsigned* abort_word;
+    int* err;
+    unsigned long long limit_ns;
+};
+
 // The block's partials of K values to slot `slot` and the arrival: each
 // warp sums its lanes in FP32, then warp k sums value k over the warps in
 // float-float (the trees of block_partial) and stores it; thread 0 arrives
 // after a named barrier of those warps (its release covers their stores) and
 // waits.  S.ws is read only between this call's first and last barriers.
-template <int K>
-__device__ __forceinline__ void block_publish(float (&v)[K], float2* parts, int slot, unsigned seq, LoopShared& S,
-                                              unsigned* counter, unsigned* abort_word, int* err,
-                                              unsigned long long limit_ns)
+// CL: lane j of warp k stores the partial into block j, then the cluster's
+// barrier.
+template <bool CL, int K>
+__device__ __forceinline__ void block_publish(float (&v)[K], const Sync& y, int slot, unsigned seq, LoopShared& S)
 {
     static_assert(K >= 1 && K <= 8, "one warp per value");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -210,28 +248,51 @@ __device__ __forceinline__ void block_publish(float (&v)[K], float2* parts, int 
     if (warp < K) {
         const int nw = (blockDim.x + 31) >> 5;
         const FF bt = warp_sum_ff(FF{lane < nw ? S.ws[lane][warp] : 0.f, 0.f});
-        if (lane == 0) parts[(slot + warp) * kMaxParts + blockIdx.x] = make_float2(bt.hi, bt.lo);
-        if constexpr (K > 1) asm volatile("bar.sync 2, %0;" ::"r"(32 * K) : "memory");
-        if (threadIdx.x == 0) S.ok = grid_arrive_wait(counter, seq * gridDim.x, abort_word, err, limit_ns) ? 1 : 0;
+        if constexpr (CL) {
+            const float2 t = make_float2(__shfl_sync(0xffffffffu, bt.hi, 0), __shfl_sync(0xffffffffu, bt.lo, 0));
+            if (lane < (int)gridDim.x) store_remote(y.cparts + (slot + warp) * kClusterMax + blockIdx.x, lane, t);
+        } else {
+            if (lane == 0) y.parts[(slot + warp) * kMaxParts + blockIdx.x] = make_float2(bt.hi, bt.lo);
+            if constexpr (K > 1) asm volatile("bar.sync 2, %0;" ::"r"(32 * K) : "memory");
+            if (threadIdx.x == 0)
+                S.ok = grid_arrive_wait(y.counter, seq * gridDim.x, y.abort_word, y.err, y.limit_ns) ? 1 : 0;
+        }
     }
-    __syncthreads();
+    if constexpr (CL) {
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+}
+
+// The grid total of the value in `slot`, by one warp.
+template <bool CL>
+__device__ __forceinline__ FF warp_total(const Sync& y, int slot)
+{
+    if constexpr (CL) {
+        const int lane = threadIdx.x & 31;
+        const float2 v = lane < (int)gridDim.x ? y.cparts[slot * kClusterMax + lane] : make_float2(0.f, 0.f);
+        return warp_sum_ff(FF{v.x, v.y});
+    } else {
+        return warp_sum_parts(y.parts + slot * kMaxParts, gridDim.x);
+    }
 }
 
 // Block partials of K values to slot `slot`, the synchronisation, then the
 // grid totals as float-float pairs in S.redf, readable by every thread on
 // return.  seq counts the synchronisations of the launch (the same in every
 // thread).
-template <int K>
-__device__ __forceinline__ bool grid_reduce(float (&v)[K], float2* parts, int slot, unsigned& seq, LoopShared& S,
-                                            unsigned* counter, unsigned* abort_word, int* err,
-                                            unsigned long long limit_ns)
+template <bool CL, int K>
+__device__ __forceinline__ bool grid_reduce(float (&v)[K], const Sync& y, int slot, unsigned& seq, LoopShared& S)
 {
     ++seq;
-    block_publish<K>(v, parts, slot, seq, S, counter, abort_word, err, limit_ns);
-    if (!S.ok) return false;
+    block_publish<CL, K>(v, y, slot, seq, S);
+    if (!CL && !S.ok) return false;
     const int warp = threadIdx.x >> 5;
     if (warp < K) {
-        const FF a = warp_sum_parts(parts + (slot + warp) * kMaxParts, gridDim.x);
+        const FF a = warp_total<CL>(y, slot + warp);
         if ((threadIdx.x & 31) == 0) S.redf[warp] = a;
     }
     __syncthreads();
@@ -241,14 +302,12 @@ __device__ __forceinline__ bool grid_reduce(float (&v)[K], float2* parts, int sl
 // The first half of grid_reduce: the block partials to slot `slot` and the
 // synchronisation; the totals are formed later (deferred_parts_fetch /
 // deferred_parts_sum), off the critical path.
-template <int K>
-__device__ __forceinline__ bool grid_arrive_parts(float (&v)[K], float2* parts, int slot, unsigned& seq,
-                                                  LoopShared& S, unsigned* counter, unsigned* abort_word, int* err,
-                                                  unsigned long long limit_ns)
+template <bool CL, int K>
+__device__ __forceinline__ bool grid_arrive_parts(float (&v)[K], const Sync& y, int slot, unsigned& seq, LoopShared& S)
 {
     ++seq;
-    block_publish<K>(v, parts, slot, seq, S, counter, abort_word, err, limit_ns);
-    return S.ok != 0;
+    block_publish<CL, K>(v, y, slot, seq, S);
+    return CL || S.ok != 0;
 }
 
 // Copies the K x gridDim.x partials of a past synchronisation into shared
@@ -271,13 +330,20 @@ __device__ __forceinline__ void deferred_parts_fetch(const float2* parts, int sl
 
 // Waits for deferred_parts_fetch's copies; warps 1..K sum value k = warp - 1
 // of the block partials in index order (as warp_sum_parts) into S.red.
-// Contains __syncthreads() and a named barrier over warps 1..K+1 (K + 1 <= 15).
-template <int K>
-__device__ __forceinline__ void deferred_parts_sum(const float2* pbuf, LoopShared& S)
+// Contains __syncthreads().  CL: the partials are in shared memory already.
+template <bool CL, int K>
+__device__ __forceinline__ void deferred_parts_sum(const Sync& y, int slot, const float2* pbuf, LoopShared& S)
 {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if constexpr (CL) {
+        if (warp >= 1 && warp <= K) {
+            const FF t = warp_total<true>(y, slot + warp - 1);
+            if (lane == 0) S.red[warp - 1] = ff_to_double(t);
+        }
+        return;
+    }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = (gridDim.x + 1) >> 1;
     if (warp >= 1 && warp <= K) {
         const float2* v = pbuf + (warp - 1) * 2 * nch;
@@ -878,13 +944,16 @@ __device__ __forceinline__ void phase_ls(const Reg& reg, const Rows& R, const fl
 
 // ------------------------------------------------------------------ kernel
 
-template <int MC>
+// CL: the grid is one cluster (at most kClusterMax blocks).
+template <int MC, bool CL>
 __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
 {
     static_assert(MC > 0, "the loop kernel needs a compile-time FFT size");
     using G = Geo<MC>;
     extern __shared__ float2 sm[];
     __shared__ LoopShared S;
+    __shared__ float2 cparts[CL ? kPartSlots * kClusterMax : 1];
+    const Sync y{A.parts, cparts, A.counter, A.abort_word, A.err, A.wait_ns};
     const int N = A.N, RB = A.RB;
     Rows R;
     R.N = N;
@@ -937,16 +1006,22 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             fftd::build_staged_twiddles<MC>(A.tw, stw);
         }
         const int nc = (R.hhi - R.hlo + 1) * N;
-        const float2* src = A.f0 + (int64_t)R.hlo * N;
+        const float2 zero = make_float2(0.f, 0.f);
+        const float2* src = A.x0 ? A.x0 + (int64_t)R.hlo * N : nullptr;
         float2* dst = cf + R.cache(R.hlo);
-        for (int e = threadIdx.x; e < nc; e += kLoopThreads) dst[e] = __ldcg(src + e);
+        for (int e = threadIdx.x; e < nc; e += kLoopThreads) dst[e] = src ? __ldcg(src + e) : zero;
         const int64_t o = (int64_t)R.R0 * N;
         for (int e = threadIdx.x; e < R.nown * N; e += kLoopThreads) {
-            cRes[e] = __ldcg(A.res + o + e);
-            cD[e] = __ldg(A.D + o + e);
+            const float2 dv = __ldg(A.D + o + e), tx = src ? __ldcg(A.res + o + e) : zero;
+            cD[e] = dv;
+            cRes[e] = cgd::f2sub(tx, dv);
         }
     }
     __syncthreads();
+    if constexpr (CL) {  // every block of the cluster runs before the first store into it
+        cluster_arrive();
+        cluster_wait();
+    }
     if (A.stall) {
         // a test's injected stall: wait for one arrival more than the grid
         // makes, so that the bounded wait runs out in every block
@@ -963,7 +1038,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             phase_update<MC, true, RX2>(A, R, fbuf, stw, cf, cd, cRes, cD, cg, cTd, 0.f, A.iters > 0, a);
         else
             phase_update<MC, true, 1>(A, R, fbuf, stw, cf, cd, cRes, cD, cg, cTd, 0.f, A.iters > 0, a);
-        if (!grid_reduce<kUpdVals>(a, A.parts, L_A, seq, S, A.counter, A.abort_word, A.err, A.wait_ns)) return;
+        if (!grid_reduce<CL, kUpdVals>(a, y, L_A, seq, S)) return;
         if (threadIdx.x == 0) {
             for (int v = 0; v < kUpdVals; ++v) S.red[v] = ff_to_double(S.redf[v]);
             double J, beta;
@@ -984,7 +1059,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
         const bool deferred = k > 0;
         bool fetch = deferred;  // issued once the first column group is staged
         auto fetch_parts = [&] {
-            if (fetch) deferred_parts_fetch<kUpdVals>(A.parts, L_A, pbuf);
+            if (!CL && fetch) deferred_parts_fetch<kUpdVals>(A.parts, L_A, pbuf);
             fetch = false;
         };
         if constexpr (!G::FOURSTEP) fetch_parts();
@@ -992,7 +1067,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
         for (int gi = blockIdx.x; gi < col_groups; gi += gridDim.x) {
             const int x0 = gi * cpc;
             if constexpr (G::FOURSTEP)
-                cols_split(A.X, N, x0, A.ChatS, stw, stw + 512, fbuf, fetch_parts);
+                cols_split(A.X, N, x0, A.Chat, stw, stw + 512, fbuf, fetch_parts);
             else if (wide_cols)
                 fftd::cols_group<MC, G::CBPT2, 1>(A.X, N, N, x0, cpc, cpc, A.fp, stw, A.Chat, fbuf, nullptr);
             else
@@ -1006,16 +1081,26 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
         // partials and warp 7 forms J and beta from them (the column pass does
         // not need beta: T d = -T g + beta T d_old is formed in the row pass)
         fetch_parts();  // a block without a column group
-        if (deferred) deferred_parts_sum<kUpdVals>(pbuf, S);
-        else __syncthreads();
         ++seq;
-        if (threadIdx.x == 0) S.ok = grid_arrive_wait(A.counter, seq * gridDim.x, A.abort_word, A.err, A.wait_ns) ? 1 : 0;
+        if constexpr (CL) {
+            cluster_arrive();
+            if (deferred) deferred_parts_sum<CL, kUpdVals>(y, L_A, pbuf, S);
+        } else {
+            if (deferred) deferred_parts_sum<CL, kUpdVals>(y, L_A, pbuf, S);
+            else __syncthreads();
+            if (threadIdx.x == 0)
+                S.ok = grid_arrive_wait(A.counter, seq * gridDim.x, A.abort_word, A.err, A.wait_ns) ? 1 : 0;
+        }
         if (deferred && (threadIdx.x >> 5) >= 1 && (threadIdx.x >> 5) <= kUpdVals + 1) {
             asm volatile("bar.sync 1, %0;" ::"r"(32 * (kUpdVals + 1)) : "memory");
             if (threadIdx.x == 32 * (kUpdVals + 1)) finish_update(A, S, k);
         }
+        if constexpr (CL) {
+            __syncwarp();
+            cluster_wait();
+        }
         __syncthreads();
-        if (!S.ok) return;
+        if (!CL && !S.ok) return;
         mark(1);
         const float beta = S.beta_f;
         const bool restart = S.restart != 0;
@@ -1027,7 +1112,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             else
                 phase_rows<MC, 1>(A, R, fbuf, stw, cf, cd, cRes, cD, cg, cTd, beta, restart, acc);
             mark(2);
-            if (!grid_reduce<4>(acc, A.parts, L_C, seq, S, A.counter, A.abort_word, A.err, A.wait_ns)) return;
+            if (!grid_reduce<CL, 4>(acc, y, L_C, seq, S)) return;
             // every thread forms t1 from the totals (no broadcast, no barrier);
             // thread 0 keeps q1, q2 and t1 for the next steps
             const FF t1 = cgd::ls_next_ff(FF{0.f, 0.f}, S.redf[0], S.redf[3], S.redf[1], S.redf[2]);
@@ -1045,7 +1130,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             float acc[2] = {0.f, 0.f};
             phase_ls<MC>(A.reg, R, cf, cd, fbuf, t_f, acc);
             mark(4 + 2 * j);
-            if (!grid_reduce<2>(acc, A.parts, j == 0 ? L_D : L_E, seq, S, A.counter, A.abort_word, A.err, A.wait_ns)) return;
+            if (!grid_reduce<CL, 2>(acc, y, j == 0 ? L_D : L_E, seq, S)) return;
             // t2 from t1 (tb[0] -> tb[1]), then t3 from t2 (tb[1] -> tb[0]),
             // in every thread; the step read and the step written never share
             // a slot
@@ -1062,7 +1147,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             else
                 phase_update<MC, false, 1>(A, R, fbuf, stw, cf, cd, cRes, cD, cg, cTd, t_f, k + 1 < A.iters, a);
             mark(8);
-            if (!grid_arrive_parts<kUpdVals>(a, A.parts, L_A, seq, S, A.counter, A.abort_word, A.err, A.wait_ns)) return;
+            if (!grid_arrive_parts<CL, kUpdVals>(a, y, L_A, seq, S)) return;
             mark(9);
         }
     }
@@ -1070,7 +1155,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
     if (A.iters > 0) {
         const int warp = threadIdx.x >> 5;
         if (warp < kUpdVals) {
-            const FF a = warp_sum_parts(A.parts + (L_A + warp) * kMaxParts, gridDim.x);
+            const FF a = warp_total<CL>(y, L_A + warp);
             if ((threadIdx.x & 31) == 0) S.red[warp] = ff_to_double(a);
         }
         __syncthreads();
@@ -1089,7 +1174,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
         const int64_t o = (int64_t)R.R0 * N;
         const float2* fo = cf + R.cache(R.R0);
         for (int e = threadIdx.x; e < R.nown * N; e += kLoopThreads) {
-            A.f0[o + e] = fo[e];
+            A.out[o + e] = fo[e];
             A.res[o + e] = cRes[e];
         }
     }
@@ -1101,6 +1186,11 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
     }
 }
 
+// Grid sizes whose loop may run as a cluster: M <= 256 (at most 16 column groups
+// and, for the first shapes, row blocks).
+template <int MC>
+constexpr bool loop_has_cluster() { return MC <= 256; }
+
 // Sets the function's shared-memory cap (once per device, to the largest
 // size any shape may ask for) and returns it.
 template <int MC>
@@ -1110,9 +1200,10 @@ bool loop_cap(size_t* cap_out)
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return false;
-    auto kern = k_cg_loop<MC>;
+    // (the cluster form has the larger static part)
+    constexpr bool has_cl = loop_has_cluster<MC>();
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return false;
+    if (cudaFuncGetAttributes(&fa, k_cg_loop<MC, has_cl>) != cudaSuccess) return false;
     const size_t cap = (size_t)optin - fa.sharedSizeBytes;
     // the cap is a property of the function shared by every plan and thread:
     // set once to the largest shape, never lowered (a concurrent launch with
@@ -1122,7 +1213,12 @@ bool loop_cap(size_t* cap_out)
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= 64) return false;
     if (set_cap[dev] < (int)cap) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_cg_loop<MC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess)
+            return false;
+        if (has_cl &&
+            (cudaFuncSetAttribute(k_cg_loop<MC, has_cl>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) !=
+                 cudaSuccess ||
+             cudaFuncSetAttribute(k_cg_loop<MC, has_cl>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))
             return false;
         set_cap[dev] = (int)cap;
     }
@@ -1159,7 +1255,7 @@ bool loop_fits(int N, int RB, size_t cap, int sms, bool wide, int* grid_out, siz
     const size_t smem = loop_smem<MC>(N, RB, (size_t)grid);
     if (smem > cap) return false;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_loop<MC>, kLoopThreads, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_loop<MC, false>, kLoopThreads, smem) != cudaSuccess)
         return false;
     if (per_sm < 1 || grid > sms * per_sm || grid > kMaxParts) return false;
     *grid_out = grid;
@@ -1207,20 +1303,44 @@ bool loop_shape(const spirec_plan_s* p, int* RB_out, int* grid_out, size_t* smem
     return true;
 }
 
-// The spectrum in the split order of the M = 1024 column pass:
-// out[c * 1024 + h * 512 + k] = Chat[kx * 1024 + 2 k + h], kx = 2 (c mod 512) + c / 512
-// (column c of the split row layout holds the frequency kx).
-__global__ void k_chat_split(const float* __restrict__ Chat, float* __restrict__ out)
+cudaLaunchConfig_t cluster_config(int grid, size_t smem, cudaLaunchAttribute* at)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // < 1024 * 1024
-    const int c = i >> 10, h = (i >> 9) & 1, k = i & 511;
-    const int kx = 2 * (c & 511) + (c >> 9);
-    out[i] = __ldg(Chat + kx * 1024 + 2 * k + h);
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)grid;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kLoopThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether a loop of `grid` blocks runs as one cluster: up to 16 blocks, where the
+// device places such a cluster.  An iteration (us) with the grid barrier and as a
+// cluster: N = 64, M = 128 (8 blocks) 20.9 and 17.6; N = 128, M = 256 (16 blocks)
+// 24.4 and 20.6: the five synchronisations 9.9 -> 5.1.
+template <int MC>
+bool cluster_fits(int grid, size_t smem)
+{
+    if (grid > kClusterMax) return false;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(grid, smem, &at);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (const void*)k_cg_loop<MC, true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
 }
 
 struct LaunchLoop {
     spirec_plan p;
     int iters;
+    const float2* x0;
+    float2* out;
     template <int MC>
     int operator()()
     {
@@ -1239,20 +1359,13 @@ struct LaunchLoop {
             A.N = p->N;
             A.iters = iters;
             A.RB = RB;
-            A.f0 = p->f[0];
+            A.x0 = x0;
+            A.out = out;
             A.g = p->g;
             A.res = p->res;
             A.D = p->D;
             A.X = p->X;
             A.Chat = p->Chat;
-            if constexpr (Geo<MC>::FOURSTEP) {
-                // the split-order copy, in the spectrum build's scratch (M x M complex)
-                float* chs = reinterpret_cast<float*>(p->cwork);
-                k_chat_split<<<1024 * 1024 / 256, 256, 0, p->stream>>>(p->Chat, chs);
-                SPIREC_CK(cudaGetLastError());
-                p->launches += 1;
-                A.ChatS = chs;
-            }
             A.tw = p->twiddle;
             A.fp = p->fft;
             A.reg = p->reg;
@@ -1266,8 +1379,18 @@ struct LaunchLoop {
             A.stall = injected_stall(kStallLoop) ? 1 : 0;
             // no arrivals, no abort
             SPIREC_CK(cudaMemsetAsync(A.counter, 0, 3 * sizeof(unsigned), p->stream));
+            if constexpr (loop_has_cluster<MC>()) {
+                if (cluster_fits<MC>(grid, smem)) {
+                    cudaLaunchAttribute at;
+                    cudaLaunchConfig_t cfg = cluster_config(grid, smem, &at);
+                    cfg.stream = p->stream;
+                    SPIREC_CK(cudaLaunchKernelEx(&cfg, k_cg_loop<MC, true>, A));
+                    p->launches += 1;
+                    return SPIREC_OK;
+                }
+            }
             void* args[] = {&A};
-            SPIREC_CK(cudaLaunchCooperativeKernel((const void*)k_cg_loop<MC>, dim3(grid), dim3(kLoopThreads), args,
+            SPIREC_CK(cudaLaunchCooperativeKernel((const void*)k_cg_loop<MC, false>, dim3(grid), dim3(kLoopThreads), args,
                                                   smem, p->stream));
             p->launches += 1;
             return SPIREC_OK;
@@ -1299,7 +1422,7 @@ struct Shapes {
                 if (capacity) {
                     int sms = 0, per_sm = 0;
                     if (device_sms(&sms) != SPIREC_OK ||
-                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_loop<MC>, kLoopThreads, smem) !=
+                        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_loop<MC, false>, kLoopThreads, smem) !=
                             cudaSuccess) {
                         cudaGetLastError();
                         return 0;
@@ -1341,15 +1464,15 @@ int loop_demand(spirec_plan p, int* blocks, int* capacity)
     return shapes_for(p, &RB, blocks, 1, true, capacity);
 }
 
-int launch_cg_loop(spirec_plan p, int iters)
+int launch_cg_loop(spirec_plan p, int iters, const float2* x0, float2* out)
 {
     switch (p->MF) {
-    case 64: return LaunchLoop{p, iters}.operator()<64>();
-    case 128: return LaunchLoop{p, iters}.operator()<128>();
-    case 256: return LaunchLoop{p, iters}.operator()<256>();
-    case 512: return LaunchLoop{p, iters}.operator()<512>();
-    case 1024: return LaunchLoop{p, iters}.operator()<1024>();
-    default: return LaunchLoop{p, iters}.operator()<0>();
+    case 64: return LaunchLoop{p, iters, x0, out}.operator()<64>();
+    case 128: return LaunchLoop{p, iters, x0, out}.operator()<128>();
+    case 256: return LaunchLoop{p, iters, x0, out}.operator()<256>();
+    case 512: return LaunchLoop{p, iters, x0, out}.operator()<512>();
+    case 1024: return LaunchLoop{p, iters, x0, out}.operator()<1024>();
+    default: return LaunchLoop{p, iters, x0, out}.operator()<0>();
     }
 }
 

@@ -499,15 +499,6 @@ k_rows_inv_split(const float2* __restrict__ X, int N, int ldx, float2* __restric
     }
 }
 
-// Position of frequency k in the columns of X and in Chat at M = MC: the class
-// order of the split passes, else k itself.
-template <int MC>
-__host__ __device__ __forceinline__ int split_pos(int k)
-{
-    constexpr int S = MC >= 2048 ? MC / 1024 : 1;
-    return S > 1 ? (k & (S - 1)) * 1024 + k / S : k;
-}
-
 // ------------------------------------------------------- kernel spectrum
 //
 // Chat[kx][ky] = (1 / M^2) sum_{u,v} c_{u,v} exp(-i2pi (kx u + ky v) / M) with
@@ -866,13 +857,8 @@ int launch_spectrum(spirec_plan p)
 // Complex values of X.
 size_t x_elems(int N, int MF) { return (size_t)(MF >= 2048 ? split_ld(N) : N) * MF; }
 
-// Complex values of cwork: the N x M rows of a spectrum build on either grid,
-// and the persistent loop's split-order spectrum at MF = 1024 (k_chat_split).
-size_t cwork_elems(int N, int M, int MF)
-{
-    const size_t rows = (size_t)N * (M > MF ? M : MF), split = MF == 1024 ? (size_t)1024 * 1024 / 2 : 0;
-    return rows > split ? rows : split;
-}
+// Complex values of cwork: the N x M rows of a spectrum build on either grid.
+size_t cwork_elems(int N, int M, int MF) { return (size_t)N * (M > MF ? M : MF); }
 
 int launch_spectrum_out(spirec_plan p, float* out)
 {
@@ -927,14 +913,15 @@ __global__ void k_noalloc_twiddles(float2* tw, int M)
 }
 
 // spectrum[ky][kx] (the layout spirec_kernel_spectrum_dev returns) into the
-// column-major form the column pass reads, chat[kx][ky].
+// column-major form the column pass reads, chat[kx][ky] (both at split_pos).
+template <int MC>
 __global__ void k_noalloc_spectrum(const float* __restrict__ spec, int M, float* __restrict__ chat)
 {
     const int64_t MM = (int64_t)M * M;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < MM;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t kx = e / M, ky = e % M;
-        chat[e] = spec[ky * M + kx];
+        const int kx = (int)(e / M), ky = (int)(e % M);
+        chat[(int64_t)split_pos<MC>(kx) * M + split_pos<MC>(ky)] = spec[(int64_t)ky * M + kx];
     }
 }
 
@@ -1015,7 +1002,8 @@ extern "C" int spirec_toeplitz_noalloc(const float* x, const float* spectrum, fl
     cudaStream_t st = (cudaStream_t)stream;
     k_noalloc_twiddles<<<(M + 255) / 256, 256, 0, st>>>(tw, M);
     SPIREC_CK(cudaGetLastError());
-    k_noalloc_spectrum<<<4 * 152, 256, 0, st>>>(spectrum, M, chat);
+    if (M == 1024) k_noalloc_spectrum<1024><<<4 * 152, 256, 0, st>>>(spectrum, M, chat);
+    else k_noalloc_spectrum<0><<<4 * 152, 256, 0, st>>>(spectrum, M, chat);
     SPIREC_CK(cudaGetLastError());
     return with_size(M, LaunchNoAlloc{(const float2*)x, (float2*)Tx, rows, chat, tw, fp, N, st});
 }

@@ -93,6 +93,17 @@ __host__ __device__ constexpr int seq_len(int M)
     return MC > 0 ? M + (M >> 4) : M;
 }
 
+// Position of frequency k in Chat (both indices) at M = MC and, from M = 2048 on,
+// in the columns of X: by classes k mod S of M / S each, as the transforms split
+// into S DFTs leave them (S = 2 at M = 1024 in the persistent loop; S = M / 1024
+// in the split passes of fft.cu); k itself below.
+template <int MC>
+__host__ __device__ __forceinline__ int split_pos(int k)
+{
+    constexpr int S = MC >= 2048 ? MC / 1024 : MC == 1024 ? 2 : 1;
+    return S > 1 ? (k & (S - 1)) * (MC / S) + k / S : k;
+}
+
 // --------------------------------------------- runtime mixed-radix Stockham
 
 template <int R, bool INV>
@@ -354,7 +365,7 @@ __device__ __forceinline__ void rows_inv_group(const float2* X, int r0, int nr, 
 // ------------------------------------------------------ column pass, a group
 
 // Columns [x0, x0 + nc) of the buffer X (M columns): FFT of the n_in nonzero
-// rows, times Chat[x][ky], IFFT, rows < n_out back into X.  Sequences sit at
+// rows, times Chat[x][ky] (at split_pos), IFFT, rows < n_out back into X.  Sequences sit at
 // stride seq_len + 4 (spreads the banks of the transposed loads).
 // MODE 1 (the persistent CG loop, compile-time M only): the twiddle table is
 // in shared memory and Chat is read through L2 only.
@@ -380,9 +391,8 @@ __device__ __forceinline__ void cols_group(float2* X, int n_in, int n_out, int x
             const bool in = y < n_in && cc < nc;
             v[i] = in ? __ldcg(X + (int64_t)y * M + x0 + cc) : make_float2(0.f, 0.f);
             const int hc = e / M, hk = e - hc * M;
-            h[i] = hc < nc ? (MODE == 1 ? __ldcg(&Chat[(int64_t)(x0 + hc) * M + hk])
-                                        : __ldg(&Chat[(int64_t)(x0 + hc) * M + hk]))
-                           : 0.f;
+            const int64_t ho = (int64_t)split_pos<MC>(x0 + hc) * M + split_pos<MC>(hk);
+            h[i] = hc < nc ? (MODE == 1 ? __ldcg(Chat + ho) : __ldg(Chat + ho)) : 0.f;
         }
 #pragma unroll
         for (int i = 0; i < E; ++i) {

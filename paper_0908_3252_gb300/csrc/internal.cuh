@@ -127,8 +127,8 @@ struct spirec_plan_s {
     double* hpin;
 
     float2* G;     // N x (2N-1)
-    float* Chat;   // MF x MF real, transposed: Chat[kx*MF + ky]
-    float2* cwork; // cwork_elems: rows of the spectrum builds, the loop's split-order spectrum
+    float* Chat;   // MF x MF real, transposed: Chat[kx*MF + ky], both at split_pos (fft_device.cuh)
+    float2* cwork; // cwork_elems: rows of the spectrum builds
     float2* X;     // x_elems: N x MF complex (Toeplitz rows; by columns at MF >= 2048)
     float2* D;     // N x N
     float2* s;     // L (+32 padding)
@@ -226,9 +226,10 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev);
 // The whole loop (first gradient + iters iterations) as one persistent
 // cooperative kernel (cg_loop.cu); MF in [64, 1024] only, and
 // SPIREC_EUNSUPPORTED (nothing enqueued) when the image does not fit its
-// shared-memory caches.  The iterate ends in f[0].
+// shared-memory caches.  Starts from x0 (device; null: zeros), with p->res = T x0
+// when x0 is given; the last iterate goes to `out` (device, may be x0).
 bool loop_supported(int M);
-int launch_cg_loop(spirec_plan p, int iters);
+int launch_cg_loop(spirec_plan p, int iters, const float2* x0, float2* out);
 
 // Pairing of the output columns.  The B operand is a pure phase,
 // E(l, j) = exp(sb i2pi kb_l (j + half/2)), and its conjugate is the phase of
