@@ -91,20 +91,54 @@ bool smooth235(int m)
 }
 
 constexpr int kCacheMaxTerms = 64;
+// The interleaves of a plan's trajectory: index in the cache, first sample
+// there, and first sample in the plan (pos[n] = L).
 struct CacheTerms {
     int n;
     int idx[kCacheMaxTerms];
+    int64_t from[kCacheMaxTerms];
+    int64_t pos[kCacheMaxTerms + 1];
 };
 
-// dst[e] = sum_j src[idx[j] * stride + e], j in the listed order.
-__global__ void k_sum_cached(const float* __restrict__ src, int64_t stride, CacheTerms t, float* __restrict__ dst)
+// A plan's trajectory from a cache in one kernel: its samples, and the sums of
+// the interleaves' spectra and G (in the listed order); the error word is
+// cleared.  (Four interleaves at 128^2 to 256^2: eight copies, a clear and two
+// sums were eleven launches and about 20 us on the GPU.)
+__global__ void __launch_bounds__(256) k_load_cached(const int64_t* __restrict__ ckx, const int64_t* __restrict__ cky,
+                                                     const float4* __restrict__ cspec, int64_t spec4,
+                                                     const float2* __restrict__ cG, int64_t nG, const CacheTerms t,
+                                                     int64_t* __restrict__ kxq, int64_t* __restrict__ kyq,
+                                                     float4* __restrict__ spec, float2* __restrict__ G, int* flag)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < stride;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        float acc = 0.f;
-        for (int j = 0; j < t.n; ++j) acc += __ldg(src + t.idx[j] * stride + e);
-        dst[e] = acc;
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (first == 0) *flag = 0;
+    for (int64_t e = first; e < spec4; e += step) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < t.n; ++j) {
+            const float4 v = __ldg(cspec + t.idx[j] * spec4 + e);
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+        spec[e] = a;
     }
+    for (int64_t e = first; e < nG; e += step) {
+        float2 a = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < t.n; ++j) {
+            const float2 v = __ldg(cG + t.idx[j] * nG + e);
+            a.x += v.x;
+            a.y += v.y;
+        }
+        G[e] = a;
+    }
+    for (int j = 0; j < t.n; ++j)
+        for (int64_t i = first; i < t.pos[j + 1] - t.pos[j]; i += step) {
+            kxq[t.pos[j] + i] = ckx[t.from[j] + i];
+            kyq[t.pos[j] + i] = cky[t.from[j] + i];
+        }
 }
 
 // The plan's stream after the caller's stream, and the caller's stream after
@@ -326,13 +360,16 @@ int build_trajectory(spirec_plan p, const double* kx_dev, const double* ky_dev, 
     return SPIREC_OK;
 }
 
-int build_data(spirec_plan p)
+// p->s, ||s||^2 and D of the data set s (device, 8-byte aligned); `read`, if given,
+// is recorded once s has been read.
+int build_data(spirec_plan p, const float2* s, cudaEvent_t read = nullptr)
 {
     int rc;
-    if ((rc = launch_data_norm(p)) != SPIREC_OK) return rc;
     cudaEvent_t e;
     if ((rc = tstart(p, 2, &e)) != SPIREC_OK) return rc;
-    if ((rc = launch_adjoint(p, p->s, p->D)) != SPIREC_OK) return rc;
+    if ((rc = launch_pair_weights(p, s, true)) != SPIREC_OK) return rc;
+    if (read) SPIREC_CK(cudaEventRecord(read, p->stream));
+    if ((rc = launch_adjoint_prepared(p, p->D)) != SPIREC_OK) return rc;
     if ((rc = tstop(p, e)) != SPIREC_OK) return rc;
     p->have_data = true;
     return SPIREC_OK;
@@ -945,6 +982,8 @@ int spirec_set_trajectory_cached(spirec_plan p, spirec_kcache c, const int32_t* 
             return SPIREC_EINVAL;
         }
         t.idx[j] = which[j];
+        t.from[j] = c->off[which[j]];
+        t.pos[j] = total;
         total += c->off[which[j] + 1] - c->off[which[j]];
     }
     if (total != p->L) {
@@ -954,25 +993,15 @@ int spirec_set_trajectory_cached(spirec_plan p, spirec_kcache c, const int32_t* 
     Join j(p);
     p->have_traj = false;
     p->have_data = false;
-    SPIREC_CK(cudaMemsetAsync(p->dflag, 0, sizeof(int), p->stream));
-    int64_t pos = 0;
-    for (int k = 0; k < count; ++k) {
-        const int64_t o = c->off[which[k]], Li = c->off[which[k] + 1] - o;
-        SPIREC_CK(cudaMemcpyAsync(p->kxq + pos, c->kxq + o, sizeof(int64_t) * Li, cudaMemcpyDeviceToDevice, p->stream));
-        SPIREC_CK(cudaMemcpyAsync(p->kyq + pos, c->kyq + o, sizeof(int64_t) * Li, cudaMemcpyDeviceToDevice, p->stream));
-        pos += Li;
-    }
-    const int64_t MM = (int64_t)p->MF * p->MF, NG2 = 2 * (int64_t)p->N * (2 * p->N - 1);
-    int blocks = (int)((MM + 255) / 256);
+    t.pos[count] = total;
+    const int64_t spec4 = (int64_t)p->MF * p->MF / 4, nG = (int64_t)p->N * (2 * p->N - 1);
+    int64_t blocks = (std::max(spec4, nG) + 255) / 256;
     if (blocks > 8 * 152) blocks = 8 * 152;
-    k_sum_cached<<<blocks, 256, 0, p->stream>>>(c->spec, MM, t, p->Chat);
+    k_load_cached<<<(unsigned)blocks, 256, 0, p->stream>>>(
+        c->kxq, c->kyq, reinterpret_cast<const float4*>(c->spec), spec4, c->G, nG, t, p->kxq, p->kyq,
+        reinterpret_cast<float4*>(p->Chat), p->G, p->dflag);
     SPIREC_CK(cudaGetLastError());
-    blocks = (int)((NG2 + 255) / 256);
-    if (blocks > 8 * 152) blocks = 8 * 152;
-    k_sum_cached<<<blocks, 256, 0, p->stream>>>(reinterpret_cast<const float*>(c->G), NG2, t,
-                                                reinterpret_cast<float*>(p->G));
-    SPIREC_CK(cudaGetLastError());
-    p->launches += 2;
+    p->launches += 1;
     p->have_traj = true;
     return SPIREC_OK;
 }
@@ -1030,7 +1059,7 @@ int spirec_set_data(spirec_plan p, const float* s)
     Join j(p);
     // The caller's buffer is copied on a side stream and the call returns
     // once that copy is done, not after the trajectory work queued before it
-    // on the plan's stream; the plan's stream then moves it into place.
+    // on the plan's stream; the plan's stream then reads it there.
     const size_t bytes = sizeof(float2) * p->L;
     if (!p->s_in) {
         SPIREC_CK(cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking));
@@ -1043,9 +1072,7 @@ int spirec_set_data(spirec_plan p, const float* s)
     SPIREC_CK(cudaMemcpyAsync(p->s_in, s, bytes, cudaMemcpyHostToDevice, p->copy_stream));
     SPIREC_CK(cudaEventRecord(p->ev_s_ready, p->copy_stream));
     SPIREC_CK(cudaStreamWaitEvent(p->stream, p->ev_s_ready, 0));
-    SPIREC_CK(cudaMemcpyAsync(p->s, p->s_in, bytes, cudaMemcpyDeviceToDevice, p->stream));
-    SPIREC_CK(cudaEventRecord(p->ev_sin_free, p->stream));
-    rc = build_data(p);
+    rc = build_data(p, p->s_in, p->ev_sin_free);
     if (rc == SPIREC_OK) SPIREC_CK(cudaEventSynchronize(p->ev_s_ready));
     return rc;
 }
@@ -1063,8 +1090,11 @@ int spirec_set_data_dev(spirec_plan p, const float* s)
         return SPIREC_ESTATE;
     }
     Join j(p);
-    SPIREC_CK(cudaMemcpyAsync(p->s, s, sizeof(float2) * p->L, cudaMemcpyDeviceToDevice, p->stream));
-    return build_data(p);
+    if (((uintptr_t)s & (sizeof(float2) - 1)) != 0) {  // not readable as float2
+        SPIREC_CK(cudaMemcpyAsync(p->s, s, sizeof(float2) * p->L, cudaMemcpyDeviceToDevice, p->stream));
+        return build_data(p, p->s);
+    }
+    return build_data(p, reinterpret_cast<const float2*>(s));
 }
 
 int spirec_set_reg(spirec_plan p, double lambda1, double alpha1, double lambda0, double alpha0,

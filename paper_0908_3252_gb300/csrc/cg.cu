@@ -50,30 +50,6 @@ namespace {
 
 using cgd::redot;
 
-// ||s||^2 -> scal[S_SS]
-__global__ void k_sumsq(const float2* __restrict__ s, int64_t L, float2* parts, unsigned* counter,
-                        double* scal)
-{
-    float acc = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 v = s[i];
-        acc += redot(v, v);
-    }
-    float v[1] = {acc};
-    FF bt[1];
-    block_partial<1>(v, bt);
-    store_parts<1>(bt, parts, kMaxParts);
-    if (last_block(counter)) {
-        FF t[1];
-        sum_parts_ff<1>(parts, kMaxParts, gridDim.x, t);
-        if (threadIdx.x == 0) {
-            scal[S_SS] = ff_to_double(t[0]);
-            *counter = 0u;
-        }
-    }
-}
-
 // A block's part of an N x N image: `rows` rows (fewer at the end) of a strip of
 // 256 columns, a thread a column.  The right neighbour of a value comes from
 // the next lane, that of a warp's last lane (`edge`) from memory.
@@ -233,16 +209,6 @@ __global__ void k_res_init(float2* res, const float2* __restrict__ D, int64_t n,
 int launch_res_init(spirec_plan p, float2* res, bool have_tx)
 {
     k_res_init<<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(res, p->D, (int64_t)p->N * p->N, have_tx ? 1 : 0);
-    SPIREC_CK(cudaGetLastError());
-    p->launches += 1;
-    return SPIREC_OK;
-}
-
-int launch_data_norm(spirec_plan p)
-{
-    int blocks = (int)((p->L + 255) / 256);
-    if (blocks > 4 * 152) blocks = 4 * 152;
-    k_sumsq<<<blocks, 256, 0, p->stream>>>(p->s, p->L, slot(p, P_MISC), p->counters + C_MISC, p->scal);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
     return SPIREC_OK;

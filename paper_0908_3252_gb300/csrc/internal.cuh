@@ -199,12 +199,12 @@ size_t cwork_elems(int N, int M, int MF);
 size_t x_elems(int N, int MF);
 int launch_adjoint(spirec_plan p, const float2* y, float2* x);  // x = H^H y
 int launch_forward(spirec_plan p, const float2* x, float2* y);  // y = H x
+int launch_adjoint_prepared(spirec_plan p, float2* x);  // x = H^H y after launch_pair_weights(p, y, ...)
 
 // Toeplitz T x -> Tx; with cg also q2 = Re<x, T x> and the first line-search step.
 int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, const CgPass* cg = nullptr);
 int fft_setup_attributes(int maxM);
 // CG pieces (cg.cu).  Iteration k reads f[k & 1] and writes f[(k + 1) & 1].
-int launch_data_norm(spirec_plan p);
 // res = Tx - D where res holds T x (have_tx), else res = -D (x = 0)
 int launch_res_init(spirec_plan p, float2* res, bool have_tx);
 // gradient at f (res = T f - D given): g, J -> Jout, <g,g>; first = no step taken
@@ -258,9 +258,10 @@ struct PairGeom {
 };
 
 PairGeom pair_geom(const spirec_plan_s* p, int knob);
-// p->wpair = w' (see PairGeom): w_l exp(sb i2pi (kb_l / 2) shift2) for l < L, its
-// padding past L left at zero; with amax2 also max_l |w'_l|^2 as float bits.
-int launch_pair_weights(spirec_plan p, const float2* w, const int64_t* kb, int sb, int shift2, unsigned* amax2);
+// p->wpair = the weights w' of H^H y (see PairGeom), zero padding past L kept, and
+// max_l |w'_l|^2 as float bits in the counter C_AMAX.  data: y is a data set,
+// also copied to p->s, with ||y||^2 into scal[S_SS].
+int launch_pair_weights(spirec_plan p, const float2* y, bool data);
 
 // FP32 contractions (nudft_simt.cu)
 size_t kpart_floats_simt(int N, int64_t L);
@@ -268,7 +269,7 @@ int simt_setup_attributes();
 
 // tensor-core contractions (FP16x3 / BF16x3)
 int launch_gram_tc(spirec_plan p);
-int launch_adjoint_tc(spirec_plan p, const float2* y, float2* x);
+int launch_adjoint_tc(spirec_plan p, float2* x);  // H^H of the prepared weights
 int launch_forward_tc(spirec_plan p, const float2* x, float2* y);
 size_t fsplit_bytes_tc(int N, int precision);  // the forward's split-image buffer
 size_t kpart_floats_tc(int N, int64_t L, int precision);  // split-K buffer need

@@ -406,25 +406,16 @@ void launch_gemm(cudaStream_t st, const int64_t* ka, const int64_t* kb, const fl
         k_phase_gemm<false, ROWS><<<grid, G::THREADS, sizeof(typename G::Smem), st>>>(ka, kb, w, L, pg, oa, sa, sb, cps, part);
 }
 
-// out[i][c] = scale sum_l A(l,i) B(l,c) with A(l,i) = exp(sa i2pi ka_l (i + oa)),
-// B(l,c) = w_l exp(sb i2pi kb_l (c + ob)).
-int phase_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, const float2* w, int oa, int ob, int sa,
-               int sb, float scale, float2* out)
+// out[i][c] = scale sum_l A(l,i) B(l,c), as tc_pair_gemm.
+int phase_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, bool weighted, int oa, int sa, int sb,
+               float scale, float2* out)
 {
     const PairGeom pg = pair_geom(p, knob);
     const int64_t nchunks = (p->L + KC - 1) / KC;
     const int64_t RC = (int64_t)pg.R * pg.C;
     int sms = 0, rc;
     if ((rc = device_sms(&sms)) != SPIREC_OK) return rc;
-    const int shift2 = pg.C2 + 2 * ob;  // twice the phase offset of the centre column
-    if (!w && shift2 != 0) {
-        set_error("an unweighted paired contraction needs its centre at phase zero");
-        return SPIREC_EUNSUPPORTED;
-    }
-    if (w) {
-        if ((rc = launch_pair_weights(p, w, kb, sb, shift2, nullptr)) != SPIREC_OK) return rc;
-        w = p->wpair;
-    }
+    const float2* w = weighted ? p->wpair : nullptr;
     const int S = choose_splits(p, knob, sms, pg, nchunks);
     const int64_t cps = (nchunks + S - 1) / S;
     const int Seff = (int)((nchunks + cps - 1) / cps);
@@ -445,16 +436,21 @@ int launch_gram(spirec_plan p)
     if (p->precision != SPIREC_FP32) return launch_gram_tc(p);
     const int N = p->N;
     // G[u][v+N-1] = (1/N^2) sum_l exp(i2pi kx_l u) exp(i2pi ky_l v)
-    return phase_gemm(p, SPIREC_KNOB_GRAM_SPLIT, p->kxq, p->kyq, nullptr, 0, -(N - 1), +1, +1,
+    return phase_gemm(p, SPIREC_KNOB_GRAM_SPLIT, p->kxq, p->kyq, false, 0, +1, +1,
                       1.0f / ((float)N * (float)N), p->G);
+}
+
+int launch_adjoint_prepared(spirec_plan p, float2* x)
+{
+    if (p->precision != SPIREC_FP32) return launch_adjoint_tc(p, x);
+    // x[n][m] = (1/N) sum_l exp(-i2pi ky_l n) * (y_l exp(-i2pi kx_l m))
+    return phase_gemm(p, SPIREC_KNOB_ADJOINT_SPLIT, p->kyq, p->kxq, true, 0, -1, -1, 1.0f / (float)p->N, x);
 }
 
 int launch_adjoint(spirec_plan p, const float2* y, float2* x)
 {
-    if (p->precision != SPIREC_FP32) return launch_adjoint_tc(p, y, x);
-    const int N = p->N;
-    // x[n][m] = (1/N) sum_l exp(-i2pi ky_l n) * (y_l exp(-i2pi kx_l m))
-    return phase_gemm(p, SPIREC_KNOB_ADJOINT_SPLIT, p->kyq, p->kxq, y, 0, 0, -1, -1, 1.0f / (float)N, x);
+    const int rc = launch_pair_weights(p, y, false);
+    return rc != SPIREC_OK ? rc : launch_adjoint_prepared(p, x);
 }
 
 int contraction_split(spirec_plan p, int knob, int* value, int* sms_used)

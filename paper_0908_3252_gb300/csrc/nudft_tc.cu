@@ -72,6 +72,7 @@
 
 #include "internal.cuh"
 #include "phase.cuh"
+#include "reduce.cuh"
 
 namespace spirec {
 
@@ -1068,24 +1069,62 @@ __global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* __rest
 }
 
 // w'_l = w_l exp(sb i2pi (kb_l / 2) shift2) for l < L (the weight of the
-// original B operand and the phase of the pairing's centre column, shift2 =
-// C2 + 2 ob); the plan's buffer keeps its zero padding past L.  amax2 (zeroed
-// before the launch; may be null) receives max_l |w'_l|^2 as float bits, as
-// k_absmax2.
-__global__ void k_pair_weights(const float2* __restrict__ w, const int64_t* __restrict__ kb, int64_t L, int sb,
-                               int shift2, float2* __restrict__ wp, unsigned* amax2)
+// original B operand and the phase of the pairing's centre column); the plan's
+// buffer keeps its zero padding past L.  The last block writes amax2 = max_l
+// |w'_l|^2 (as float bits; warps that met a value that is not finite do not
+// count).  DATA: w is a data set, also copied to s (unless it is s), and the
+// last block writes ||w||^2 to scal[S_SS]: one kernel of about 5 us where a
+// copy, a clear, the norm and the weights took four launches and 13.
+template <bool DATA>
+__global__ void __launch_bounds__(256) k_pair_weights(const float2* w, const int64_t* __restrict__ kb, int64_t L, int sb,
+                                                      int shift2, float2* __restrict__ wp, float2* s, float2* parts,
+                                                      unsigned* counter, unsigned* amax2, double* scal)
 {
-    float mx = 0.f;
+    float mx = 0.f, ss = 0.f;
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < L; l += (int64_t)gridDim.x * blockDim.x) {
         float2 e = phasor_q(kb[l] >> 1, shift2);
         if (sb < 0) e.y = -e.y;
-        const float2 v = cmul(w[l], e);
+        const float2 u = w[l];
+        const float2 v = cmul(u, e);
         wp[l] = v;
         mx = fmaxf(mx, fmaf(v.x, v.x, v.y * v.y));
+        if (DATA) {
+            if (s != w) s[l] = u;
+            ss += fmaf(u.x, u.x, u.y * u.y);
+        }
     }
+    __shared__ float wmax[8];
+    auto block_max = [&](float m) {  // of the 8 warps, valid in thread 0
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (amax2 && (threadIdx.x & 31) == 0 && isfinite(mx)) atomicMax(amax2, __float_as_uint(mx));
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = isfinite(m) ? m : 0.f;
+        __syncthreads();
+        m = wmax[0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) m = fmaxf(m, wmax[k]);
+        __syncthreads();
+        return m;
+    };
+    const float bm = block_max(mx);
+    if (threadIdx.x == 0) parts[kMaxParts + blockIdx.x] = make_float2(bm, 0.f);
+    if (DATA) {
+        float v[1] = {ss};
+        FF bt[1];
+        block_partial<1>(v, bt);
+        store_parts<1>(bt, parts, kMaxParts);
+    }
+    if (last_block(counter)) {
+        float m = 0.f;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) m = fmaxf(m, __ldcg(parts + kMaxParts + i).x);
+        m = block_max(m);
+        FF t[1] = {};
+        if (DATA) sum_parts_ff<1>(parts, kMaxParts, gridDim.x, t);
+        if (threadIdx.x == 0) {
+            *amax2 = __float_as_uint(m);
+            if (DATA) scal[S_SS] = ff_to_double(t[0]);
+            *counter = 0u;
+        }
+    }
 }
 
 // ------------------------------------------------------------ forward H f
@@ -1613,9 +1652,11 @@ void launch_reduce(cudaStream_t st, const float* part, int64_t U, int64_t K, int
 }
 
 // The paired contraction out[i][c] = scale sum_l A(l,i) B(l,c) with
-// A(l,i) = exp(sa i2pi ka_l (i + oa)), B(l,c) = w_l exp(sb i2pi kb_l (c + ob)).
-int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, const float2* w, int oa, int ob,
-                 int sa, int sb, float scale, float2* out)
+// A(l,i) = exp(sa i2pi ka_l (i + oa)), B(l,c) = w_l exp(sb i2pi kb_l (c + ob));
+// weighted: the weights are prepared in p->wpair (their maximum in C_AMAX);
+// unweighted: ob puts the pairing's centre column at phase zero.
+int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, bool weighted, int oa, int sa, int sb,
+                 float scale, float2* out)
 {
     const PairGeom pg = pair_geom(p, knob);
     int sms = 0, rc;
@@ -1630,23 +1671,10 @@ int tc_pair_gemm(spirec_plan p, int knob, const int64_t* ka, const int64_t* kb, 
         set_error("%lld contraction units exceed the kernel's 32-bit unit counters", (long long)U);
         return SPIREC_EUNSUPPORTED;
     }
-    if (!w && pg.half) {
-        set_error("an unweighted paired contraction takes integer offsets");
-        return SPIREC_EUNSUPPORTED;
-    }
     int64_t P = 0;
     if ((rc = tc_ctas(p, knob, sms, &P)) != SPIREC_OK) return rc;
-    unsigned* amax = nullptr;
-    const int shift2 = pg.C2 + 2 * ob;  // twice the phase offset of the centre column
-    if (!w && shift2 != 0) {
-        set_error("an unweighted paired contraction needs its centre at phase zero");
-        return SPIREC_EUNSUPPORTED;
-    }
-    if (w) {
-        amax = p->counters + C_AMAX;
-        if ((rc = launch_pair_weights(p, w, kb, sb, shift2, amax)) != SPIREC_OK) return rc;
-        w = p->wpair;
-    }
+    const float2* w = weighted ? p->wpair : nullptr;
+    unsigned* amax = weighted ? p->counters + C_AMAX : nullptr;
     float* part = p->kpart;
     const bool bf16 = p->precision == SPIREC_MIXED_BF16X3;
     const unsigned long long wait_ns = wait_limit_ns();
@@ -1686,12 +1714,20 @@ PairGeom pair_geom(const spirec_plan_s* p, int knob)
     return g;
 }
 
-int launch_pair_weights(spirec_plan p, const float2* w, const int64_t* kb, int sb, int shift2, unsigned* amax2)
+int launch_pair_weights(spirec_plan p, const float2* y, bool data)
 {
     int blocks = (int)((p->L + 255) / 256);
     if (blocks > 4 * kMaxCtas) blocks = 4 * kMaxCtas;
-    if (amax2) SPIREC_CK(cudaMemsetAsync(amax2, 0, sizeof(unsigned), p->stream));
-    k_pair_weights<<<blocks, 256, 0, p->stream>>>(w, kb, p->L, sb, shift2, p->wpair, amax2);
+    const int shift2 = pair_geom(p, SPIREC_KNOB_ADJOINT_SPLIT).C2;  // twice the centre column
+    float2* parts = reinterpret_cast<float2*>(p->part) + (size_t)P_MISC * kMaxParts;
+    unsigned* counter = p->counters + C_MISC;
+    unsigned* amax = p->counters + C_AMAX;
+    if (data)
+        k_pair_weights<true><<<blocks, 256, 0, p->stream>>>(y, p->kxq, p->L, -1, shift2, p->wpair, p->s, parts, counter,
+                                                            amax, p->scal);
+    else
+        k_pair_weights<false><<<blocks, 256, 0, p->stream>>>(y, p->kxq, p->L, -1, shift2, p->wpair, nullptr, parts,
+                                                             counter, amax, nullptr);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
     return SPIREC_OK;
@@ -1795,15 +1831,14 @@ int launch_gram_tc(spirec_plan p)
 {
     const int N = p->N;
     // G[u][v+N-1] = (1/N^2) sum_l exp(i2pi kx_l u) exp(i2pi ky_l v), v = +-j
-    return tc_pair_gemm(p, SPIREC_KNOB_GRAM_SPLIT, p->kxq, p->kyq, nullptr, 0, -(N - 1), +1, +1,
+    return tc_pair_gemm(p, SPIREC_KNOB_GRAM_SPLIT, p->kxq, p->kyq, false, 0, +1, +1,
                         1.0f / ((float)N * (float)N), p->G);
 }
 
-int launch_adjoint_tc(spirec_plan p, const float2* y, float2* x)
+int launch_adjoint_tc(spirec_plan p, float2* x)
 {
-    const int N = p->N;
     // x[n][m] = (1/N) sum_l exp(-i2pi ky_l n) y_l exp(-i2pi kx_l m)
-    return tc_pair_gemm(p, SPIREC_KNOB_ADJOINT_SPLIT, p->kyq, p->kxq, y, 0, 0, -1, -1, 1.0f / (float)N, x);
+    return tc_pair_gemm(p, SPIREC_KNOB_ADJOINT_SPLIT, p->kyq, p->kxq, true, 0, -1, -1, 1.0f / (float)p->N, x);
 }
 
 // The tile shape of a contraction (knob SPIREC_KNOB_GRAM_TILE or
