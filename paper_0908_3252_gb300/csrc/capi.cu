@@ -10,7 +10,6 @@
 #include <algorithm>
 #include <atomic>
 #include <map>
-#include <memory>
 #include <new>
 #include <vector>
 
@@ -813,27 +812,8 @@ int spirec_plan_create(spirec_plan* out, int32_t N, int64_t L, int32_t M, int32_
     TRYCUDA(cudaMemsetAsync(p->dbuf[0], 0, NN * sizeof(float2), p->stream));
     TRYCUDA(cudaMemsetAsync(p->dbuf[1], 0, NN * sizeof(float2), p->stream));
     TRYCUDA(cudaMemsetAsync(p->g, 0, NN * sizeof(float2), p->stream));
-    {
-        std::unique_ptr<float2[]> tw(new (std::nothrow) float2[(size_t)MF + M]);
-        if (!tw) {
-            free_plan(p);
-            set_error("host allocation failed");
-            return SPIREC_ENOMEM;
-        }
-        auto table = [](int m, float2* t) {
-            for (int k = 0; k < m; ++k) {
-                const double a = -2.0 * M_PI * (double)k / (double)m;
-                t[k] = make_float2((float)cos(a), (float)sin(a));
-            }
-        };
-        table(MF, tw.get());
-        if (M != MF) table(M, tw.get() + MF);
-        e = cudaMemcpyAsync(p->twiddle, tw.get(), sizeof(float2) * MF, cudaMemcpyHostToDevice, p->stream);
-        if (e == cudaSuccess && M != MF)
-            e = cudaMemcpyAsync(p->twiddle_M, tw.get() + MF, sizeof(float2) * M, cudaMemcpyHostToDevice, p->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-        TRYCUDA(e);
-    }
+    TRY(launch_twiddles(p->twiddle, MF, p->stream));
+    if (M != MF) TRY(launch_twiddles(p->twiddle_M, M, p->stream));
     {
         // kernel attributes (shared-memory limits) are per device context:
         // set once, not per plan

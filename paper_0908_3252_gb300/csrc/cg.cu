@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "cg_device.cuh"
+#include "chain.cuh"
 #include "fft_device.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
@@ -87,25 +88,25 @@ struct Strip {
 // two took 160 us; they take 41 + 48.
 template <int KIND>
 __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
-k_direction(const float2* __restrict__ g, const float2* __restrict__ d_old, float2* __restrict__ d_new,
-            const float2* __restrict__ f, const float2* __restrict__ res, int N, int rows, Reg reg, float2* parts,
+k_direction(const float2* g, const float2* d_old, float2* d_new, const float2* f, const float2* res, int N, int rows, Reg reg, float2* parts,
             unsigned* counter, double* scal)
 {
+    chain_enter();
     const double bd = scal[S_BETA];
     const float beta = (float)bd;
     const bool restart = (__double_as_longlong(bd) << 1) == 0;  // beta = 0 (an FP64 compare would be redone every pixel)
     const Strip st(N, rows);
     const float2 zero = make_float2(0.f, 0.f);
-    auto dir = [&](int64_t o) { return fftd::new_direction(g[o], restart ? zero : d_old[o], beta, restart); };
+    auto dir = [&](int64_t o) { return fftd::new_direction(__ldcg(g + o), restart ? zero : __ldcg(d_old + o), beta, restart); };
     float v[3] = {0.f, 0.f, 0.f};
     int64_t o = st.first;
-    float2 dn = st.in ? dir(o) : zero, fn = st.in ? f[o] : zero;
+    float2 dn = st.in ? dir(o) : zero, fn = st.in ? __ldcg(f + o) : zero;
 #pragma unroll 2
     for (int n = st.n0; n < st.n1; ++n, o += N) {
         const bool has_d = n + 1 < N;
-        const float2 dd = st.in && has_d ? dir(o + N) : dn, fd = st.in && has_d ? f[o + N] : fn;
-        const float2 rs = st.in ? res[o] : zero;
-        const float2 dr = st.right(dn, st.edge ? dir(o + 1) : dn), fr = st.right(fn, st.edge ? f[o + 1] : fn);
+        const float2 dd = st.in && has_d ? dir(o + N) : dn, fd = st.in && has_d ? __ldcg(f + o + N) : fn;
+        const float2 rs = st.in ? __ldcg(res + o) : zero;
+        const float2 dr = st.right(dn, st.edge ? dir(o + 1) : dn), fr = st.right(fn, st.edge ? __ldcg(f + o + 1) : fn);
         if (st.in) {
             d_new[o] = dn;
             v[0] += 2.f * redot(dn, rs);
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_line_search(const float2* f, const float2* d, int N, Reg reg, int step, float2* parts,
               unsigned* counter, double* scal)
 {
+    chain_enter();
     const double t = scal[S_T1 + step - 1];
     const float tf = (float)t;
     const int P = N * N;
@@ -163,6 +165,7 @@ k_update(const float2* f_in, float2* f_out, const float2* d, float2* res, const 
          const float2* __restrict__ D, float2* g, int N, Reg reg, float2* parts, unsigned* counter,
          double* scal, double* Jout)
 {
+    chain_enter();
     const float t = FIRST ? 0.f : (float)scal[S_T3];
     const int P = N * N;
     float a[kUpdVals];
@@ -218,7 +221,7 @@ namespace {
 template <int KIND>
 void line_search_k(spirec_plan p, const float2* f, const float2* d, int step)
 {
-    k_line_search<KIND><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(f, d, p->N, p->reg, step, slot(p, P_LS),
+    chain(k_line_search<KIND>, vec_blocks(p->N), kVecThreads, 0, p->stream, f, d, p->N, p->reg, step, slot(p, P_LS),
                                                                          p->counters + C_LS, p->scal);
 }
 
@@ -227,10 +230,10 @@ void update_k(spirec_plan p, const float2* f_in, float2* f_out, const float2* d,
               float2* g, int first, double* Jout)
 {
     if (first)
-        k_update<true, KIND><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(
+        chain(k_update<true, KIND>, vec_blocks(p->N), kVecThreads, 0, p->stream, 
             f_in, f_out, d, res, Td, p->D, g, p->N, p->reg, slot(p, P_UPD), p->counters + C_UPD, p->scal, Jout);
     else
-        k_update<false, KIND><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(
+        chain(k_update<false, KIND>, vec_blocks(p->N), kVecThreads, 0, p->stream, 
             f_in, f_out, d, res, Td, p->D, g, p->N, p->reg, slot(p, P_UPD), p->counters + C_UPD, p->scal, Jout);
 }
 }  // namespace
@@ -278,7 +281,7 @@ void direction_k(spirec_plan p, int k)
 {
     int rows = 0;
     const dim3 grid = strip_grid(p->N, &rows);
-    k_direction<KIND><<<grid, kVecThreads, 0, p->stream>>>(p->g, p->dbuf[(k + 1) & 1], p->dbuf[k & 1], p->f[k & 1], p->res,
+    chain(k_direction<KIND>, grid, kVecThreads, 0, p->stream, p->g, p->dbuf[(k + 1) & 1], p->dbuf[k & 1], p->f[k & 1], p->res,
                                                            p->N, rows, p->reg, slot(p, P_ROWA), p->counters + C_ROWA,
                                                            p->scal);
 }
@@ -303,6 +306,7 @@ int launch_direction(spirec_plan p, int k)
 __global__ void k_q2_t1(const float2* d, const float2* Td, int64_t n, float2* parts, unsigned* counter,
                         double* scal)
 {
+    chain_enter();
     float v[1] = {0.f};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float2 a = __ldcg(d + i), b = __ldcg(Td + i);
@@ -334,7 +338,7 @@ int launch_normal_direct(spirec_plan p, const float2* x, float2* Tx, bool dot_q2
     if ((rc = launch_forward(p, x, p->ydir)) != SPIREC_OK) return rc;
     if ((rc = launch_adjoint(p, p->ydir, Tx)) != SPIREC_OK) return rc;
     if (dot_q2_t1) {
-        k_q2_t1<<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(x, Tx, (int64_t)p->N * p->N, slot(p, P_ROWC),
+        chain(k_q2_t1, vec_blocks(p->N), kVecThreads, 0, p->stream, x, Tx, (int64_t)p->N * p->N, slot(p, P_ROWC),
                                                                   p->counters + C_ROWC, p->scal);
         SPIREC_CK(cudaGetLastError());
         p->launches += 1;

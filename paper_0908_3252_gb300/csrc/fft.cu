@@ -28,6 +28,7 @@
 #include <atomic>
 #include <mutex>
 
+#include "chain.cuh"
 #include "fft_device.cuh"
 #include "fft_reg.cuh"
 #include "internal.cuh"
@@ -66,6 +67,8 @@ template <int MC>
 __global__ void __launch_bounds__(1024) k_rows_fwd(const float2* in, int ld_in, int n_in, int rows, float2* X, FftPlan fp,
                            const float2* __restrict__ tw, int rpc)
 {
+    chain_enter();
+    chain_next();
     extern __shared__ float2 sm[];
     float2* a = sm;
     float2* b = sm + rpc * seq_len<MC>(fp.M);
@@ -103,6 +106,8 @@ template <int MC, bool CG>
 __global__ void __launch_bounds__(1024) k_rows_inv(const float2* X, int rows, float2* out, int n_out, FftPlan fp,
                            const float2* __restrict__ tw, int rpc, const float2* dotx, CgPass c)
 {
+    chain_enter();
+    chain_next();
     extern __shared__ float2 sm[];
     float2* a = sm;
     float2* b = sm + rpc * seq_len<MC>(fp.M);
@@ -119,6 +124,8 @@ template <int MC>
 __global__ void __launch_bounds__(1024) k_cols_filter(float2* X, int n_in, int n_out, FftPlan fp, const float2* __restrict__ tw,
                               const float* __restrict__ Chat, int cpc)
 {
+    chain_enter();
+    chain_next();
     extern __shared__ float2 sm[];
     const int ld = seq_len<MC>(fp.M) + 4;
     const int x0 = blockIdx.x * cpc;
@@ -217,9 +224,10 @@ __device__ __forceinline__ void store_sector(float2* p, float2 a, float2 b, floa
 }
 __device__ __forceinline__ void load_sector(const float2* p, float2 (&v)[4])
 {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y)
-        : "l"(p));
+        : "l"(p)
+        : "memory");
 }
 
 // Barrier of `threads` threads of the block (whole warps), id 1 .. 15.
@@ -310,6 +318,7 @@ template <int S, bool CG>
 __global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
 k_cols_split(float2* X, int N, int ldx, const float2* __restrict__ tw, const float* __restrict__ Chat, CgPass dot)
 {
+    chain_enter();
     constexpr int M = 1024 * S, C = kSplitWarps / (2 * S), T = 64 * S;  // pairs a block, threads a team
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StagedSmem& ss = *reinterpret_cast<StagedSmem*>(smem_raw);
@@ -390,6 +399,7 @@ template <int S>
 __global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
 k_rows_fwd_split(const float2* __restrict__ in, int N, float2* X, int ldx, const float2* __restrict__ tw)
 {
+    chain_enter();
     constexpr int R = kSplitWarps / S, T = 32 * S;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StagedSmem& ss = *reinterpret_cast<StagedSmem*>(smem_raw);
@@ -447,6 +457,7 @@ template <int S>
 __global__ void __launch_bounds__(kSplitThreads, kSplitCtasPerSm)
 k_rows_inv_split(const float2* __restrict__ X, int N, int ldx, float2* __restrict__ out, const float2* __restrict__ tw)
 {
+    chain_enter();
     constexpr int R = kSplitWarps / S;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SplitSmem& sm = *reinterpret_cast<SplitSmem*>(smem_raw);
@@ -583,13 +594,17 @@ struct Shape {
     size_t smem;
 };
 
-// Compile-time path: nseq * M / 4 threads (<= 1024), single buffer.
+// Compile-time path: nseq * M / 4 threads (<= 1024), single buffer; as few rows
+// and columns a block as keep two warps busy and 32-byte pieces whole, so that
+// small grids spread over the SMs and their stages' barriers span few warps
+// (T at N = 64 with 8 rows and 32 columns a block and plain launches 18.5 us, now
+// 7.7; at N = 256 21.8 and 15.9).
 // Runtime path: 256 threads, ping-pong buffers.
 Shape row_shape(int M, bool pow2)
 {
     if (pow2) {
         const int nb = M / 4;
-        const int rpc = nb >= 256 ? 1 : 256 / nb;
+        const int rpc = nb >= 64 ? 1 : 64 / nb;
         return Shape{rpc, rpc * nb, (size_t)rpc * seq_len<1>(M) * sizeof(float2)};
     }
     const int rpc = M >= 1024 ? 1 : 1024 / M;
@@ -600,7 +615,7 @@ Shape col_shape(int M, bool pow2)
 {
     if (pow2) {
         const int nb = M / 4;
-        int cpc = nb >= 1024 ? 1 : 1024 / nb;
+        int cpc = nb >= 256 ? (nb >= 1024 ? 1 : 1024 / nb) : 4;
         const size_t ld = seq_len<1>(M) + 4;
         while (cpc > 1 && (size_t)cpc * ld * sizeof(float2) > (size_t)kFftSmemCap) cpc /= 2;
         return Shape{cpc, cpc * nb, (size_t)cpc * ld * sizeof(float2)};
@@ -683,10 +698,10 @@ struct LaunchRowsFwd {
             constexpr int S = MC / 1024;
             int grid = 0, rc;
             if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
-            k_rows_fwd_split<S><<<grid, kSplitThreads, sizeof(StagedSmem), p->stream>>>(in, N, p->X, split_ld(N), p->twiddle);
+            chain(k_rows_fwd_split<S>, grid, kSplitThreads, sizeof(StagedSmem), p->stream, in, N, p->X, split_ld(N), p->twiddle);
         } else {
             const Shape s = row_shape(p->MF, MC > 0);
-            k_rows_fwd<MC><<<(N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+            chain(k_rows_fwd<MC>, (N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 in, N, N, N, p->X, p->fft, p->twiddle, s.per_cta);
         }
         SPIREC_CK(cudaGetLastError());
@@ -707,11 +722,11 @@ struct LaunchCols {
             int grid = 0, rc;
             if ((rc = split_grid(MC / 2, kSplitWarps / (2 * S), &grid)) != SPIREC_OK) return rc;
             auto kern = cg ? k_cols_split<S, true> : k_cols_split<S, false>;
-            kern<<<grid, kSplitThreads, sizeof(StagedSmem), p->stream>>>(p->X, N, split_ld(N), p->twiddle, p->Chat,
+            chain(kern, grid, kSplitThreads, sizeof(StagedSmem), p->stream, p->X, N, split_ld(N), p->twiddle, p->Chat,
                                                                         cg ? *cg : CgPass{});
         } else {
             const Shape s = col_shape(p->MF, MC > 0);
-            k_cols_filter<MC><<<(p->MF + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+            chain(k_cols_filter<MC>, (p->MF + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 p->X, N, N, p->fft, p->twiddle, p->Chat, s.per_cta);
         }
         SPIREC_CK(cudaGetLastError());
@@ -733,11 +748,11 @@ struct LaunchRowsInv {
             constexpr int S = MC / 1024;
             int grid = 0, rc;
             if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
-            k_rows_inv_split<S><<<grid, kSplitThreads, sizeof(SplitSmem), p->stream>>>(p->X, N, split_ld(N), out, p->twiddle);
+            chain(k_rows_inv_split<S>, grid, kSplitThreads, sizeof(SplitSmem), p->stream, p->X, N, split_ld(N), out, p->twiddle);
         } else {
             const Shape s = row_shape(p->MF, MC > 0);
             auto kern = cg ? k_rows_inv<MC, true> : k_rows_inv<MC, false>;
-            kern<<<(N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream>>>(
+            chain(kern, (N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 p->X, N, out, N, p->fft, p->twiddle, s.per_cta, cg ? x : nullptr, cg ? *cg : CgPass{});
         }
         SPIREC_CK(cudaGetLastError());
@@ -817,6 +832,25 @@ int fft_setup_attributes(int)
     if ((rc = set_split_attrs<4>()) != SPIREC_OK) return rc;
     for (int M = 16; M <= 4096; M *= 2)
         if ((rc = with_size(M, AttrAll{})) != SPIREC_OK) return rc;
+    return SPIREC_OK;
+}
+
+namespace {
+// tw[k] = exp(-2 pi i k / M), formed in FP64 and rounded once
+__global__ void k_twiddles(float2* tw, int M)
+{
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
+        double s, c;
+        sincospi(-2.0 * (double)k / (double)M, &s, &c);
+        tw[k] = make_float2((float)c, (float)s);
+    }
+}
+}  // namespace
+
+int launch_twiddles(float2* tw, int M, cudaStream_t st)
+{
+    k_twiddles<<<(M + 255) / 256, 256, 0, st>>>(tw, M);
+    SPIREC_CK(cudaGetLastError());
     return SPIREC_OK;
 }
 
@@ -901,16 +935,6 @@ constexpr int kNoAllocMaxDevices = 64;
 // host threads on one device run the set-up once
 std::atomic<void*> g_noalloc_base[kNoAllocMaxDevices];
 std::mutex g_noalloc_mu;
-
-// tw[k] = exp(-2 pi i k / M)
-__global__ void k_noalloc_twiddles(float2* tw, int M)
-{
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < M; k += gridDim.x * blockDim.x) {
-        double s, c;
-        sincospi(-2.0 * (double)k / (double)M, &s, &c);
-        tw[k] = make_float2((float)c, (float)s);
-    }
-}
 
 // spectrum[ky][kx] (the layout spirec_kernel_spectrum_dev returns) into the
 // column-major form the column pass reads, chat[kx][ky] (both at split_pos).
@@ -1000,8 +1024,8 @@ extern "C" int spirec_toeplitz_noalloc(const float* x, const float* spectrum, fl
     float* chat = reinterpret_cast<float*>(base + kNoAllocRowsBytes);
     float2* tw = reinterpret_cast<float2*>(base + kNoAllocRowsBytes + kNoAllocSpecBytes);
     cudaStream_t st = (cudaStream_t)stream;
-    k_noalloc_twiddles<<<(M + 255) / 256, 256, 0, st>>>(tw, M);
-    SPIREC_CK(cudaGetLastError());
+    const int rc = launch_twiddles(tw, M, st);
+    if (rc != SPIREC_OK) return rc;
     if (M == 1024) k_noalloc_spectrum<1024><<<4 * 152, 256, 0, st>>>(spectrum, M, chat);
     else k_noalloc_spectrum<0><<<4 * 152, 256, 0, st>>>(spectrum, M, chat);
     SPIREC_CK(cudaGetLastError());

@@ -44,6 +44,7 @@
 #include <stdint.h>
 
 #include "cg_device.cuh"
+#include "chain.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
 
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_hq_outer(const float2* f, const float2* res, const float2* __restrict__ D, int N, Reg reg, HqW W, float2* parts,
            unsigned* counter, double* scal, double* Jout)
 {
+    chain_enter();
     const int P = N * N;
     float v[3] = {0.f, 0.f, 0.f};  // R, Re<f, D>, Re<f, res>
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -176,6 +178,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_hq_residual(const float2* f, const float2* res, HqW W, int N, float2* r,
               float2* pv, float2* sv, float2* Ts, float2* parts, unsigned* counter, double* scal)
 {
+    chain_enter();
     const int P = N * N;
     float v[1] = {0.f};
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -210,6 +213,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_hq_apply(const float2* pv, const float2* Tp, HqW W, const float2* f, int N, float2* q, float2* parts,
            unsigned* counter, double* scal)
 {
+    chain_enter();
     const int P = N * N;
     float v[1] = {0.f};
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -243,6 +247,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_hq_step(float2* f, float2* res, float2* r, const float2* pv, const float2* Tp, const float2* q, int N,
           float2* parts, unsigned* counter, double* scal)
 {
+    chain_enter();
     const float a = (float)scal[S_HQ_ALPHA];
     const int P = N * N;
     float v[1] = {0.f};
@@ -271,6 +276,7 @@ k_hq_step(float2* f, float2* res, float2* r, const float2* pv, const float2* Tp,
 // p = r + beta p.
 __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm) k_hq_dir(const float2* r, float2* pv, int N, const double* scal)
 {
+    chain_enter();
     const float b = (float)scal[S_HQ_BETA];
     const int P = N * N;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x)
@@ -286,6 +292,7 @@ __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_nt_ls0(const float2* f, const float2* sv, const float2* Ts, const float2* res, int N,
          Reg reg, float2* parts, unsigned* counter, double* scal)
 {
+    chain_enter();
     const int P = N * N;
     float v[4] = {0.f, 0.f, 0.f, 0.f};  // q1, q2, num0, den0
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -317,6 +324,7 @@ k_nt_ls0(const float2* f, const float2* sv, const float2* Ts, const float2* res,
 __global__ void __launch_bounds__(kVecThreads, kVecBlocksPerSm)
 k_nt_update(float2* f, float2* res, const float2* sv, const float2* Ts, int N, const double* scal)
 {
+    chain_enter();
     const float t = (float)scal[S_T3];
     const int P = N * N;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -336,7 +344,7 @@ HqW weights_of(spirec_plan p)
 template <int KIND>
 void nt_ls0_k(spirec_plan p, const float2* sv, const float2* Ts)
 {
-    k_nt_ls0<KIND><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(p->f[0], sv, Ts, p->res, p->N, p->reg,
+    chain(k_nt_ls0<KIND>, vec_blocks(p->N), kVecThreads, 0, p->stream, p->f[0], sv, Ts, p->res, p->N, p->reg,
                                                                     slot(p, P_UPD), p->counters + C_UPD, p->scal);
 }
 
@@ -349,10 +357,10 @@ int launch_hq_objective(spirec_plan p, double* Jout)
         return SPIREC_ESTATE;
     }
     if (p->minimiser == SPIREC_MIN_NEWTON)
-        k_hq_outer<true><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(
+        chain(k_hq_outer<true>, vec_blocks(p->N), kVecThreads, 0, p->stream, 
             p->f[0], p->res, p->D, p->N, p->reg, weights_of(p), slot(p, P_UPD), p->counters + C_UPD, p->scal, Jout);
     else
-        k_hq_outer<false><<<vec_blocks(p->N), kVecThreads, 0, p->stream>>>(
+        chain(k_hq_outer<false>, vec_blocks(p->N), kVecThreads, 0, p->stream, 
             p->f[0], p->res, p->D, p->N, p->reg, weights_of(p), slot(p, P_UPD), p->counters + C_UPD, p->scal, Jout);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
@@ -368,7 +376,7 @@ int hq_outer_step(spirec_plan p, int k, double* Jdev)
     float2 *f = p->f[0], *pv = p->dbuf[0];
     int rc;
     if ((rc = launch_hq_objective(p, Jdev ? Jdev + k : nullptr)) != SPIREC_OK) return rc;
-    k_hq_residual<false><<<blocks, kVecThreads, 0, p->stream>>>(f, p->res, W, N, p->g, pv, nullptr, nullptr,
+    chain(k_hq_residual<false>, blocks, kVecThreads, 0, p->stream, f, p->res, W, N, p->g, pv, nullptr, nullptr,
                                                                 slot(p, P_UPD), p->counters + C_UPD, p->scal);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
@@ -376,13 +384,13 @@ int hq_outer_step(spirec_plan p, int k, double* Jdev)
         rc = p->mode == SPIREC_MODE_DIRECT ? launch_normal_direct(p, pv, p->Td, false)
                                            : launch_toeplitz(p, pv, p->Td);
         if (rc != SPIREC_OK) return rc;
-        k_hq_apply<false><<<blocks, kVecThreads, 0, p->stream>>>(pv, p->Td, W, nullptr, N, p->tmp, slot(p, P_UPD),
+        chain(k_hq_apply<false>, blocks, kVecThreads, 0, p->stream, pv, p->Td, W, nullptr, N, p->tmp, slot(p, P_UPD),
                                                                  p->counters + C_UPD, p->scal);
         SPIREC_CK(cudaGetLastError());
-        k_hq_step<<<blocks, kVecThreads, 0, p->stream>>>(f, p->res, p->g, pv, p->Td, p->tmp, N, slot(p, P_UPD),
+        chain(k_hq_step, blocks, kVecThreads, 0, p->stream, f, p->res, p->g, pv, p->Td, p->tmp, N, slot(p, P_UPD),
                                                          p->counters + C_UPD, p->scal);
         SPIREC_CK(cudaGetLastError());
-        k_hq_dir<<<blocks, kVecThreads, 0, p->stream>>>(p->g, pv, N, p->scal);
+        chain(k_hq_dir, blocks, kVecThreads, 0, p->stream, p->g, pv, N, p->scal);
         SPIREC_CK(cudaGetLastError());
         p->launches += 3;
     }
@@ -399,7 +407,7 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev)
     float2 *f = p->f[0], *pv = p->dbuf[0], *sv = p->dbuf[1], *Ts = p->f[1];
     int rc;
     if ((rc = launch_hq_objective(p, Jdev ? Jdev + k : nullptr)) != SPIREC_OK) return rc;
-    k_hq_residual<true><<<blocks, kVecThreads, 0, p->stream>>>(f, p->res, W, N, p->g, pv, sv, Ts,
+    chain(k_hq_residual<true>, blocks, kVecThreads, 0, p->stream, f, p->res, W, N, p->g, pv, sv, Ts,
                                                                slot(p, P_UPD), p->counters + C_UPD, p->scal);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
@@ -407,13 +415,13 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev)
         rc = p->mode == SPIREC_MODE_DIRECT ? launch_normal_direct(p, pv, p->Td, false)
                                            : launch_toeplitz(p, pv, p->Td);
         if (rc != SPIREC_OK) return rc;
-        k_hq_apply<true><<<blocks, kVecThreads, 0, p->stream>>>(pv, p->Td, W, f, N, p->tmp, slot(p, P_UPD),
+        chain(k_hq_apply<true>, blocks, kVecThreads, 0, p->stream, pv, p->Td, W, f, N, p->tmp, slot(p, P_UPD),
                                                                 p->counters + C_UPD, p->scal);
         SPIREC_CK(cudaGetLastError());
-        k_hq_step<<<blocks, kVecThreads, 0, p->stream>>>(sv, Ts, p->g, pv, p->Td, p->tmp, N, slot(p, P_UPD),
+        chain(k_hq_step, blocks, kVecThreads, 0, p->stream, sv, Ts, p->g, pv, p->Td, p->tmp, N, slot(p, P_UPD),
                                                          p->counters + C_UPD, p->scal);
         SPIREC_CK(cudaGetLastError());
-        k_hq_dir<<<blocks, kVecThreads, 0, p->stream>>>(p->g, pv, N, p->scal);
+        chain(k_hq_dir, blocks, kVecThreads, 0, p->stream, p->g, pv, N, p->scal);
         SPIREC_CK(cudaGetLastError());
         p->launches += 3;
     }
@@ -426,7 +434,7 @@ int nt_outer_step(spirec_plan p, int k, double* Jdev)
     p->launches += 1;
     if ((rc = launch_line_search(p, f, sv, 1)) != SPIREC_OK) return rc;
     if ((rc = launch_line_search(p, f, sv, 2)) != SPIREC_OK) return rc;
-    k_nt_update<<<blocks, kVecThreads, 0, p->stream>>>(f, p->res, sv, Ts, N, p->scal);
+    chain(k_nt_update, blocks, kVecThreads, 0, p->stream, f, p->res, sv, Ts, N, p->scal);
     SPIREC_CK(cudaGetLastError());
     p->launches += 1;
     return SPIREC_OK;

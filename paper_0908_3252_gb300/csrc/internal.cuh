@@ -109,7 +109,7 @@ struct spirec_plan_s {
     // into s; made on first use
     cudaStream_t copy_stream;
     cudaEvent_t ev_s_ready;   // s_in holds the caller's data
-    cudaEvent_t ev_sin_free;  // the plan's stream has moved s_in into s
+    cudaEvent_t ev_sin_free;  // the plan's stream has read s_in
     cudaEvent_t ev_traj_in;   // a host trajectory is on the device (spirec_set_trajectory)
     float2* s_in;             // L (+32)
 
@@ -203,6 +203,7 @@ int launch_adjoint_prepared(spirec_plan p, float2* x);  // x = H^H y after launc
 
 // Toeplitz T x -> Tx; with cg also q2 = Re<x, T x> and the first line-search step.
 int launch_toeplitz(spirec_plan p, const float2* x, float2* Tx, const CgPass* cg = nullptr);
+int launch_twiddles(float2* tw, int M, cudaStream_t st);  // tw[k] = exp(-2 pi i k / M)
 int fft_setup_attributes(int maxM);
 // CG pieces (cg.cu).  Iteration k reads f[k & 1] and writes f[(k + 1) & 1].
 // res = Tx - D where res holds T x (have_tx), else res = -D (x = 0)
