@@ -32,6 +32,13 @@
 // half runs each as a register four-step (16 x 32): the row buffers hold a
 // row as [h][k] (element 2k + h of the DFT at h * 512 + k), the column pass
 // runs two warps per column, and the row passes two warps per row.
+// At M = 256 and 512 a half-warp carries a 256-point DFT as 16 x 16 (16 values a
+// lane, one exchange): a sequence at M = 256, one of the two halves above of a
+// sequence at M = 512.  Below, radix-4 stages over shared memory by the block.
+// What bounds an iteration is its chain: five synchronisations of 0.8-1.5 us and
+// the latencies of the phases between them.  Radix-4 stages with a block barrier
+// each cost more than the arithmetic (four iterations at N = 128: 108 us, with
+// these 87; an iteration at N = 192: 24 us, with these 19.6).
 // An initial update without a step gives g(x0), J(x0) and beta = 0.  Every
 // halo value is recomputed by the block that caches it from the same
 // operands as its owner uses, so all copies of a pixel are bitwise equal.
@@ -112,11 +119,6 @@ struct LoopShared {
 template <int MC>
 struct Geo {
     static constexpr int RPC = 4 * kLoopThreads / MC;  // rows per FFT group: RPC * MC = 4 * threads
-    static constexpr int CBPT = MC >= 256 ? 2 : 1;     // column groups: CBPT butterflies per thread
-    static constexpr int CPC = CBPT * RPC;
-    // the wide column group (twice the butterflies per thread), when it fits
-    static constexpr int CBPT2 = CBPT;  // (wider column groups spill registers)
-    static constexpr int CPC2 = CBPT2 * RPC;
     static constexpr int LDR = fftd::seq_len<MC>(MC);
     static constexpr int LDC = LDR + 4;
     // M = 1024: the split 512-point FFTs (fwd512 / inv512), two warps per
@@ -128,13 +130,26 @@ struct Geo {
     static constexpr int FS_COLS = 8;
     static constexpr int WA = 544;  // 16 x 33 (forward), 32 x 17 (inverse)
     static constexpr int LDF = 1090;
+    // M = 256, 512: 256-point FFTs of half a warp each (fft256), a half-warp
+    // (M = 256) or a warp, split by output parity (M = 512), a sequence.  The
+    // column pass stages H_COLS columns of at most M / 2 rows at H_LD (odd
+    // multiples of the pieces that neighbouring lanes store, for the banks) and
+    // eight warps transform; each half-warp has an exchange area of 16 x 17.
+    static constexpr bool HALFWARP = MC == 256 || MC == 512;
+    static constexpr int H_COLS = MC == 512 ? 8 : 16;
+    static constexpr int H_LD = MC == 512 ? 258 : 129;
+    static constexpr int H_AREA = 16 * 17;
+    static constexpr int H_ROWS = MC == 512 ? 8 : 16;  // rows a round of the eight warps
     static constexpr int FB_ROWS = FOURSTEP ? 16 * WA : 2 * RPC * LDR;
-    static constexpr int FB_COLS = FOURSTEP ? FS_COLS * LDF : CPC2 * LDC;
-    static constexpr int FBUF = FB_ROWS > FB_COLS ? FB_ROWS : FB_COLS;
-    // staged radix-4 twiddles (not at M = 1024), then (M = 1024) the tables
-    // T16[k2][l] = w512^(l k2) and WN[j][l] = w1024^(l + 32 j)
-    static constexpr int TW_R4 = FOURSTEP ? 0 : (fftd::staged_twiddles_size(MC) + 1) & ~1;  // 16-byte aligned
-    static constexpr int TW = TW_R4 + (FOURSTEP ? 1024 : 0);
+    static constexpr int FB_COLS = FOURSTEP ? FS_COLS * LDF : RPC * LDC;
+    static constexpr int FBUF = HALFWARP ? H_COLS * H_LD + 16 * H_AREA : FB_ROWS > FB_COLS ? FB_ROWS : FB_COLS;
+    // columns of a group of the column pass
+    static constexpr int COLS = FOURSTEP ? FS_COLS : HALFWARP ? H_COLS : RPC;
+    // staged radix-4 twiddles (M <= 128); the tables T16[k2][l] = w512^(l k2) and
+    // WN[j][l] = w1024^(l + 32 j) (M = 1024); T256[k1][l] = w256^(l k1) and
+    // w512^n (M = 256, 512)
+    static constexpr int TW_R4 = FOURSTEP || HALFWARP ? 0 : (fftd::staged_twiddles_size(MC) + 1) & ~1;  // 16-byte aligned
+    static constexpr int TW = TW_R4 + (FOURSTEP ? 1024 : HALFWARP ? 512 : 0);
 };
 
 // dynamic shared memory of one of `grid` blocks owning RB rows of an N-wide
@@ -582,6 +597,141 @@ __device__ __forceinline__ void rows_fwd_split(const float2* src, int N, int nro
     }
 }
 
+// ---------------------------------------- half-warp FFTs, M = 256 and 512
+
+// The 256-point DFT (conjugate twiddles when INV) of the sequence whose element
+// l + 16 j is in x[j] of lane l of a half-warp, both halves of the warp a
+// sequence each: DFT16 over the registers, twiddles w256^(l k1) from t, an
+// exchange through the half-warp's area (16 x 17), DFT16 over the registers.
+// Element l + 16 k of the result ends in x[k].  HALF_IN: x[8 ..] is zero.
+template <bool INV, bool HALF_IN>
+__device__ __forceinline__ void fft256(float2 (&x)[16], float2* area, const float2* t, int l)
+{
+    freg::dft16_dif<INV, HALF_IN>(x);
+#pragma unroll
+    for (int k1 = 0; k1 < 16; ++k1) {
+        const float2 w = t[k1 * 16 + l];
+        area[k1 * 17 + l] = cmul(x[freg::bitrev4(k1)], INV ? conjf2(w) : w);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = area[l * 17 + i];
+    __syncwarp();
+    freg::dft16_dif<INV>(x);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {  // bit-reversed order to the natural one (a renaming)
+        const int b = freg::bitrev4(k);
+        if (k < b) {
+            const float2 v = x[k];
+            x[k] = x[b];
+            x[b] = v;
+        }
+    }
+}
+
+// Forward transform of a sequence of M = MC points whose elements n < N <= M / 2
+// are at src (zero beyond, and all when N = 0): frequency freq(k) = l + 16 k (M =
+// 256) or 2 (l + 16 k) + h (M = 512, half h: DFT256 of x w512^(h n)) in x[k].
+template <int MC>
+__device__ __forceinline__ void half_fwd(float2 (&x)[16], const float2* src, int N, float2* area, const float2* t,
+                                         int l, int h)
+{
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if (MC == 256 && j >= 8) break;
+        const int n = l + 16 * j;
+        const float2 v = n < N ? src[n] : make_float2(0.f, 0.f);
+        x[j] = MC == 512 && h ? cmul(v, t[256 + n]) : v;
+    }
+    fft256<false, MC == 256>(x, area, t, l);
+}
+
+template <int MC>
+__device__ __forceinline__ int half_freq(int l, int h, int k)
+{
+    return MC == 512 ? 2 * (l + 16 * k) + h : l + 16 * k;
+}
+
+// The inverse of half_fwd's order: out[i], i < 8, is element l + 16 i (M = 256) or
+// l + 16 (8 h + i) (M = 512: u_0 + w512^(-n) u_1, the halves of the warp handing
+// each other what the other needs) of the transform, n < M / 2.
+template <int MC>
+__device__ __forceinline__ void half_inv(float2 (&x)[16], float2 (&out)[8], float2* area, const float2* t, int l, int h)
+{
+    fft256<true, false>(x, area, t, l);
+    if constexpr (MC == 256) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) out[i] = x[i];
+    } else {
+        if (h)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) x[k] = cmul(x[k], conjf2(t[256 + l + 16 * k]));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 give = h ? x[i] : x[8 + i], keep = h ? x[8 + i] : x[i];
+            const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 16), __shfl_xor_sync(0xffffffffu, give.y, 16));
+            out[i] = freg::add(keep, got);
+        }
+    }
+}
+
+template <int MC>
+__device__ __forceinline__ int half_elem(int l, int h, int i)
+{
+    return l + 16 * (MC == 512 ? 8 * h + i : i);
+}
+
+// Columns [x0, x0 + H_COLS) of the Toeplitz pass: staged in shared memory as row
+// pieces, a sequence each for the half-warps (M = 256) or warps (M = 512) of
+// warps 0-7, and back.
+template <int MC, typename F>
+__device__ __forceinline__ void cols_half(float2* X, int N, int x0, const float* __restrict__ Chat, const float2* t,
+                                          float2* fbuf, F&& after_staging)
+{
+    using G = Geo<MC>;
+    constexpr int E = G::H_COLS * (MC / 2) / kLoopThreads;
+    const int tid = threadIdx.x, warp = tid >> 5, h = (tid >> 4) & 1, l = tid & 15;
+    {
+        float2 v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int e = tid + i * kLoopThreads, y = e / G::H_COLS, c = e % G::H_COLS;
+            v[i] = y < N ? __ldcg(X + (int64_t)y * MC + x0 + c) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int e = tid + i * kLoopThreads;
+            fbuf[(e % G::H_COLS) * G::H_LD + e / G::H_COLS] = v[i];
+        }
+    }
+    const int c = MC == 512 ? warp : 2 * warp + h;  // column of the group
+    float hs[16];
+    if (warp < 8) {
+        const float* ch = Chat + (int64_t)(x0 + c) * MC;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) hs[k] = __ldcg(ch + half_freq<MC>(l, h, k));
+    }
+    __syncthreads();
+    after_staging();
+    if (warp < 8) {
+        float2* area = fbuf + G::H_COLS * G::H_LD + (tid >> 4) * G::H_AREA;
+        float2* col = fbuf + c * G::H_LD;
+        float2 x[16], y[8];
+        half_fwd<MC>(x, col, N, area, t, l, h);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = make_float2(x[k].x * hs[k], x[k].y * hs[k]);
+        half_inv<MC>(x, y, area, t, l, h);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) col[half_elem<MC>(l, h, i)] = y[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const int e = tid + i * kLoopThreads, y = e / G::H_COLS, cc = e % G::H_COLS;
+        if (y < N) X[(int64_t)y * MC + x0 + cc] = fbuf[cc * G::H_LD + y];
+    }
+}
+
 // ---------------------------------------------------------------- phase A
 
 // Gradient of every own pixel (phi fixed at compile time): g into the
@@ -772,6 +922,25 @@ __device__ __forceinline__ void phase_update(const LoopArgs& A, const Rows& R, f
                 rows_fwd_split(cg + g0 * N, N, min(8, R.nown - g0), A.X + (int64_t)(R.R0 + g0) * MC, fbuf, stw,
                                stw + 512);
         }
+    } else if constexpr (G::HALFWARP) {
+        // gradient of every own pixel, then the row FFTs of g by eight warps
+        grad_rows_any<FIRST>(A, R, cf, cd, cRes, cD, cg, a);
+        if (do_fft) {
+            __syncthreads();  // g of every own row is in cg
+            const int warp = threadIdx.x >> 5, h = (threadIdx.x >> 4) & 1, l = threadIdx.x & 15;
+            if (warp < 8)
+                for (int g0 = 0; g0 < R.nown; g0 += G::H_ROWS) {
+                    const int q = g0 + (MC == 512 ? warp : 2 * warp + h);
+                    const bool own = q < R.nown;
+                    float2 x[16];
+                    half_fwd<MC>(x, cg + q * N, own ? N : 0, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw,
+                                 l, h);
+                    float2* out = A.X + (int64_t)(R.R0 + q) * MC;
+                    if (own)
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) out[half_freq<MC>(l, h, k)] = x[k];
+                }
+        }
     } else {
         // gradient of every own pixel, then the row FFTs of g, RX * RPC rows
         // at a time
@@ -849,7 +1018,33 @@ __device__ __forceinline__ void phase_rows(const LoopArgs& A, const Rows& R, flo
 {
     using G = Geo<MC>;
     const int N = R.N;
-    const bool dir_aside = G::FOURSTEP && R.nown <= 4;  // warps 8 .. 15 have no row to transform
+    const bool dir_aside = G::HALFWARP || (G::FOURSTEP && R.nown <= 4);  // warps 8 .. 15 have no row to transform
+    if constexpr (G::HALFWARP) {
+        // the row IFFTs of Y by warps 0-7, the new direction by the others
+        const int warp = threadIdx.x >> 5, h = (threadIdx.x >> 4) & 1, l = threadIdx.x & 15;
+        if (warp >= 8) {
+            direction_rows(A.g, R, cd, cg, beta, restart, (int)threadIdx.x - 256, kLoopThreads - 256);
+        } else {
+            for (int g0 = 0; g0 < R.nown; g0 += G::H_ROWS) {
+                const int q = g0 + (MC == 512 ? warp : 2 * warp + h);
+                const bool own = q < R.nown;
+                const float2* yr = A.X + (int64_t)(R.R0 + q) * MC;
+                float2 x[16], tg[8];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) x[k] = own ? __ldcg(yr + half_freq<MC>(l, h, k)) : make_float2(0.f, 0.f);
+                half_inv<MC>(x, tg, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int m = half_elem<MC>(l, h, i);
+                    if (own && m < N) {
+                        float2& td = cTd[q * N + m];
+                        td = fftd::new_direction(tg[i], td, beta, restart);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
     if constexpr (G::FOURSTEP) {
         // the split row IFFTs of Y, two warps a row (warp 2 q + h takes the
         // elements 2 k + h), eight rows at a time: T g = u_0 + w1024^(-m) u_1
@@ -898,7 +1093,7 @@ __device__ __forceinline__ void phase_rows(const LoopArgs& A, const Rows& R, flo
             __syncthreads();
         }
     }
-    for (int g0 = 0; g0 < (G::FOURSTEP ? 0 : R.nown); g0 += RX * G::RPC) {
+    for (int g0 = 0; g0 < (G::FOURSTEP || G::HALFWARP ? 0 : R.nown); g0 += RX * G::RPC) {
         const int nr = min(RX * G::RPC, R.nown - g0);
         float2 v[4 * RX];
 #pragma unroll
@@ -971,13 +1166,10 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
     float2* cTd = cg + RB * N;
     float2* pbuf = cTd + RB * N;  // deferred update partials (kUpdVals x even (grid + 1))
     pbuf += ((uintptr_t)pbuf & 15) ? 1 : 0;  // 16-byte copies
-    // column groups: the wide ones when every block still gets one
-    const bool wide_cols = G::CBPT2 > G::CBPT && MC / G::CPC2 >= (int)gridDim.x;
-    const int cpc = G::FOURSTEP ? G::FS_COLS : wide_cols ? G::CPC2 : G::CPC;
-    const int col_groups = MC / cpc;
-    // rows: two FFT groups per batch (the split FFTs of M = 1024 have no groups)
-    const bool rx2 = !G::FOURSTEP && RB >= 2 * G::RPC;
-    constexpr int RX2 = G::FOURSTEP ? 1 : 2;
+    constexpr int cpc = G::COLS, col_groups = MC / cpc;
+    // rows: two FFT groups per batch (the register FFTs of M >= 256 have no such groups)
+    const bool rx2 = !G::FOURSTEP && !G::HALFWARP && RB >= 2 * G::RPC;
+    constexpr int RX2 = G::FOURSTEP || G::HALFWARP ? 1 : 2;
     const bool prof = blockIdx.x == 0;
     unsigned seq = 0;
     float t_f = 0.f;  // the current line-search step, the same in every thread
@@ -1001,6 +1193,12 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             for (int e = threadIdx.x; e < 512; e += kLoopThreads) {
                 stw[e] = __ldg(A.tw + ((2 * (e & 31) * (e >> 5)) & (MC - 1)));
                 stw[512 + e] = __ldg(A.tw + e);
+            }
+        } else if constexpr (G::HALFWARP) {
+            // T256[k1][l] = w256^(l k1), then w512^n
+            for (int e = threadIdx.x; e < 256; e += kLoopThreads) {
+                stw[e] = __ldg(A.tw + (MC / 256) * (e & 15) * (e >> 4));
+                if (MC == 512) stw[256 + e] = __ldg(A.tw + e);
             }
         } else {
             fftd::build_staged_twiddles<MC>(A.tw, stw);
@@ -1062,16 +1260,16 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
             if (!CL && fetch) deferred_parts_fetch<kUpdVals>(A.parts, L_A, pbuf);
             fetch = false;
         };
-        if constexpr (!G::FOURSTEP) fetch_parts();
+        if constexpr (!G::FOURSTEP && !G::HALFWARP) fetch_parts();
         // ---- B: columns
         for (int gi = blockIdx.x; gi < col_groups; gi += gridDim.x) {
             const int x0 = gi * cpc;
             if constexpr (G::FOURSTEP)
                 cols_split(A.X, N, x0, A.Chat, stw, stw + 512, fbuf, fetch_parts);
-            else if (wide_cols)
-                fftd::cols_group<MC, G::CBPT2, 1>(A.X, N, N, x0, cpc, cpc, A.fp, stw, A.Chat, fbuf, nullptr);
+            else if constexpr (G::HALFWARP)
+                cols_half<MC>(A.X, N, x0, A.Chat, stw, fbuf, fetch_parts);
             else
-                fftd::cols_group<MC, G::CBPT, 1>(A.X, N, N, x0, cpc, cpc, A.fp, stw, A.Chat, fbuf, nullptr);
+                fftd::cols_group<MC, 1, 1>(A.X, N, N, x0, cpc, cpc, A.fp, stw, A.Chat, fbuf, nullptr);
             // the next group refills fbuf (after the last one, the
             // synchronisation below starts with a block barrier)
             if (gi + (int)gridDim.x < col_groups) __syncthreads();
@@ -1228,7 +1426,7 @@ bool loop_cap(size_t* cap_out)
 
 // Columns of a group of the column pass, and their number.
 template <int MC>
-constexpr int loop_col_groups() { return MC / (Geo<MC>::FOURSTEP ? Geo<MC>::FS_COLS : Geo<MC>::CPC); }
+constexpr int loop_col_groups() { return MC / Geo<MC>::COLS; }
 
 // Rows per block of the i-th shape, i < kMaxGroupsPerBlock: whole row-FFT
 // groups, or at M = 1024, whose row FFTs take two warps a row, any number.

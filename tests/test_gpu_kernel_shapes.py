@@ -173,3 +173,20 @@ def test_loop_grids(sp, monkeypatch, N, M):
         monkeypatch.setenv("SPIREC_NO_LOOP", "1")
         y, Jy = sp.spirec_solve(p.h, x0, 3, N)
     assert rel(x, y) < 1e-5 and rel(J, Jy) < 1e-5
+
+
+# The loop's half-warp FFTs (M = 256, 512) at the edges of their ranges: the
+# smallest image of each grid, one short of the largest and the largest.
+# Distance as above.
+@pytest.mark.parametrize("N,M", [(65, 0), (72, 512), (127, 0), (128, 0), (129, 0), (255, 0), (256, 0)])
+def test_loop_half_warp_ffts(sp, monkeypatch, N, M):
+    g = synth.rng(N)
+    kx, ky = synth.spiral(N, 4, 1100, "variable")
+    s = synth.complex_normal(kx.shape[0], g).astype(np.complex64)
+    with sp.Plan(N, kx.shape[0], M, 1, _stream(), kx, ky) as p:
+        sp.spirec_set_data(p.h, s)
+        sp.spirec_set_reg(p.h, 0.05, 0.05, 0.02, 0.1, 0)
+        x, J = sp.spirec_solve(p.h, None, 3, N)
+        monkeypatch.setenv("SPIREC_NO_LOOP", "1")
+        y, Jy = sp.spirec_solve(p.h, None, 3, N)
+    assert rel(x, y) < 1e-5 and rel(J, Jy) < 1e-5
