@@ -13,6 +13,7 @@
 #include <new>
 #include <vector>
 
+#include "chain.cuh"
 #include "internal.cuh"
 
 // the per-interleave kernel cache (spirec_kcache_*)
@@ -62,6 +63,7 @@ __global__ void k_traj_fixed(const double* __restrict__ kx, const double* __rest
                              int64_t L, int64_t* __restrict__ kxq, int64_t* __restrict__ kyq,
                              int* flag)
 {
+    chain_next();
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < L;
          l += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll

@@ -1,10 +1,12 @@
 // chain.cuh -- kernels that follow each other on one stream without a gap
 // (programmatic dependent launch).  A kernel launched by `chain` may be placed
 // on the device before its predecessor has ended: from the predecessor's
-// chain_next on, else as its blocks exit.  chain_enter, its first statement,
-// waits until the predecessor has completed and its writes are visible.
-// chain_next comes after chain_enter, so at most two kernels of a chain overlap
-// and everything from before the predecessor is complete when a kernel starts.
+// chain_next on, else as its blocks exit.  chain_enter, its first statement (or
+// the first after a set-up that reads no global memory: barriers, tensor
+// memory), waits until the predecessor has completed and its writes are visible.
+// chain_next comes after chain_enter, or in a kernel with a plain launch, so at
+// most two kernels of a chain overlap and everything from before the
+// predecessor is complete when a kernel starts.
 // What the predecessor wrote must not be read through the read-only path (__ldg,
 // const __restrict__): the compiler may move such loads above the wait.
 //

@@ -522,10 +522,11 @@ k_rows_inv_split(const float2* __restrict__ X, int N, int ldx, float2* __restric
 
 // Rows u of G's half, conjugated, at v mod M: T[u][ky] to X[u * M + split_pos(ky)].
 template <int MC>
-__global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict__ G, int N, float2* X, FftPlan fp,
+__global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* G, int N, float2* X, FftPlan fp,
                                                         const float2* __restrict__ tw, int rpc)
 {
     extern __shared__ float2 sm[];
+    chain_enter();
     const int M = fp.M, ld = seq_len<MC>(M), W = 2 * N - 1;
     float2* a = sm;
     float2* b = sm + rpc * ld;
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict
         const int v = y < N ? y : y - M;  // -N < v < N holds a lag
         float2 c = make_float2(0.f, 0.f);
         if (q < nr && v > -N) {
-            const float2 g = __ldg(G + (int64_t)(u0 + q) * W + (v + N - 1));
+            const float2 g = G[(int64_t)(u0 + q) * W + (v + N - 1)];
             c = make_float2(g.x, -g.y);
         }
         a[q * ld + sidx<MC>(y)] = c;
@@ -552,10 +553,11 @@ __global__ void __launch_bounds__(1024) k_rows_spectrum(const float2* __restrict
 // out[kx * M + ky], both by split_pos (Chat), or out[ky * M + kx] (ROWS_KY, the
 // caller's grid when it is not a power of two).
 template <int MC, bool ROWS_KY>
-__global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* __restrict__ X, int N, FftPlan fp, const float2* __restrict__ tw,
+__global__ void __launch_bounds__(1024) k_cols_spectrum(const float2* X, int N, FftPlan fp, const float2* __restrict__ tw,
                                 float* out, int cpc)
 {
     extern __shared__ float2 sm[];
+    chain_enter();
     const int M = fp.M;
     const int ld = seq_len<MC>(M) + 4;
     float2* a = sm;
@@ -774,14 +776,12 @@ struct LaunchSpectrum {
     int operator()()
     {
         const int M = fp->M, N = p->N;
-        k_rows_spectrum<MC><<<(N + rs.per_cta - 1) / rs.per_cta, rs.threads, rs.smem, p->stream>>>(
-            p->G, N, p->cwork, *fp, tw, rs.per_cta);
+        chain(k_rows_spectrum<MC>, dim3((N + rs.per_cta - 1) / rs.per_cta), dim3(rs.threads), rs.smem, p->stream, p->G, N,
+              p->cwork, *fp, tw, rs.per_cta);
         SPIREC_CK(cudaGetLastError());
         const int blocks = (M + cs.per_cta - 1) / cs.per_cta;
-        if (rows_ky)
-            k_cols_spectrum<MC, true><<<blocks, cs.threads, cs.smem, p->stream>>>(p->cwork, N, *fp, tw, out, cs.per_cta);
-        else
-            k_cols_spectrum<MC, false><<<blocks, cs.threads, cs.smem, p->stream>>>(p->cwork, N, *fp, tw, out, cs.per_cta);
+        chain(rows_ky ? k_cols_spectrum<MC, true> : k_cols_spectrum<MC, false>, dim3(blocks), dim3(cs.threads), cs.smem, p->stream,
+              p->cwork, N, *fp, tw, out, cs.per_cta);
         SPIREC_CK(cudaGetLastError());
         p->launches += 2;
         return SPIREC_OK;

@@ -70,6 +70,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "internal.cuh"
 #include "phase.cuh"
 #include "reduce.cuh"
@@ -626,8 +627,7 @@ struct SegWalk {
 // barrier at the same offset in both CTAs.
 template <bool BF16, bool WEIGHTED, bool PAIR>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-k_tc_pair_gemm(const int64_t* __restrict__ ka, const int64_t* __restrict__ kb, const float2* __restrict__ w,
-               const unsigned* __restrict__ amax2, int64_t L, int tilesC, int oa, int sa, int sb, int half, int J,
+k_tc_pair_gemm(const int64_t* ka, const int64_t* kb, const float2* w, const unsigned* amax2, int64_t L, int tilesC, int oa, int sa, int sb, int half, int J,
                int64_t K, int64_t U, float* __restrict__ part, int* err, unsigned long long wait_ns, int stall)
 {
     using SH = PairShape<PAIR>;
@@ -674,6 +674,7 @@ k_tc_pair_gemm(const int64_t* __restrict__ ka, const int64_t* __restrict__ kb, c
     if constexpr (PAIR) cluster_sync();  // both CTAs' barriers are initialised before any arrival from the other
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    chain_enter();  // the predecessor's samples or weights are read from here on
 
     if (warp < TC_PRODUCERS / 32) {
         // ------------------------------------------------ producers
@@ -982,14 +983,15 @@ k_tc_pair_gemm(const int64_t* __restrict__ ka, const int64_t* __restrict__ kb, c
 // other, on 64 SMs (48 us at N = 250, L = 31665 for 40 MB of L2-resident
 // partials).  launch_reduce picks the shape.
 template <int TY, int S>
-__global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* __restrict__ part, int64_t U, int64_t K,
+__global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* part, int64_t U, int64_t K,
                                                              int64_t P, bool pairs, PairGeom pg, int tilesC,
-                                                             float scale, const unsigned* __restrict__ amax2,
+                                                             float scale, const unsigned* amax2,
                                                              float2* __restrict__ out)
 {
     constexpr int W = 4 * TY;  // columns of the patch
     __shared__ float2 patch[W][33];
     __shared__ float4 sums[S > 1 ? 2 * (S - 1) * TY * 32 : 1];
+    chain_enter();
     const int i0 = blockIdx.y * 32;
     const int tcol = blockIdx.x / (TC_COLS / W), q0 = (blockIdx.x % (TC_COLS / W)) * W;  // tile column, first partial column
     if (tcol * PG_COLS + (q0 & (PG_COLS - 1)) >= pg.J) return;  // no output column in the patch
@@ -1068,6 +1070,22 @@ __global__ void __launch_bounds__(32 * TY * S) k_reduce_pair(const float* __rest
     }
 }
 
+// The largest of a block's 256 values (warps whose own largest is not finite do
+// not count), in every thread.
+__device__ __forceinline__ float block_max(float m)
+{
+    __shared__ float wmax[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = isfinite(m) ? m : 0.f;
+    __syncthreads();
+    m = wmax[0];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) m = fmaxf(m, wmax[k]);
+    __syncthreads();
+    return m;
+}
+
 // w'_l = w_l exp(sb i2pi (kb_l / 2) shift2) for l < L (the weight of the
 // original B operand and the phase of the pairing's centre column); the plan's
 // buffer keeps its zero padding past L.  The last block writes amax2 = max_l
@@ -1080,6 +1098,7 @@ __global__ void __launch_bounds__(256) k_pair_weights(const float2* w, const int
                                                       int shift2, float2* __restrict__ wp, float2* s, float2* parts,
                                                       unsigned* counter, unsigned* amax2, double* scal)
 {
+    chain_next();
     float mx = 0.f, ss = 0.f;
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < L; l += (int64_t)gridDim.x * blockDim.x) {
         float2 e = phasor_q(kb[l] >> 1, shift2);
@@ -1093,18 +1112,6 @@ __global__ void __launch_bounds__(256) k_pair_weights(const float2* w, const int
             ss += fmaf(u.x, u.x, u.y * u.y);
         }
     }
-    __shared__ float wmax[8];
-    auto block_max = [&](float m) {  // of the 8 warps, valid in thread 0
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = isfinite(m) ? m : 0.f;
-        __syncthreads();
-        m = wmax[0];
-#pragma unroll
-        for (int k = 1; k < 8; ++k) m = fmaxf(m, wmax[k]);
-        __syncthreads();
-        return m;
-    };
     const float bm = block_max(mx);
     if (threadIdx.x == 0) parts[kMaxParts + blockIdx.x] = make_float2(bm, 0.f);
     if (DATA) {
@@ -1200,9 +1207,11 @@ __host__ __device__ __forceinline__ FwGeom fw_geom(int N)
 // 2^-(e+1), 2^e >= max |f| (amax2 = max |f|^2), so the FP16 halves stay in
 // range; k_tc_forward undoes the scale.
 template <bool BF16>
-__global__ void k_split_image(const float2* __restrict__ f, FwGeom fg, const unsigned* __restrict__ amax2,
+__global__ void k_split_image(const float2* __restrict__ f, FwGeom fg, const unsigned* amax2,
                               uint8_t* __restrict__ FB)
 {
+    chain_enter();
+    chain_next();
     const float wmul = 0.5f * weight_scale_inv(amax2);
     const int N = fg.N, cols = fg.mtiles * fg.mw;
     const int64_t total = (int64_t)cols * fg.kchunks * 4;  // (m, chunk, group of 8 j)
@@ -1252,7 +1261,7 @@ __global__ void k_split_image(const float2* __restrict__ f, FwGeom fg, const uns
 template <bool BF16>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_tc_forward(const int64_t* __restrict__ kxq, const int64_t* __restrict__ kyq, const uint8_t* __restrict__ FB,
-             const unsigned* __restrict__ amax2, int64_t L, FwGeom fg, float scale, float2* __restrict__ y, int* err,
+             const unsigned* amax2, int64_t L, FwGeom fg, float scale, float2* __restrict__ y, int* err,
              unsigned long long wait_ns, int stall)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -1300,6 +1309,7 @@ k_tc_forward(const int64_t* __restrict__ kxq, const int64_t* __restrict__ kyq, c
     cluster_sync();  // both CTAs' barriers are initialised before any arrival from the other
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    chain_enter();  // the split image is read from here on
 
     if (warp < TC_PRODUCERS / 32) {
         // ------------------------------------------------ producers
@@ -1535,18 +1545,29 @@ k_tc_forward(const int64_t* __restrict__ kxq, const int64_t* __restrict__ kyq, c
     }
 }
 
-// amax2 = max_l |y_l|^2 as float bits (non-negative floats order like unsigned).
-__global__ void k_absmax2(const float2* __restrict__ y, int64_t n, unsigned* amax2)
+// amax2 = max_l |y_l|^2 as float bits (warps that met a value that is not finite
+// do not count), by the last block: no clear before the kernel.
+__global__ void __launch_bounds__(256) k_absmax2(const float2* __restrict__ y, int64_t n, float2* parts, unsigned* counter,
+                                                 unsigned* amax2)
 {
+    chain_next();
     float m = 0.f;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float2 v = y[i];
         m = fmaxf(m, fmaf(v.x, v.x, v.y * v.y));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && isfinite(m)) atomicMax(amax2, __float_as_uint(m));
+    m = block_max(m);
+    if (threadIdx.x == 0) parts[blockIdx.x] = make_float2(m, 0.f);
+    if (last_block(counter)) {
+        m = 0.f;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) m = fmaxf(m, __ldcg(parts + i).x);
+        m = block_max(m);
+        if (threadIdx.x == 0) {
+            *amax2 = __float_as_uint(m);
+            *counter = 0u;
+        }
+    }
 }
 
 // Clusters of two k_tc_pair_gemm CTAs the device runs at once (cached per
@@ -1587,17 +1608,19 @@ cudaError_t launch_pair_kernel(int64_t P, cudaStream_t stream, const int64_t* ka
                                int64_t K, int64_t U, float* part, int* err, unsigned long long wait_ns, int stall)
 {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (see chain.cuh)
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)P);
     cfg.blockDim = dim3(TC_THREADS);
     cfg.dynamicSmemBytes = PairShape<PAIR>::SMEM;
     cfg.stream = stream;
-    cfg.attrs = PAIR ? at : nullptr;
-    cfg.numAttrs = PAIR ? 1 : 0;
+    cfg.attrs = at;
+    cfg.numAttrs = PAIR ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, k_tc_pair_gemm<BF16, WEIGHTED, PAIR>, ka, kb, w, amax, L, tilesC, oa, sa, sb, half,
                               J, K, U, part, err, wait_ns, stall);
 }
@@ -1626,7 +1649,7 @@ void launch_reduce_shape(cudaStream_t st, const float* part, int64_t U, int64_t 
                          const PairGeom& pg, int tilesC, float scale, const unsigned* amax2, float2* out)
 {
     const dim3 grid((unsigned)(tilesC * (TC_COLS / (4 * TY))), (unsigned)((pg.R + 31) / 32));
-    k_reduce_pair<TY, S><<<grid, dim3(32, TY, S), 0, st>>>(part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
+    chain(k_reduce_pair<TY, S>, grid, dim3(32, TY, S), 0, st, part, U, K, P, pairs, pg, tilesC, scale, amax2, out);
 }
 
 // The shape of k_reduce_pair by the owners of a tile, P / T: how many partials
@@ -1745,18 +1768,16 @@ int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
     unsigned* amax = p->counters + C_AMAX;
     {
         const int64_t NN = (int64_t)N * N;
-        SPIREC_CK(cudaMemsetAsync(amax, 0, sizeof(unsigned), p->stream));
         int blocks = (int)((NN + 255) / 256);
         if (blocks > 4 * kMaxCtas) blocks = 4 * kMaxCtas;
-        k_absmax2<<<blocks, 256, 0, p->stream>>>(x, NN, amax);
+        k_absmax2<<<blocks, 256, 0, p->stream>>>(x, NN, reinterpret_cast<float2*>(p->part) + (size_t)P_MISC * kMaxParts,
+                                                 p->counters + C_MISC, amax);
         SPIREC_CK(cudaGetLastError());
         const int64_t total = (int64_t)fg.mtiles * fg.mw * fg.kchunks * 4;
         blocks = (int)((total + 255) / 256);
         if (blocks > 8 * kMaxCtas) blocks = 8 * kMaxCtas;
-        if (bf16)
-            k_split_image<true><<<blocks, 256, 0, p->stream>>>(x, fg, amax, p->fsplit);
-        else
-            k_split_image<false><<<blocks, 256, 0, p->stream>>>(x, fg, amax, p->fsplit);
+        chain(bf16 ? k_split_image<true> : k_split_image<false>, dim3((unsigned)blocks), dim3(256), 0, p->stream, x, fg, amax,
+              p->fsplit);
         SPIREC_CK(cudaGetLastError());
     }
     int sms = 0, clusters = 0, rc;
@@ -1767,17 +1788,19 @@ int launch_forward_tc(spirec_plan p, const float2* x, float2* yout)
     if (P2 > clusters) P2 = clusters;
     if (P2 > ntiles) P2 = ntiles;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (see chain.cuh)
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)(2 * P2));
     cfg.blockDim = dim3(TC_THREADS);
     cfg.dynamicSmemBytes = FW_SMEM;
     cfg.stream = p->stream;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const float scale = 1.0f / (float)N;
     const int stall = injected_stall(kStallContraction) ? 1 : 0;
     const uint8_t* fb = p->fsplit;
