@@ -67,6 +67,7 @@
 
 #include "cg_device.cuh"
 #include "fft_device.cuh"
+#include "fft_half.cuh"
 #include "fft_reg.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
@@ -130,15 +131,15 @@ struct Geo {
     static constexpr int FS_COLS = 8;
     static constexpr int WA = 544;  // 16 x 33 (forward), 32 x 17 (inverse)
     static constexpr int LDF = 1090;
-    // M = 256, 512: 256-point FFTs of half a warp each (fft256), a half-warp
+    // M = 256, 512: 256-point FFTs of half a warp each (fft_half.cuh), a half-warp
     // (M = 256) or a warp, split by output parity (M = 512), a sequence.  The
     // column pass stages H_COLS columns of at most M / 2 rows at H_LD (odd
     // multiples of the pieces that neighbouring lanes store, for the banks) and
     // eight warps transform; each half-warp has an exchange area of 16 x 17.
-    static constexpr bool HALFWARP = MC == 256 || MC == 512;
+    static constexpr bool HALFWARP = fftd::half_warp_size<MC>();
     static constexpr int H_COLS = MC == 512 ? 8 : 16;
     static constexpr int H_LD = MC == 512 ? 258 : 129;
-    static constexpr int H_AREA = 16 * 17;
+    static constexpr int H_AREA = fftd::kHalfArea;
     static constexpr int H_ROWS = MC == 512 ? 8 : 16;  // rows a round of the eight warps
     static constexpr int FB_ROWS = FOURSTEP ? 16 * WA : 2 * RPC * LDR;
     static constexpr int FB_COLS = FOURSTEP ? FS_COLS * LDF : RPC * LDC;
@@ -149,7 +150,7 @@ struct Geo {
     // WN[j][l] = w1024^(l + 32 j) (M = 1024); T256[k1][l] = w256^(l k1) and
     // w512^n (M = 256, 512)
     static constexpr int TW_R4 = FOURSTEP || HALFWARP ? 0 : (fftd::staged_twiddles_size(MC) + 1) & ~1;  // 16-byte aligned
-    static constexpr int TW = TW_R4 + (FOURSTEP ? 1024 : HALFWARP ? 512 : 0);
+    static constexpr int TW = TW_R4 + (FOURSTEP ? 1024 : HALFWARP ? fftd::kHalfTables : 0);
 };
 
 // dynamic shared memory of one of `grid` blocks owning RB rows of an N-wide
@@ -599,88 +600,6 @@ __device__ __forceinline__ void rows_fwd_split(const float2* src, int N, int nro
 
 // ---------------------------------------- half-warp FFTs, M = 256 and 512
 
-// The 256-point DFT (conjugate twiddles when INV) of the sequence whose element
-// l + 16 j is in x[j] of lane l of a half-warp, both halves of the warp a
-// sequence each: DFT16 over the registers, twiddles w256^(l k1) from t, an
-// exchange through the half-warp's area (16 x 17), DFT16 over the registers.
-// Element l + 16 k of the result ends in x[k].  HALF_IN: x[8 ..] is zero.
-template <bool INV, bool HALF_IN>
-__device__ __forceinline__ void fft256(float2 (&x)[16], float2* area, const float2* t, int l)
-{
-    freg::dft16_dif<INV, HALF_IN>(x);
-#pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) {
-        const float2 w = t[k1 * 16 + l];
-        area[k1 * 17 + l] = cmul(x[freg::bitrev4(k1)], INV ? conjf2(w) : w);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = area[l * 17 + i];
-    __syncwarp();
-    freg::dft16_dif<INV>(x);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {  // bit-reversed order to the natural one (a renaming)
-        const int b = freg::bitrev4(k);
-        if (k < b) {
-            const float2 v = x[k];
-            x[k] = x[b];
-            x[b] = v;
-        }
-    }
-}
-
-// Forward transform of a sequence of M = MC points whose elements n < N <= M / 2
-// are at src (zero beyond, and all when N = 0): frequency freq(k) = l + 16 k (M =
-// 256) or 2 (l + 16 k) + h (M = 512, half h: DFT256 of x w512^(h n)) in x[k].
-template <int MC>
-__device__ __forceinline__ void half_fwd(float2 (&x)[16], const float2* src, int N, float2* area, const float2* t,
-                                         int l, int h)
-{
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        if (MC == 256 && j >= 8) break;
-        const int n = l + 16 * j;
-        const float2 v = n < N ? src[n] : make_float2(0.f, 0.f);
-        x[j] = MC == 512 && h ? cmul(v, t[256 + n]) : v;
-    }
-    fft256<false, MC == 256>(x, area, t, l);
-}
-
-template <int MC>
-__device__ __forceinline__ int half_freq(int l, int h, int k)
-{
-    return MC == 512 ? 2 * (l + 16 * k) + h : l + 16 * k;
-}
-
-// The inverse of half_fwd's order: out[i], i < 8, is element l + 16 i (M = 256) or
-// l + 16 (8 h + i) (M = 512: u_0 + w512^(-n) u_1, the halves of the warp handing
-// each other what the other needs) of the transform, n < M / 2.
-template <int MC>
-__device__ __forceinline__ void half_inv(float2 (&x)[16], float2 (&out)[8], float2* area, const float2* t, int l, int h)
-{
-    fft256<true, false>(x, area, t, l);
-    if constexpr (MC == 256) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) out[i] = x[i];
-    } else {
-        if (h)
-#pragma unroll
-            for (int k = 0; k < 16; ++k) x[k] = cmul(x[k], conjf2(t[256 + l + 16 * k]));
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 give = h ? x[i] : x[8 + i], keep = h ? x[8 + i] : x[i];
-            const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 16), __shfl_xor_sync(0xffffffffu, give.y, 16));
-            out[i] = freg::add(keep, got);
-        }
-    }
-}
-
-template <int MC>
-__device__ __forceinline__ int half_elem(int l, int h, int i)
-{
-    return l + 16 * (MC == 512 ? 8 * h + i : i);
-}
-
 // Columns [x0, x0 + H_COLS) of the Toeplitz pass: staged in shared memory as row
 // pieces, a sequence each for the half-warps (M = 256) or warps (M = 512) of
 // warps 0-7, and back.
@@ -709,7 +628,7 @@ __device__ __forceinline__ void cols_half(float2* X, int N, int x0, const float*
     if (warp < 8) {
         const float* ch = Chat + (int64_t)(x0 + c) * MC;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) hs[k] = __ldcg(ch + half_freq<MC>(l, h, k));
+        for (int k = 0; k < 16; ++k) hs[k] = __ldcg(ch + fftd::half_freq<MC>(l, h, k));
     }
     __syncthreads();
     after_staging();
@@ -717,12 +636,12 @@ __device__ __forceinline__ void cols_half(float2* X, int N, int x0, const float*
         float2* area = fbuf + G::H_COLS * G::H_LD + (tid >> 4) * G::H_AREA;
         float2* col = fbuf + c * G::H_LD;
         float2 x[16], y[8];
-        half_fwd<MC>(x, col, N, area, t, l, h);
+        fftd::half_fwd<MC>(x, [&](int n) { return col[n]; }, N, area, t, l, h);
 #pragma unroll
         for (int k = 0; k < 16; ++k) x[k] = make_float2(x[k].x * hs[k], x[k].y * hs[k]);
-        half_inv<MC>(x, y, area, t, l, h);
+        fftd::half_inv<MC>(x, y, area, t, l, h);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) col[half_elem<MC>(l, h, i)] = y[i];
+        for (int i = 0; i < 8; ++i) col[fftd::half_elem<MC>(l, h, i)] = y[i];
     }
     __syncthreads();
 #pragma unroll
@@ -933,12 +852,13 @@ __device__ __forceinline__ void phase_update(const LoopArgs& A, const Rows& R, f
                     const int q = g0 + (MC == 512 ? warp : 2 * warp + h);
                     const bool own = q < R.nown;
                     float2 x[16];
-                    half_fwd<MC>(x, cg + q * N, own ? N : 0, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw,
-                                 l, h);
+                    const float2* row = cg + q * N;
+                    fftd::half_fwd<MC>(x, [&](int n) { return row[n]; }, own ? N : 0,
+                                       fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
                     float2* out = A.X + (int64_t)(R.R0 + q) * MC;
                     if (own)
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) out[half_freq<MC>(l, h, k)] = x[k];
+                        for (int k = 0; k < 16; ++k) out[fftd::half_freq<MC>(l, h, k)] = x[k];
                 }
         }
     } else {
@@ -1031,11 +951,11 @@ __device__ __forceinline__ void phase_rows(const LoopArgs& A, const Rows& R, flo
                 const float2* yr = A.X + (int64_t)(R.R0 + q) * MC;
                 float2 x[16], tg[8];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) x[k] = own ? __ldcg(yr + half_freq<MC>(l, h, k)) : make_float2(0.f, 0.f);
-                half_inv<MC>(x, tg, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
+                for (int k = 0; k < 16; ++k) x[k] = own ? __ldcg(yr + fftd::half_freq<MC>(l, h, k)) : make_float2(0.f, 0.f);
+                fftd::half_inv<MC>(x, tg, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const int m = half_elem<MC>(l, h, i);
+                    const int m = fftd::half_elem<MC>(l, h, i);
                     if (own && m < N) {
                         float2& td = cTd[q * N + m];
                         td = fftd::new_direction(tg[i], td, beta, restart);
@@ -1195,11 +1115,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(LoopArgs A)
                 stw[512 + e] = __ldg(A.tw + e);
             }
         } else if constexpr (G::HALFWARP) {
-            // T256[k1][l] = w256^(l k1), then w512^n
-            for (int e = threadIdx.x; e < 256; e += kLoopThreads) {
-                stw[e] = __ldg(A.tw + (MC / 256) * (e & 15) * (e >> 4));
-                if (MC == 512) stw[256 + e] = __ldg(A.tw + e);
-            }
+            fftd::half_tables<MC>(stw, A.tw);
         } else {
             fftd::build_staged_twiddles<MC>(A.tw, stw);
         }

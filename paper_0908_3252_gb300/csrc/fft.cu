@@ -30,6 +30,7 @@
 
 #include "chain.cuh"
 #include "fft_device.cuh"
+#include "fft_half.cuh"
 #include "fft_reg.cuh"
 #include "internal.cuh"
 #include "phase.cuh"
@@ -60,16 +61,42 @@ namespace {
 
 using namespace fftd;
 
+// Threads of a T pass's block, at most.
+template <int MC>
+__host__ __device__ constexpr int t_threads() { return half_warp_size<MC>() ? 128 : 1024; }
+
 // ------------------------------------------------------------- row pass 1
 
-// Row FFTs of `in` (n_in nonzero entries a row) into X.
+// Row FFTs of `in` (n_in nonzero entries a row) into X.  At M = 256 and 512 the T
+// passes are register transforms (fft_half.cuh) whose tables are loaded before the
+// wait for the predecessor: latency bounds these passes (loads, one exchange,
+// stores), and the radix-4 stages with a block barrier each added to it.  T at N =
+// 256, M = 512 15.6 us with radix-4 stages, now 11.0; at N = 128, M = 256 9.7 and
+// 8.6.
 template <int MC>
-__global__ void __launch_bounds__(1024) k_rows_fwd(const float2* in, int ld_in, int n_in, int rows, float2* X, FftPlan fp,
+__global__ void __launch_bounds__(t_threads<MC>()) k_rows_fwd(const float2* in, int ld_in, int n_in, int rows, float2* X, FftPlan fp,
                            const float2* __restrict__ tw, int rpc)
 {
+    extern __shared__ float2 sm[];
+    if constexpr (half_warp_size<MC>()) {
+        half_tables<MC>(sm, tw);
+        chain_enter();
+        chain_next();
+        __syncthreads();
+        const int l = threadIdx.x & 15, h = (threadIdx.x >> 4) & 1;
+        const int q = blockIdx.x * rpc + (int)(threadIdx.x / (MC / 16));
+        const bool own = q < rows;
+        const float2* row = in + (int64_t)q * ld_in;
+        float2 x[16];
+        half_fwd<MC>(x, [&](int n) { return __ldcg(row + n); }, own ? n_in : 0,
+                     sm + kHalfTables + (threadIdx.x >> 4) * kHalfArea, sm, l, h);
+        if (own)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) X[(int64_t)q * MC + half_freq<MC>(l, h, k)] = x[k];
+        return;
+    }
     chain_enter();
     chain_next();
-    extern __shared__ float2 sm[];
     float2* a = sm;
     float2* b = sm + rpc * seq_len<MC>(fp.M);
     const int r0 = blockIdx.x * rpc;
@@ -103,32 +130,103 @@ __device__ __forceinline__ void finish_q2(float acc, const CgPass& c)
 
 // Row IFFTs of X, first n_out columns to out; CG: also Re<dotx, out> and finish_q2.
 template <int MC, bool CG>
-__global__ void __launch_bounds__(1024) k_rows_inv(const float2* X, int rows, float2* out, int n_out, FftPlan fp,
+__global__ void __launch_bounds__(t_threads<MC>()) k_rows_inv(const float2* X, int rows, float2* out, int n_out, FftPlan fp,
                            const float2* __restrict__ tw, int rpc, const float2* dotx, CgPass c)
 {
-    chain_enter();
-    chain_next();
     extern __shared__ float2 sm[];
-    float2* a = sm;
-    float2* b = sm + rpc * seq_len<MC>(fp.M);
-    const int r0 = blockIdx.x * rpc;
-    const int nr = min(rpc, rows - r0);
     float acc = 0.f;
-    rows_inv_group<MC>(X, r0, nr, rpc, out, n_out, fp, tw, dotx, a, b, acc);
+    if constexpr (half_warp_size<MC>()) {
+        half_tables<MC>(sm, tw);
+        chain_enter();
+        chain_next();
+        __syncthreads();
+        const int l = threadIdx.x & 15, h = (threadIdx.x >> 4) & 1;
+        const int q = blockIdx.x * rpc + (int)(threadIdx.x / (MC / 16));
+        const bool own = q < rows;
+        const float2* row = X + (int64_t)q * MC;
+        float2 x[16], y[8];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = own ? __ldcg(row + half_freq<MC>(l, h, k)) : make_float2(0.f, 0.f);
+        half_inv<MC>(x, y, sm + kHalfTables + (threadIdx.x >> 4) * kHalfArea, sm, l, h);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int m = half_elem<MC>(l, h, i);
+            if (own && m < n_out) {
+                const int64_t o = (int64_t)q * n_out + m;
+                out[o] = y[i];
+                if (dotx) acc += redot(__ldcg(dotx + o), y[i]);
+            }
+        }
+    } else {
+        chain_enter();
+        chain_next();
+        float2* a = sm;
+        float2* b = sm + rpc * seq_len<MC>(fp.M);
+        const int r0 = blockIdx.x * rpc;
+        const int nr = min(rpc, rows - r0);
+        rows_inv_group<MC>(X, r0, nr, rpc, out, n_out, fp, tw, dotx, a, b, acc);
+    }
     if (CG) finish_q2(acc, c);
 }
 
 // ------------------------------------------------------------- column pass
 
+// M = 256, 512: kHalfCols columns a block, staged as row pieces of 32 bytes at
+// half_col_ld (4 mod 16: the stores of 16 lanes, four rows of four columns, meet
+// distinct banks).  Chat is older than the predecessor, so it is read before the wait.
+constexpr int kHalfCols = 4;
+
 template <int MC>
-__global__ void __launch_bounds__(1024) k_cols_filter(float2* X, int n_in, int n_out, FftPlan fp, const float2* __restrict__ tw,
+__host__ __device__ constexpr int half_col_ld() { return MC / 2 + 4; }
+
+template <int MC>
+__global__ void __launch_bounds__(t_threads<MC>()) k_cols_filter(float2* X, int n_in, int n_out, FftPlan fp, const float2* __restrict__ tw,
                               const float* __restrict__ Chat, int cpc)
 {
+    extern __shared__ float2 sm[];
+    const int x0 = blockIdx.x * cpc;
+    if constexpr (half_warp_size<MC>()) {
+        constexpr int LD = half_col_ld<MC>(), THREADS = kHalfCols * MC / 16, E = kHalfCols * (MC / 2) / THREADS;
+        float2* cols = sm + kHalfTables;
+        half_tables<MC>(sm, tw);
+        const int tid = threadIdx.x, l = tid & 15, h = (tid >> 4) & 1, c = tid / (MC / 16);
+        float hs[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) hs[k] = __ldg(Chat + (int64_t)(x0 + c) * MC + half_freq<MC>(l, h, k));
+        chain_enter();
+        chain_next();
+        float2 v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int e = tid + i * THREADS, y = e / kHalfCols;
+            v[i] = y < n_in ? __ldcg(X + (int64_t)y * MC + x0 + e % kHalfCols) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int e = tid + i * THREADS;
+            cols[(e % kHalfCols) * LD + e / kHalfCols] = v[i];
+        }
+        __syncthreads();
+        float2* area = cols + kHalfCols * LD + (tid >> 4) * kHalfArea;
+        float2* col = cols + c * LD;
+        float2 x[16], out[8];
+        half_fwd<MC>(x, [&](int n) { return col[n]; }, n_in, area, sm, l, h);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = make_float2(x[k].x * hs[k], x[k].y * hs[k]);
+        half_inv<MC>(x, out, area, sm, l, h);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) col[half_elem<MC>(l, h, i)] = out[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int e = tid + i * THREADS, y = e / kHalfCols;
+            if (y < n_out) X[(int64_t)y * MC + x0 + e % kHalfCols] = cols[(e % kHalfCols) * LD + y];
+        }
+        return;
+    }
     chain_enter();
     chain_next();
-    extern __shared__ float2 sm[];
     const int ld = seq_len<MC>(fp.M) + 4;
-    const int x0 = blockIdx.x * cpc;
     cols_group<MC>(X, n_in, n_out, x0, min(cpc, fp.M - x0), cpc, fp, tw, Chat, sm, sm + cpc * ld);
 }
 
@@ -600,7 +698,7 @@ struct Shape {
 // and columns a block as keep two warps busy and 32-byte pieces whole, so that
 // small grids spread over the SMs and their stages' barriers span few warps
 // (T at N = 64 with 8 rows and 32 columns a block and plain launches 18.5 us, now
-// 7.7; at N = 256 21.8 and 15.9).
+// 7.7).  The T passes at M = 256, 512 have shapes of their own (t_row_shape).
 // Runtime path: 256 threads, ping-pong buffers.
 Shape row_shape(int M, bool pow2)
 {
@@ -689,6 +787,27 @@ int split_grid(int items, int per, int* grid)
     return SPIREC_OK;
 }
 
+// The shapes of the T passes: at M = 256, 512 two warps a block of rows (one row a
+// warp or two) and kHalfCols columns a block, M / 16 threads a sequence.
+template <int MC>
+Shape t_row_shape(int M)
+{
+    if constexpr (half_warp_size<MC>())
+        return Shape{1024 / MC, 64, (kHalfTables + 4 * kHalfArea) * sizeof(float2)};
+    else
+        return row_shape(M, MC > 0);
+}
+
+template <int MC>
+Shape t_col_shape(int M)
+{
+    if constexpr (half_warp_size<MC>())
+        return Shape{kHalfCols, kHalfCols * MC / 16,
+                     (kHalfTables + kHalfCols * (half_col_ld<MC>() + MC / 256 * kHalfArea)) * sizeof(float2)};
+    else
+        return col_shape(M, MC > 0);
+}
+
 struct LaunchRowsFwd {
     spirec_plan p;
     const float2* in;
@@ -702,7 +821,7 @@ struct LaunchRowsFwd {
             if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
             chain(k_rows_fwd_split<S>, grid, kSplitThreads, sizeof(StagedSmem), p->stream, in, N, p->X, split_ld(N), p->twiddle);
         } else {
-            const Shape s = row_shape(p->MF, MC > 0);
+            const Shape s = t_row_shape<MC>(p->MF);
             chain(k_rows_fwd<MC>, (N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 in, N, N, N, p->X, p->fft, p->twiddle, s.per_cta);
         }
@@ -727,7 +846,7 @@ struct LaunchCols {
             chain(kern, grid, kSplitThreads, sizeof(StagedSmem), p->stream, p->X, N, split_ld(N), p->twiddle, p->Chat,
                                                                         cg ? *cg : CgPass{});
         } else {
-            const Shape s = col_shape(p->MF, MC > 0);
+            const Shape s = t_col_shape<MC>(p->MF);
             chain(k_cols_filter<MC>, (p->MF + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 p->X, N, N, p->fft, p->twiddle, p->Chat, s.per_cta);
         }
@@ -752,7 +871,7 @@ struct LaunchRowsInv {
             if ((rc = split_grid(N, kSplitWarps / S, &grid)) != SPIREC_OK) return rc;
             chain(k_rows_inv_split<S>, grid, kSplitThreads, sizeof(SplitSmem), p->stream, p->X, N, split_ld(N), out, p->twiddle);
         } else {
-            const Shape s = row_shape(p->MF, MC > 0);
+            const Shape s = t_row_shape<MC>(p->MF);
             auto kern = cg ? k_rows_inv<MC, true> : k_rows_inv<MC, false>;
             chain(kern, (N + s.per_cta - 1) / s.per_cta, s.threads, s.smem, p->stream, 
                 p->X, N, out, N, p->fft, p->twiddle, s.per_cta, cg ? x : nullptr, cg ? *cg : CgPass{});
@@ -962,8 +1081,7 @@ struct LaunchNoAlloc {
     int operator()()
     {
         const int M = fp.M;
-        const bool pow2 = MC > 0;
-        const Shape rs = row_shape(M, pow2), cs = col_shape(M, pow2);
+        const Shape rs = t_row_shape<MC>(M), cs = t_col_shape<MC>(M);
         const int rblocks = (N + rs.per_cta - 1) / rs.per_cta;
         k_rows_fwd<MC><<<rblocks, rs.threads, rs.smem, st>>>(x, N, N, N, rows, fp, tw, rs.per_cta);
         SPIREC_CK(cudaGetLastError());

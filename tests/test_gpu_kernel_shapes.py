@@ -190,3 +190,27 @@ def test_loop_half_warp_ffts(sp, monkeypatch, N, M):
         monkeypatch.setenv("SPIREC_NO_LOOP", "1")
         y, Jy = sp.spirec_solve(p.h, None, 3, N)
     assert rel(x, y) < 1e-5 and rel(J, Jy) < 1e-5
+
+
+# T on grids of 256 and 512 points (256-point transforms of half a warp each): the
+# smallest and largest sides, odd ones (the last block with fewer rows), sides
+# far below the grid's, through a plan and without one.
+@pytest.mark.parametrize("N,M", [(2, 256), (9, 512), (65, 0), (127, 0), (128, 0), (129, 0), (255, 0), (256, 0)])
+def test_toeplitz_half_warp_grids(sp, N, M):
+    import torch
+    from oracle import factored as F
+    from oracle import toeplitz_cpu as TC
+    g = synth.rng(N)
+    kx, ky = synth.uniform_k(40, g)
+    x = c64(synth.complex_normal((N, N), g))
+    with sp.Plan(N, 40, M, 0, _stream(), kx, ky) as p:
+        Mp = max(1 << (2 * N - 2).bit_length(), M)
+        spec = TC.kernel_spectrum(F.gram(kx, ky, N), N, Mp)
+        want = TC.toeplitz_apply(spec, x)
+        Tx = empty_c64((N, N))
+        sp.spirec_toeplitz_dev(p.h, to_dev(x), Tx)
+        sp.spirec_sync(p.h)
+        assert rel(from_dev(Tx), want) < 1e-5
+        C = torch.from_numpy((spec.real / Mp**2).astype(np.float32)).cuda()  # the library scales its spectrum by 1 / M^2
+        sp.spirec_toeplitz_noalloc(to_dev(x), C, Tx, N, Mp, _stream())
+        assert rel(from_dev(Tx), want) < 1e-5
