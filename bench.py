@@ -48,10 +48,10 @@ ITERS = 50
 NCU_TRAFFIC = {"k_cg_loop": (10_712_832, "9a5d48a08d744779"), "k_tc_pair_gemm_G": (2_171_904, "09eacbd42c77e41e"),
                "k_tc_pair_gemm_D": (3_207_936, "09eacbd42c77e41e")}
 KERNEL_SOURCES = {
-    "k_cg_loop": ["cg_loop.cu", "cg_device.cuh", "fft_device.cuh", "fft_reg.cuh", "reduce.cuh", "penalty.cuh",
-                  "internal.cuh"],
-    "k_tc_pair_gemm_G": ["nudft_tc.cu", "phase.cuh", "internal.cuh"],
-    "k_tc_pair_gemm_D": ["nudft_tc.cu", "phase.cuh", "internal.cuh"],
+    "k_cg_loop": ["cg_loop.cu", "cg_device.cuh", "fft_device.cuh", "fft_half.cuh", "fft_reg.cuh", "reduce.cuh",
+                  "penalty.cuh", "internal.cuh"],
+    "k_tc_pair_gemm_G": ["nudft_tc.cu", "chain.cuh", "phase.cuh", "internal.cuh"],
+    "k_tc_pair_gemm_D": ["nudft_tc.cu", "chain.cuh", "phase.cuh", "internal.cuh"],
 }
 
 

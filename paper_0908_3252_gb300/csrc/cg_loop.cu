@@ -1357,9 +1357,9 @@ int loop_rb(int i)
 // of the grid co-resident (the grid synchronisations need that).  With `wide`
 // the grid has a block for every column group too, as far as they fit: blocks
 // beyond the rows only work in the column pass, which otherwise takes two
-// rounds where there are fewer row blocks than column groups (N = 192, M =
-// 512, 48 row blocks for 64 groups: column pass 12.1 -> 6.2 us, an iteration 30.0 ->
-// 24.3; N = 384, M = 1024, 96 of 128 and rows of 4 or 3 a block: 30.0 -> 23.8).
+// rounds where there are fewer row blocks than column groups (with radix-4
+// transforms, N = 192, M = 512, 48 row blocks for 64 groups: column pass 12.1 -> 6.2
+// us, an iteration 30.0 -> 24.3; with the register ones 3.1 and 19.7; N = 384, M = 1024, 96 of 128 and rows of 4 or 3 a block: 30.0 -> 23.8).
 template <int MC>
 bool loop_fits(int N, int RB, size_t cap, int sms, bool wide, int* grid_out, size_t* smem_out)
 {
@@ -1435,7 +1435,8 @@ cudaLaunchConfig_t cluster_config(int grid, size_t smem, cudaLaunchAttribute* at
 // Whether a loop of `grid` blocks runs as one cluster: up to 16 blocks, where the
 // device places such a cluster.  An iteration (us) with the grid barrier and as a
 // cluster: N = 64, M = 128 (8 blocks) 20.9 and 17.6; N = 128, M = 256 (16 blocks)
-// 24.4 and 20.6: the five synchronisations 9.9 -> 5.1.
+// 24.4 and 20.6 (15.7 with the register transforms): the five synchronisations
+// 9.9 -> 5.1.
 template <int MC>
 bool cluster_fits(int grid, size_t smem)
 {

@@ -11,7 +11,8 @@
 //   columns: per column FFT (N nonzero inputs) -> * Chat -> IFFT, rows < N,
 //   rows:    N row IFFTs, columns < N kept.
 // Inside the CG iteration the last row pass (the column pass at M >= 2048) also
-// forms q2 = Re<d, T d> and the first line-search step.  The bodies of the passes live in fft_device.cuh (shared with the persistent loop of
+// forms q2 = Re<d, T d> and the first line-search step.  The bodies of the passes
+// live in fft_device.cuh and fft_half.cuh (shared with the persistent loop of
 // cg_loop.cu); this file holds the stand-alone kernels and their launchers.
 //
 // FFTs are self-sorting Stockham transforms in shared memory.  For
@@ -21,8 +22,9 @@
 // log2 M), values in registers between a read and a write phase.  Any other
 // M = 2^a 3^b 5^c (a caller's spectrum on such a grid, spirec_toeplitz_noalloc)
 // runs the runtime mixed-radix path with a ping-pong buffer.
-// At M = 2048 and 4096 the three passes split every transform into warp-sized
-// 1024-point DFTs (k_rows_fwd_split, k_cols_split, k_rows_inv_split).
+// At M = 256 and 512 the three passes are 256-point register transforms of half a
+// warp each (fft_half.cuh); at M = 2048 and 4096 they split every transform
+// into warp-sized 1024-point DFTs (k_rows_fwd_split, k_cols_split, k_rows_inv_split).
 #include <stdint.h>
 
 #include <atomic>
