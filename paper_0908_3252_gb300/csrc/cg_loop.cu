@@ -132,18 +132,19 @@ struct Geo {
     static constexpr int WA = 544;  // 16 x 33 (forward), 32 x 17 (inverse)
     static constexpr int LDF = 1090;
     // M = 256, 512: 256-point FFTs of half a warp each (fft_half.cuh), a half-warp
-    // (M = 256) or a warp, split by output parity (M = 512), a sequence.  The
-    // column pass stages H_COLS columns of at most M / 2 rows at H_LD (odd
-    // multiples of the pieces that neighbouring lanes store, for the banks) and
-    // eight warps transform; each half-warp has an exchange area of 16 x 17.
+    // (M = 256) or a warp, split by output parity (M = 512), a sequence; eight
+    // warps transform.  The column pass stages H_COLS columns of at most M / 2
+    // rows in slots of H_LD (1 or 2 mod 16, for the banks of the staging stores),
+    // which then are the exchange areas (16 x 17 a half-warp) of their column's
+    // warp; so no shape needs more shared memory than with radix-4 stages.
     static constexpr bool HALFWARP = fftd::half_warp_size<MC>();
     static constexpr int H_COLS = MC == 512 ? 8 : 16;
-    static constexpr int H_LD = MC == 512 ? 258 : 129;
+    static constexpr int H_LD = MC == 512 ? 546 : 273;
     static constexpr int H_AREA = fftd::kHalfArea;
     static constexpr int H_ROWS = MC == 512 ? 8 : 16;  // rows a round of the eight warps
     static constexpr int FB_ROWS = FOURSTEP ? 16 * WA : 2 * RPC * LDR;
     static constexpr int FB_COLS = FOURSTEP ? FS_COLS * LDF : RPC * LDC;
-    static constexpr int FBUF = HALFWARP ? H_COLS * H_LD + 16 * H_AREA : FB_ROWS > FB_COLS ? FB_ROWS : FB_COLS;
+    static constexpr int FBUF = HALFWARP ? H_COLS * H_LD : FB_ROWS > FB_COLS ? FB_ROWS : FB_COLS;
     // columns of a group of the column pass
     static constexpr int COLS = FOURSTEP ? FS_COLS : HALFWARP ? H_COLS : RPC;
     // staged radix-4 twiddles (M <= 128); the tables T16[k2][l] = w512^(l k2) and
@@ -633,8 +634,8 @@ __device__ __forceinline__ void cols_half(float2* X, int N, int x0, const float*
     __syncthreads();
     after_staging();
     if (warp < 8) {
-        float2* area = fbuf + G::H_COLS * G::H_LD + (tid >> 4) * G::H_AREA;
         float2* col = fbuf + c * G::H_LD;
+        float2* area = col + (MC == 512 ? h * G::H_AREA : 0);
         float2 x[16], y[8];
         fftd::half_fwd<MC>(x, [&](int n) { return col[n]; }, N, area, t, l, h);
 #pragma unroll
@@ -854,7 +855,7 @@ __device__ __forceinline__ void phase_update(const LoopArgs& A, const Rows& R, f
                     float2 x[16];
                     const float2* row = cg + q * N;
                     fftd::half_fwd<MC>(x, [&](int n) { return row[n]; }, own ? N : 0,
-                                       fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
+                                       fbuf + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
                     float2* out = A.X + (int64_t)(R.R0 + q) * MC;
                     if (own)
 #pragma unroll
@@ -952,7 +953,7 @@ __device__ __forceinline__ void phase_rows(const LoopArgs& A, const Rows& R, flo
                 float2 x[16], tg[8];
 #pragma unroll
                 for (int k = 0; k < 16; ++k) x[k] = own ? __ldcg(yr + fftd::half_freq<MC>(l, h, k)) : make_float2(0.f, 0.f);
-                fftd::half_inv<MC>(x, tg, fbuf + G::H_COLS * G::H_LD + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
+                fftd::half_inv<MC>(x, tg, fbuf + (threadIdx.x >> 4) * G::H_AREA, stw, l, h);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int m = fftd::half_elem<MC>(l, h, i);

@@ -68,6 +68,7 @@ __device__ __forceinline__ void half_fwd(float2 (&x)[16], F&& load, int N, float
         const int n = l + 16 * j;
         x[j] = n < N ? load(n) : make_float2(0.f, 0.f);
     }
+    __syncwarp();  // the exchange areas may lie where the inputs do
     if (MC == 512 && h)
 #pragma unroll
         for (int j = 0; j < 16; ++j) x[j] = cmul(x[j], t[256 + l + 16 * j]);
